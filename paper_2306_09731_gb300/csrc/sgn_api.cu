@@ -262,6 +262,17 @@ std::vector<C64> staged_twiddles(int N, int lN) {
   return t;
 }
 
+// the same table in fixed point, for the FP64 passes
+std::vector<cpx<fx>> staged_twiddles_fx(int N, int lN) {
+  std::vector<cpx<fx>> t(2 * (size_t)N);
+  for (int plan = 0; plan < 2; ++plan)
+    for (int i = 0; i < N; ++i) {
+      const int k = staged_exponent(i, lN, plan);
+      if (k >= 0) t[(size_t)plan * N + i] = fx_twiddle(k, lN);
+    }
+  return t;
+}
+
 void build_tables(sgn_ctx* ctx) {
   const Geom& G = ctx->G;
   const std::vector<C64> tx = staged_twiddles(G.Nx, G.lNx), ty = staged_twiddles(G.Ny, G.lNy);
@@ -278,12 +289,20 @@ void build_tables(sgn_ctx* ctx) {
     for (int c = 0; c < G.Nxh; ++c) minv[(size_t)r * G.ldS + c] = 1.0 / (3.0 + kx[c] * kx[c] + ky[r] * ky[r]);
   ctx->tb.minv = dalloc<double>(ctx, minv.size());
   CK(cudaMemcpy(ctx->tb.minv, minv.data(), minv.size() * sizeof(double), cudaMemcpyHostToDevice));
-  ctx->tb.twx = dalloc<C64>(ctx, 2 * (size_t)G.Nx);
-  ctx->tb.twy = dalloc<C64>(ctx, 2 * (size_t)G.Ny);
+  const std::vector<cpx<fx>> qx = staged_twiddles_fx(G.Nx, G.lNx), qy = staged_twiddles_fx(G.Ny, G.lNy);
+  std::vector<double> k2x(kx), k2y(ky);
+  for (double& k : k2x) k *= two_pi / G.Lx;
+  for (double& k : k2y) k *= two_pi / G.Ly;
+  ctx->tb.twx = dalloc<cpx<fx>>(ctx, qx.size());
+  ctx->tb.twy = dalloc<cpx<fx>>(ctx, qy.size());
+  ctx->tb.k2x = dalloc<double>(ctx, G.Nxh);
+  ctx->tb.k2y = dalloc<double>(ctx, G.Ny);
+  CK(cudaMemcpy(ctx->tb.k2x, k2x.data(), G.Nxh * sizeof(double), cudaMemcpyHostToDevice));
+  CK(cudaMemcpy(ctx->tb.k2y, k2y.data(), G.Ny * sizeof(double), cudaMemcpyHostToDevice));
   ctx->tb.kx = dalloc<double>(ctx, G.Nxh);
   ctx->tb.ky = dalloc<double>(ctx, G.Ny);
-  CK(cudaMemcpy(ctx->tb.twx, tx.data(), tx.size() * sizeof(C64), cudaMemcpyHostToDevice));
-  CK(cudaMemcpy(ctx->tb.twy, ty.data(), ty.size() * sizeof(C64), cudaMemcpyHostToDevice));
+  CK(cudaMemcpy(ctx->tb.twx, qx.data(), qx.size() * sizeof(qx[0]), cudaMemcpyHostToDevice));
+  CK(cudaMemcpy(ctx->tb.twy, qy.data(), qy.size() * sizeof(qy[0]), cudaMemcpyHostToDevice));
   CK(cudaMemcpy(ctx->tb.kx, kx.data(), G.Nxh * sizeof(double), cudaMemcpyHostToDevice));
   CK(cudaMemcpy(ctx->tb.ky, ky.data(), G.Ny * sizeof(double), cudaMemcpyHostToDevice));
   if (ctx->opt.precision >= 2) {

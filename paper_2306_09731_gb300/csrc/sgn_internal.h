@@ -9,6 +9,7 @@
 
 #include "dfloat.cuh"
 #include "fft_core.cuh"
+#include "fixed.cuh"
 
 namespace sgn {
 
@@ -83,10 +84,21 @@ enum RkMode : int {
 };
 
 // Per-precision device tables.
+// Twiddles are of the transforms' type: fixed point for the FP64 passes.
+template <typename T>
+struct tw_type {
+  typedef T type;
+};
+template <>
+struct tw_type<double> {
+  typedef fx type;
+};
 template <typename T>
 struct Tables {
-  cpx<T>* twx = nullptr;  // W_Nx^k, k < Nx
-  cpx<T>* twy = nullptr;  // W_Ny^k, k < Ny
+  cpx<typename tw_type<T>::type>* twx = nullptr;  // W_Nx^k, staged layout of both radix plans
+  cpx<typename tw_type<T>::type>* twy = nullptr;  // W_Ny^k
+  T* k2x = nullptr;       // FP64: (2 pi / Lx) kx [Nxh] and (2 pi / Ly) ky [Ny] (see k_fx_mv_x)
+  T* k2y = nullptr;
   T* kx = nullptr;        // 2 pi m / Lx, m = 0..Nx/2, Nyquist 0   [Nxh]
   T* ky = nullptr;        // 2 pi m / Ly, m = 0..Ny/2-1, -Ny/2..-1, Nyquist 0 [Ny]
   T* minv = nullptr;      // 1 / (3 + kx^2 + ky^2) per half-spectrum entry [Ny][ldS] (FP64, double-float)

@@ -54,26 +54,22 @@ sgn_status noalloc_fail(sgn_status st, const std::string& msg) {
 static __device__ __align__(256) unsigned char g_noalloc_scratch[kScratchBytes];
 
 // Twiddles W_N^k = exp(-2 pi i k/N) in the staged layout of the transforms
-// (entry i is W_N^staged_exponent(i)) and the wavenumbers (Nyquist set to 0).
-__global__ void k_noalloc_tables(int Nx, int Ny, int lNx, int lNy, double Lx, double Ly, cpx<double>* twx,
-                                 cpx<double>* twy, double* kx, double* ky) {
+// (entry i is W_N^staged_exponent(i)) and the wavenumbers times ax = 2 pi/Lx,
+// ay = 2 pi/Ly (Nyquist set to 0).
+__global__ void k_noalloc_tables(int Nx, int Ny, int lNx, int lNy, double ax, double ay, cpx<fx>* twx,
+                                 cpx<fx>* twy, double* k2x, double* k2y) {
   const int i = blockIdx.x * blockDim.x + threadIdx.x;
-  const double two_pi = 6.283185307179586476925286766559;
-  double s = 0.0, c = 0.0;
   if (i < Nx) {
     const int k = staged_exponent(i, lNx);
-    if (k >= 0) sincospi(2.0 * (double)k / (double)Nx, &s, &c);
-    twx[i] = mk(c, -s);
+    twx[i] = k >= 0 ? fx_twiddle(k, lNx) : mk(fx{0}, fx{0});
   }
   if (i < Ny) {
     const int k = staged_exponent(i, lNy);
-    s = c = 0.0;
-    if (k >= 0) sincospi(2.0 * (double)k / (double)Ny, &s, &c);
-    twy[i] = mk(c, -s);
+    twy[i] = k >= 0 ? fx_twiddle(k, lNy) : mk(fx{0}, fx{0});
     const int m = i < Ny / 2 ? i : i - Ny;
-    ky[i] = (i == Ny / 2) ? 0.0 : two_pi * (double)m / Ly;
+    k2y[i] = (i == Ny / 2) ? 0.0 : (double)m * ay * ay;
   }
-  if (i <= Nx / 2) kx[i] = (i == Nx / 2) ? 0.0 : two_pi * (double)i / Lx;
+  if (i <= Nx / 2) k2x[i] = (i == Nx / 2) ? 0.0 : (double)i * ax * ax;
 }
 
 extern "C" sgn_status sgn_elliptic_apply_noalloc(int Nx, int Ny, double Lx, double Ly, const double* h,
@@ -117,10 +113,10 @@ extern "C" sgn_status sgn_elliptic_apply_noalloc(int Nx, int Ny, double Lx, doub
     return p;
   };
   Tables<double> tb{};
-  tb.twx = reinterpret_cast<cpx<double>*>(take(sizeof(cpx<double>) * Nx));
-  tb.twy = reinterpret_cast<cpx<double>*>(take(sizeof(cpx<double>) * Ny));
-  tb.kx = reinterpret_cast<double*>(take(sizeof(double) * G.Nxh));
-  tb.ky = reinterpret_cast<double*>(take(sizeof(double) * Ny));
+  tb.twx = reinterpret_cast<cpx<fx>*>(take(sizeof(cpx<fx>) * Nx));
+  tb.twy = reinterpret_cast<cpx<fx>*>(take(sizeof(cpx<fx>) * Ny));
+  tb.k2x = reinterpret_cast<double*>(take(sizeof(double) * G.Nxh));
+  tb.k2y = reinterpret_cast<double*>(take(sizeof(double) * Ny));
   double* hh = reinterpret_cast<double*>(take(sizeof(double) * G.nphys()));
   double* cr = reinterpret_cast<double*>(take(sizeof(double) * G.nphys()));
   double* cc = reinterpret_cast<double*>(take(sizeof(double) * G.nphys()));
@@ -134,8 +130,9 @@ extern "C" sgn_status sgn_elliptic_apply_noalloc(int Nx, int Ny, double Lx, doub
 
   const Exec ex{stream, nullptr};
   const int tn = (Nx > Ny ? Nx : Ny);
-  k_noalloc_tables<<<(tn + 255) / 256, 256, 0, stream>>>(Nx, Ny, G.lNx, G.lNy, Lx, Ly, tb.twx, tb.twy, tb.kx,
-                                                          tb.ky);
+  const double two_pi = 6.283185307179586476925286766559;
+  k_noalloc_tables<<<(tn + 63) / 64, 64, 0, stream>>>(Nx, Ny, G.lNx, G.lNy, two_pi / Lx, two_pi / Ly, tb.twx, tb.twy,
+                                                      tb.k2x, tb.k2y);
   e = cudaGetLastError();
   // the flags keep the previous call's value: clear them first
   if (e == cudaSuccess) e = cudaMemsetAsync(flags, 0, sizeof(int), stream);

@@ -282,27 +282,18 @@ __global__ void k_coef_x(Geom G, const cpx<T>* __restrict__ tw, const T* __restr
   fft_regs<true>(v, sm, tw, L.t, G.lNx);
   if (!L.valid) return;
   const double invN = 1.0 / (double)G.nphys();
-  if constexpr (std::is_same<T, dfl>::value) {
-    // one slot at a time from the thread's own slots of the transform buffer
-    // (free again after the transform; no other thread touches them): one
-    // copy of the double-float reciprocal code instead of sixteen.
-    // N = Nx Ny is a power of two: the scaling by 1/N is exact.
-    store_slots(v, sm, L.t, T_, 0);
-    const float fN = (float)invN;
+  // one slot at a time from the thread's own slots of the transform buffer
+  // (free again after the transform; no other thread touches them): one
+  // copy of the double-float reciprocal code instead of sixteen.
+  // N = Nx Ny is a power of two: the scaling by 1/N is exact.
+  store_slots(v, sm, L.t, T_, 0);
+  const float fN = (float)invN;
 #pragma unroll 1
-    for (int s = 0; s < 8; ++s) {
-      const int x = L.t + s * T_;
-      const cpx<T> z = sm[sidx<T>(x, 0)];
-      coef_point_df(scale_pow2(z.x, fN), fN, h, cr, cc, (size_t)L.y0 * N + x, flags, cp);
-      coef_point_df(scale_pow2(z.y, fN), fN, h, cr, cc, (size_t)L.y1 * N + x, flags, cp);
-    }
-  } else {
-#pragma unroll
-    for (int s = 0; s < 8; ++s) {
-      const int x = L.t + s * T_;
-      coef_point<T>((double)v[s].x * invN, invN, h, cr, cc, (size_t)L.y0 * N + x, flags, cp);
-      coef_point<T>((double)v[s].y * invN, invN, h, cr, cc, (size_t)L.y1 * N + x, flags, cp);
-    }
+  for (int s = 0; s < 8; ++s) {
+    const int x = L.t + s * T_;
+    const cpx<T> z = sm[sidx<T>(x, 0)];
+    coef_point_df(scale_pow2(z.x, fN), fN, h, cr, cc, (size_t)L.y0 * N + x, flags, cp);
+    coef_point_df(scale_pow2(z.y, fN), fN, h, cr, cc, (size_t)L.y1 * N + x, flags, cp);
   }
 }
 
@@ -1465,11 +1456,6 @@ template <typename T, int L>
 static void set_attrs_ln() {
   set_attrs_ln_plan<T, L, 0>();
   if constexpr (L % 3 != 0) set_attrs_ln_plan<T, L, 1>();
-  if constexpr (L == 12) {
-    set_smem<T>((const void*)ypass_fn<T, true, 1, EpiStore<T, 1>, T, L>());
-    set_smem<T>((const void*)ypass_fn<T, false, 1, EpiStore<T, 1>, T, L>());
-    set_smem<T>((const void*)ypass_fn<T, true, 1, EpiStore<T, 1>, double, L>());
-  }
 }
 
 // the same at runtime length (LN = 0)
@@ -1499,12 +1485,6 @@ void init_kernel_attributes() {
   set_attrs_ln<T, 12>();
   set_attrs_plan<T, 0>();
   set_attrs_plan<T, 1>();
-  set_smem<T>((const void*)k_x_r2c<T>);
-  set_smem<T>((const void*)k_x_c2r<T>);
-  set_smem<T>((const void*)k_coef_x<T>);
-  set_smem<T>((const void*)ypass_fn<T, false, 1, EpiStore<T, 1>>());
-  set_smem<T>((const void*)ypass_fn<T, true, 1, EpiStore<T, 1>>());
-  set_smem<T>((const void*)ypass_fn<T, true, 1, EpiStore<T, 1>, double>());
   cudaGetLastError();
 }
 
@@ -1540,34 +1520,6 @@ cudaError_t launch_x_c2r(const Geom& G, const Tables<T>& tb, const cpx<T>* const
   ex.begin(PK_IO);
   k_x_c2r<T><<<grid, block, smem, ex.s>>>(G, tb.twx, tb.kx, a, scale);
   ex.end();
-  return cudaGetLastError();
-}
-
-template <typename T>
-cudaError_t launch_y_fft(const Geom& G, const Tables<T>& tb, bool inverse, const cpx<T>* const* in,
-                         const int* deriv, int nf, cpx<T>* const* out, const Exec& ex) {
-  dim3 grid, block;
-  size_t smem;
-  if (inverse)
-    y_config<T, true, 1>(G, grid, block, smem);
-  else
-    y_config<T, false, 1>(G, grid, block, smem);
-  for (int i = 0; i < nf; ++i) {
-    YIn<T, 1> yi{};
-    yi.src[0] = in[i];
-    yi.deriv[0] = deriv ? deriv[i] : 0;
-    EpiStore<T, 1> ep{};
-    ep.dst[0] = out[i];
-    dispatch_l12(G.lNy, [&](auto ln) {
-      constexpr int L = decltype(ln)::value;
-      ex.begin(PK_IO);
-      if (inverse)
-        ypass_fn<T, true, 1, EpiStore<T, 1>, T, L>()<<<grid, block, smem, ex.s>>>(G, tb.twy, tb.ky, yi, ep);
-      else
-        ypass_fn<T, false, 1, EpiStore<T, 1>, T, L>()<<<grid, block, smem, ex.s>>>(G, tb.twy, tb.ky, yi, ep);
-      ex.end();
-    });
-  }
   return cudaGetLastError();
 }
 
@@ -1615,7 +1567,26 @@ static int y_bound(const Geom& G, int type, int pass) {
 static bool is_y_pass(int pass) { return pass <= TP_RHS_YFWD; }
 
 #ifdef SGN_SPECTRAL_COMMON
+// Columns (row pairs) per block of the FP64 passes: 256 threads, fewer where
+// the grid would leave SMs idle (fewer than two blocks each), but at least a
+// warp a block and, for columns, two neighbours (32-byte segments).
+static int fx_default_cols(const Geom& G) {
+  const int Tn = G.Ny >> 3;
+  int C = 256 / Tn;
+  C = C < 1 ? 1 : (C > 64 ? 64 : C);
+  while (C > 2 && (G.Nxh + C - 1) / C < 304 && Tn * C >= 64) C >>= 1;
+  return C;
+}
+static int fx_default_pairs(const Geom& G) {
+  const int Tn = G.Nx >> 3, half = G.Ny >> 1;
+  int P = Tn >= 256 ? 1 : 256 / Tn;
+  if (P > half) P = half;
+  while (P > 1 && (half + P - 1) / P < 304 && Tn * P >= 64) P >>= 1;
+  return P;
+}
+
 int pass_default_threads(const Geom& G, int type, int pass) {
+  if (type == TT_F64) return is_y_pass(pass) ? (G.Ny >> 3) * fx_default_cols(G) : (G.Nx >> 3) * fx_default_pairs(G);
   if (is_y_pass(pass)) {
     const int Tn = G.Ny >> 3;
     int C = y_bound(G, type, pass) / Tn;
@@ -1950,6 +1921,31 @@ void init_kernel_attributes_df() {
 }
 #endif  // SGN_SPECTRAL_DF
 
+// the RK4 stage update from K in tmp (k_rk_update)
+template <typename T, typename S>
+static cudaError_t launch_rk_update(const Geom& G, const Tables<S>& tbs, cpx<S>* const* U, const cpx<S>* sig,
+                                    cpx<T>* const* tmp, cpx<S>* const* Un, cpx<S>* const* Unext, cpx<S>* const* acc,
+                                    cpx<S>* bhat, const RkArgs& rk, const Exec& ex) {
+  RkK<T, S> a{};
+  for (int f = 0; f < 3; ++f) {
+    a.K[f] = tmp[f];
+    a.Un[f] = Un[f];
+    a.Unext[f] = Unext ? Unext[f] : nullptr;
+    a.acc[f] = acc[f];
+  }
+  a.b = bhat;
+  a.kxs = tbs.kx;
+  a.kys = tbs.ky;
+  for (int f = 0; f < 3; ++f) a.Y[f] = U[f];
+  a.sig = sig;
+  a.rk = rk;
+  ex.begin(PK_RK);
+  k_rk_update<T, S><<<NBLK, 256, 0, ex.s>>>(G, a, rk.dt / 6.0, rk.mode == RK_STAGE3 ? rk.dt : 0.5 * rk.dt,
+                                             rk.krasny_thr * rk.krasny_thr * (double)G.nphys() * (double)G.nphys());
+  ex.end();
+  return cudaGetLastError();
+}
+
 template <typename T, typename S>
 cudaError_t launch_rhs(const Geom& G, const Tables<T>& tb, const Tables<S>& tbs, cpx<S>* const* U,
                        const cpx<S>* sig, const T* h, const T* cr, cpx<T>* const* tmp, cpx<S>* const* Un,
@@ -2013,27 +2009,7 @@ cudaError_t launch_rhs(const Geom& G, const Tables<T>& tb, const Tables<S>& tbs,
     });
     ex.end();
   });
-  {
-    RkK<T, S> a{};
-    for (int f = 0; f < 3; ++f) {
-      a.K[f] = tmp[f];
-      a.Un[f] = Un[f];
-      a.Unext[f] = Unext ? Unext[f] : nullptr;
-      a.acc[f] = acc[f];
-    }
-    a.b = bhat;
-    a.kxs = tbs.kx;
-    a.kys = tbs.ky;
-    for (int f = 0; f < 3; ++f) a.Y[f] = U[f];
-    a.sig = sig;
-    a.rk = rk;
-    ex.begin(PK_RK);
-    k_rk_update<T, S><<<NBLK, 256, 0, ex.s>>>(G, a, rk.dt / 6.0, rk.mode == RK_STAGE3 ? rk.dt : 0.5 * rk.dt,
-                                               rk.krasny_thr * rk.krasny_thr * (double)G.nphys() *
-                                                   (double)G.nphys());
-    ex.end();
-  }
-  return cudaGetLastError();
+  return launch_rk_update<T, S>(G, tbs, U, sig, tmp, Un, Unext, acc, bhat, rk, ex);
 }
 
 // ------------------------------------------------ spectral pointwise kernels
@@ -2082,28 +2058,5 @@ cudaError_t launch_precond(const Geom& G, const Tables<T>& tb, const cpx<T>* in,
   ex.end();
   return cudaGetLastError();
 }
-
-// ------------------------------------------------------- instantiations
-// the launchers of one arithmetic (used by the per-type units)
-#define SGN_INST(T)                                                                                          \
-  template void init_kernel_attributes<T>();                                                                 \
-  template cudaError_t launch_x_r2c<T>(const Geom&, const Tables<T>&, const double* const*, int,             \
-                                       cpx<T>* const*, const Exec&);                                        \
-  template cudaError_t launch_x_c2r<T>(const Geom&, const Tables<T>&, const cpx<T>* const*, const int*, int, \
-                                       double* const*, double, const Exec&);                                \
-  template cudaError_t launch_y_fft<T>(const Geom&, const Tables<T>&, bool, const cpx<T>* const*,            \
-                                       const int*, int, cpx<T>* const*, const Exec&);                       \
-  template cudaError_t launch_coef_x<T>(const Geom&, const Tables<T>&, const cpx<T>*, T*, T*, T*, int*,      \
-                                        const CoefCopy&, const Exec&);                                      \
-  template cudaError_t launch_coef_phys<T>(const Geom&, const double*, T*, T*, T*, int*, const CoefCopy&,   \
-                                           const Exec&);                                                    \
-  template cudaError_t launch_matvec<T>(const Geom&, const Tables<T>&, const cpx<T>*, const T*, const T*,    \
-                                        cpx<T>*, cpx<T>* const*, bool, const Exec&, const int*, size_t,     \
-                                        const MvTma*);                                                      \
-  template cudaError_t launch_spec_div<T>(const Geom&, const Tables<T>&, const cpx<T>*, const cpx<T>*,      \
-                                          cpx<T>*, const Exec&);                                            \
-  template cudaError_t launch_precond<T>(const Geom&, const Tables<T>&, const cpx<T>*, cpx<T>*, double*,    \
-                                         const Exec&);                                                      \
-  template cudaError_t launch_hermitian_fix<T>(const Geom&, cpx<T>*, const Exec&);
 
 }  // namespace sgn
