@@ -540,7 +540,7 @@ bool gmres_fp64(sgn_ctx* ctx, int* iters_out, double* relres_out) {
   double* beta_d = ctx->scal + 1;
   CK(launch_hermitian_fix<double>(G, ctx->bh, EX(ctx)));
   CK(launch_precond<double>(G, ctx->tb, ctx->bh, ctx->cvec, ctx->partials, EX(ctx)));
-  CK(launch_reduce(ctx->partials, 1, cnorm_d, true, nullptr, EX(ctx)));
+  CK(launch_reduce(ctx->partials, 1, cnorm_d, true, nullptr, EX(ctx), sweep_partials(G)));
   CK(launch_readback_scalar(cnorm_d, ctx->flags, ctx->rb_dev, EX(ctx)));
   sync_read(ctx);
   check_flags(ctx, ctx->rb_host->flags);
@@ -562,7 +562,7 @@ bool gmres_fp64(sgn_ctx* ctx, int* iters_out, double* relres_out) {
   for (;;) {
     CK(launch_matvec<double>(G, ctx->tb, ctx->sig, ctx->cr, ctx->cc, ctx->w, ctx->tmp, true, EX(ctx)));
     CK(launch_residual<double>(G, ctx->cvec, ctx->w, V, ctx->partials, EX(ctx)));
-    CK(launch_reduce(ctx->partials, 1, beta_d, true, nullptr, EX(ctx)));
+    CK(launch_reduce(ctx->partials, 1, beta_d, true, nullptr, EX(ctx), sweep_partials(G)));
     CK(launch_readback_scalar(beta_d, ctx->flags, ctx->rb_dev, EX(ctx)));
     sync_read(ctx);
     check_flags(ctx, ctx->rb_host->flags);
@@ -615,7 +615,7 @@ bool gmres_mixed(sgn_ctx* ctx, int* iters_out, double* relres_out) {
   double* beta_d = ctx->scal + 1;
   CK(launch_hermitian_fix<double>(G, ctx->bh, EX(ctx)));
   CK(launch_precond<double>(G, ctx->tb, ctx->bh, ctx->cvec, ctx->partials, EX(ctx)));
-  CK(launch_reduce(ctx->partials, 1, cnorm_d, true, nullptr, EX(ctx)));
+  CK(launch_reduce(ctx->partials, 1, cnorm_d, true, nullptr, EX(ctx), sweep_partials(G)));
   CK(launch_readback_scalar(cnorm_d, ctx->flags, ctx->rb_dev, EX(ctx)));
   sync_read(ctx);
   check_flags(ctx, ctx->rb_host->flags);
@@ -636,7 +636,7 @@ bool gmres_mixed(sgn_ctx* ctx, int* iters_out, double* relres_out) {
   for (;;) {
     refine_matvec(ctx, true, EX_REFINE(ctx));
     CK(launch_residual<double>(G, ctx->cvec, ctx->w, ctx->r64, ctx->partials, EX(ctx)));
-    CK(launch_reduce(ctx->partials, 1, beta_d, true, nullptr, EX(ctx)));
+    CK(launch_reduce(ctx->partials, 1, beta_d, true, nullptr, EX(ctx), sweep_partials(G)));
     CK(launch_readback_scalar(beta_d, ctx->flags, ctx->rb_dev, EX(ctx)));
     sync_read(ctx);
     check_flags(ctx, ctx->rb_host->flags);
@@ -1024,7 +1024,7 @@ void graph_gmres(sgn_ctx* ctx, GraphSeg& top) {
   long long fixed = count_launches(ctx, [&] {
     CK(launch_hermitian_fix<double>(G, ctx->bh, EX(ctx)));
     CK(launch_precond<double>(G, ctx->tb, ctx->bh, ctx->cvec, ctx->partials, EX(ctx)));
-    CK(launch_reduce(ctx->partials, 1, cnorm_d, true, nullptr, EX(ctx)));
+    CK(launch_reduce(ctx->partials, 1, cnorm_d, true, nullptr, EX(ctx), sweep_partials(G)));
     CK(launch_ctl_begin(ctx->gst, cnorm_d, ctl, EX(ctx)));
     CK(launch_zero<double>(G, ctx->sig, EX(ctx), &ctx->gst->zero_sigma));
   });
@@ -1036,7 +1036,7 @@ void graph_gmres(sgn_ctx* ctx, GraphSeg& top) {
     refine_matvec(ctx, true, EX(ctx));
     C64* r = mixed ? ctx->r64 : ctx->V;
     CK(launch_residual<double>(G, ctx->cvec, ctx->w, r, ctx->partials, EX(ctx)));
-    CK(launch_reduce(ctx->partials, 1, beta_d, true, nullptr, EX(ctx)));
+    CK(launch_reduce(ctx->partials, 1, beta_d, true, nullptr, EX(ctx), sweep_partials(G)));
     CK(launch_ctl_sweep(ctx->gst, beta_d, ctl, EX(ctx)));
     if (mixed)
       CK((launch_scale<double, float>(G, r, beta_d, true, ctx->V32, EX(ctx))));
@@ -1984,7 +1984,7 @@ sgn_status sgn_invariants(sgn_t ctx, const double* h, const double* vx, const do
   inv2(ctx, in, dx, dy, 2, o);
   CK(launch_invariant_sums(ctx->G, h, vx, vy, sigma, ctx->phys[0], ctx->phys[1], ctx->g, ctx->partials,
                            EX(ctx)));
-  CK(launch_reduce(ctx->partials, 4, ctx->scal + 4, false, nullptr, EX(ctx)));
+  CK(launch_reduce(ctx->partials, 4, ctx->scal + 4, false, nullptr, EX(ctx), NBLK));
   CK(cudaMemcpyAsync(ctx->inv_host, ctx->scal + 4, 4 * sizeof(double), cudaMemcpyDeviceToHost, ctx->stream));
   CK(cudaStreamSynchronize(ctx->stream));
   const double dA = ctx->G.Lx * ctx->G.Ly / (double)ctx->G.nphys();

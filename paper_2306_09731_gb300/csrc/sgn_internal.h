@@ -405,9 +405,12 @@ cudaError_t launch_axpby(const Geom& G, double a, const cpx<T>* x, double b, cpx
 template <typename T>
 cudaError_t launch_copy_gated(const Geom& G, const cpx<T>* x, cpx<T>* y, const int* gate, const Exec& ex);
 
-// reduce partials[b][0..n) over blocks into out[0..n); if sqrt_out, take sqrt
+// reduce the first nblk block partials of n slots into out[0..n); if sqrt_out, take sqrt
 cudaError_t launch_reduce(const double* partials, int n, double* out, bool sqrt_out, const int* gate,
-                          const Exec& ex);
+                          const Exec& ex, int nblk);
+// blocks of the sweeps that leave partials for launch_reduce (launch_precond,
+// launch_residual)
+int sweep_partials(const Geom& G);
 // GMRES scalar kernels (one thread)
 cudaError_t launch_gmres_start(GmresDev* st, const double* beta, const Exec& ex);
 cudaError_t launch_backsolve(GmresDev* st, int k, const Exec& ex, const int* kdev = nullptr);

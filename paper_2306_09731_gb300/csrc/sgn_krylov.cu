@@ -71,6 +71,16 @@ __device__ __forceinline__ double reduce_slot(const double* partials, int slot, 
 // block reductions and the last block's sum over the partials are a fixed
 // cost per block)
 constexpr int KBLK = 608;
+// Blocks of a sweep over n entries: at least `per` entries a thread (256
+// threads), so that short vectors do not pay the reductions (or the launch) of
+// blocks without work; at most `most`. (256^2, 33,280 entries, averages over a step
+// of the paper's method with the reductions below: k_dots<double> 27 -> 11 us,
+// k_cgs_update<double> 15.5 -> 12.7 us.) The grid depends on the vector's length only, so that sums stay
+// deterministic and graph mode equal to the host loop.
+static inline int sweep_blocks(const Geom& G, int per, int most) {
+  const size_t n = G.nspec(), b = (n + 256 * (size_t)per - 1) / (256 * (size_t)per);
+  return b < (size_t)most ? (int)b : most;
+}
 
 // out[s] = sum of the first nblk partials of slot s (slot stride NBLK),
 // s < nslots, one warp per slot:
@@ -98,20 +108,48 @@ __device__ __forceinline__ void reduce_slots(const double* partials, int nslots,
   }
 }
 
-// Block sums of K values with one barrier: thread k (< K) returns the sum of
-// value k. Each warp sums in the accumulation type A (FP32 for the FP32
-// vectors: an FP64 shuffle tree costs more FP64-pipe time than the sweep
-// itself on this part), then the warp sums are added in FP64 in a fixed order.
-// red: K * 32 doubles of shared memory.
+// Warp sums of 8 values: the lanes with bits (4, 3, 2) = k hold the sum of
+// value k. The first three steps halve the number of values a lane carries (4 +
+// 2 + 1 additions, then 1 + 1) where a tree per value takes 40: an FP64
+// addition costs a warp 77 issue cycles here.
+template <typename A>
+__device__ __forceinline__ A warp_sum8(const A (&v)[8]) {
+  const int lane = threadIdx.x & 31;
+  const bool h4 = lane & 16, h3 = lane & 8, h2 = lane & 4;
+  A a[4], b[2];
+#pragma unroll
+  for (int k = 0; k < 4; ++k) {
+    const A keep = h4 ? v[4 + k] : v[k], give = h4 ? v[k] : v[4 + k];
+    a[k] = keep + __shfl_xor_sync(0xffffffffu, give, 16);
+  }
+#pragma unroll
+  for (int k = 0; k < 2; ++k) {
+    const A keep = h3 ? a[2 + k] : a[k], give = h3 ? a[k] : a[2 + k];
+    b[k] = keep + __shfl_xor_sync(0xffffffffu, give, 8);
+  }
+  const A keep = h2 ? b[1] : b[0], give = h2 ? b[0] : b[1];
+  A c = keep + __shfl_xor_sync(0xffffffffu, give, 4);
+  c += __shfl_xor_sync(0xffffffffu, c, 2);
+  c += __shfl_xor_sync(0xffffffffu, c, 1);
+  return c;
+}
+
+// Block sums of K <= 8 values with one barrier: thread k (< K) returns the sum
+// of value k. Each warp sums in the accumulation type A, then the warp sums
+// are added in FP64 in a fixed order. red: 8 * 32 doubles of shared memory.
 template <int K, typename A>
-__device__ __forceinline__ double block_reduce_multi(A (&v)[K], double* red) {
+__device__ __forceinline__ double block_reduce_multi(const A (&v)[K], double* red) {
   const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5, nw = blockDim.x >> 5;
+  if constexpr (K == 1) {
+    A c = v[0];
+    for (int o = 16; o > 0; o >>= 1) c += __shfl_xor_sync(0xffffffffu, c, o);
+    if (lane == 0) red[wid] = (double)c;
+  } else {
+    A e[8];
 #pragma unroll
-  for (int k = 0; k < K; ++k)
-    for (int o = 16; o > 0; o >>= 1) v[k] += __shfl_xor_sync(0xffffffffu, v[k], o);
-  if (lane == 0) {
-#pragma unroll
-    for (int k = 0; k < K; ++k) red[k * 32 + wid] = (double)v[k];
+    for (int k = 0; k < 8; ++k) e[k] = k < K ? v[k < K ? k : 0] : (A)0;
+    const A c = warp_sum8(e);
+    if ((lane & 3) == 0 && (lane >> 2) < K) red[(lane >> 2) * 32 + wid] = (double)c;
   }
   __syncthreads();
   double t = 0.0;
@@ -150,7 +188,7 @@ __global__ void __launch_bounds__(256, 4) k_dots(Geom G, const cpx<T>* V, size_t
   typedef typename Acc<T>::type A;
   if (gate && *gate == 0) return;
   if (jdev) nv = *jdev + 1;
-  __shared__ double red[(DOT_CHUNK + 1) * 32];
+  __shared__ double red[8 * 32];
   for (int i0 = 0; i0 < nv; i0 += DOT_CHUNK) {
     const int nc = min(DOT_CHUNK, nv - i0);
     const bool chunk0 = i0 == 0;
@@ -382,13 +420,13 @@ __global__ void k_zero(Geom G, cpx<T>* x, const int* gate) {
   for (Walk it(G); it.ok(); it.next()) x[it.e] = mk((T)0, (T)0);
 }
 
-// out[i] = sum_b partials[i*NBLK + b] (fixed order), i < n. Gated.
-__global__ void k_reduce(const double* partials, int n, double* out, int sqrt_out, const int* gate) {
+// out[i] = sum_b partials[i*NBLK + b] (fixed order, b < nblk), i < n. Gated.
+__global__ void k_reduce(const double* partials, int n, double* out, int sqrt_out, const int* gate, int nblk) {
   if (gate && *gate == 0) return;
   __shared__ double red[32];
   for (int i = 0; i < n; ++i) {
     double v = 0.0;
-    for (int b = threadIdx.x; b < NBLK; b += blockDim.x) v += partials[(size_t)i * NBLK + b];
+    for (int b = threadIdx.x; b < nblk; b += blockDim.x) v += partials[(size_t)i * NBLK + b];
     const double tot = block_reduce(v, red);
     if (threadIdx.x == 0) out[i] = sqrt_out ? sqrt(tot) : tot;
   }
@@ -671,12 +709,14 @@ __global__ void __launch_bounds__(256) k_invariant_sums(Geom G, const double* h,
 
 // ------------------------------------------------------------- launchers
 
+int sweep_partials(const Geom& G) { return sweep_blocks(G, 1, NBLK); }
+
 template <typename T>
 cudaError_t launch_dots(const Geom& G, const cpx<T>* V, size_t vstride, int nv, const cpx<T>* w,
                         double* partials, const int* gate, double* out, unsigned* counter, const Exec& ex,
                         const int* jdev, const double* vscl) {
   ex.begin(PK_KRYLOV);
-  k_dots<T><<<KBLK, 256, 0, ex.s>>>(G, V, vstride, nv, w, partials, gate, out, counter, jdev, vscl);
+  k_dots<T><<<sweep_blocks(G, 2, KBLK), 256, 0, ex.s>>>(G, V, vstride, nv, w, partials, gate, out, counter, jdev, vscl);
   ex.end();
   return cudaGetLastError();
 }
@@ -688,7 +728,7 @@ cudaError_t launch_cgs_update(const Geom& G, const cpx<T>* V, size_t vstride, in
   GraphCtl c{};
   if (ctl) c = *ctl;
   ex.begin(PK_KRYLOV);
-  k_cgs_update<T><<<KBLK, 256, 0, ex.s>>>(G, V, vstride, nv, coef, w, partials, gate, st, j, pass, counter, rb,
+  k_cgs_update<T><<<sweep_blocks(G, 2, KBLK), 256, 0, ex.s>>>(G, V, vstride, nv, coef, w, partials, gate, st, j, pass, counter, rb,
                                          flags, jdev, c, scaled ? 1 : 0);
   ex.end();
   return cudaGetLastError();
@@ -697,7 +737,7 @@ template <typename T>
 cudaError_t launch_residual(const Geom& G, const cpx<T>* c, const cpx<T>* w, cpx<T>* r, double* partials,
                             const Exec& ex) {
   ex.begin(PK_KRYLOV);
-  k_residual<T><<<NBLK, 256, 0, ex.s>>>(G, c, w, r, partials);
+  k_residual<T><<<sweep_blocks(G, 1, NBLK), 256, 0, ex.s>>>(G, c, w, r, partials);
   ex.end();
   return cudaGetLastError();
 }
@@ -705,7 +745,7 @@ template <typename TI, typename TO>
 cudaError_t launch_scale(const Geom& G, const cpx<TI>* x, const double* factor, bool invert, cpx<TO>* y,
                          const Exec& ex, const int* ysel, size_t ystride) {
   ex.begin(PK_KRYLOV);
-  k_scale<TI, TO><<<NBLK, 256, 0, ex.s>>>(G, x, factor, invert ? 1 : 0, y, ysel, ystride);
+  k_scale<TI, TO><<<sweep_blocks(G, 1, NBLK), 256, 0, ex.s>>>(G, x, factor, invert ? 1 : 0, y, ysel, ystride);
   ex.end();
   return cudaGetLastError();
 }
@@ -713,14 +753,14 @@ template <typename TV, typename TX>
 cudaError_t launch_axpy_multi(const Geom& G, const cpx<TV>* V, size_t vstride, int nv, const double* coef,
                               cpx<TX>* x, const Exec& ex, const int* ndev, const double* vscl) {
   ex.begin(PK_KRYLOV);
-  k_axpy_multi<TV, TX><<<NBLK, 256, 0, ex.s>>>(G, V, vstride, nv, coef, x, ndev, vscl);
+  k_axpy_multi<TV, TX><<<sweep_blocks(G, 1, NBLK), 256, 0, ex.s>>>(G, V, vstride, nv, coef, x, ndev, vscl);
   ex.end();
   return cudaGetLastError();
 }
 template <typename T>
 cudaError_t launch_zero(const Geom& G, cpx<T>* x, const Exec& ex, const int* gate) {
   ex.begin(PK_KRYLOV);
-  k_zero<T><<<NBLK, 256, 0, ex.s>>>(G, x, gate);
+  k_zero<T><<<sweep_blocks(G, 1, NBLK), 256, 0, ex.s>>>(G, x, gate);
   ex.end();
   return cudaGetLastError();
 }
@@ -729,22 +769,22 @@ template <typename T>
 cudaError_t launch_axpby(const Geom& G, double a, const cpx<T>* x, double b, cpx<T>* y, const Exec& ex,
                          const int* gate, const int* gate2) {
   ex.begin(PK_KRYLOV);
-  k_axpby<T><<<NBLK, 256, 0, ex.s>>>(G, a, x, b, y, gate, gate2);
+  k_axpby<T><<<sweep_blocks(G, 1, NBLK), 256, 0, ex.s>>>(G, a, x, b, y, gate, gate2);
   ex.end();
   return cudaGetLastError();
 }
 template <typename T>
 cudaError_t launch_copy_gated(const Geom& G, const cpx<T>* x, cpx<T>* y, const int* gate, const Exec& ex) {
   ex.begin(PK_KRYLOV);
-  k_copy_gated<T><<<NBLK, 256, 0, ex.s>>>(G, x, y, gate);
+  k_copy_gated<T><<<sweep_blocks(G, 1, NBLK), 256, 0, ex.s>>>(G, x, y, gate);
   ex.end();
   return cudaGetLastError();
 }
 
 cudaError_t launch_reduce(const double* partials, int n, double* out, bool sqrt_out, const int* gate,
-                          const Exec& ex) {
+                          const Exec& ex, int nblk) {
   ex.begin(PK_KRYLOV);
-  k_reduce<<<1, 256, 0, ex.s>>>(partials, n, out, sqrt_out ? 1 : 0, gate);
+  k_reduce<<<1, 256, 0, ex.s>>>(partials, n, out, sqrt_out ? 1 : 0, gate, nblk);
   ex.end();
   return cudaGetLastError();
 }
@@ -781,7 +821,7 @@ cudaError_t launch_ctl_after(GmresDev* st, GraphCtl ctl, const Exec& ex) {
 cudaError_t launch_same_state(const Geom& G, const cpx<double>* const* a, const cpx<double>* const* b, double rel,
                               double* partials, unsigned* counter, int* flag, const Exec& ex) {
   ex.begin(PK_KRYLOV);
-  k_same_state<<<NBLK, 256, 0, ex.s>>>(G, a[0], a[1], a[2], b[0], b[1], b[2], rel, partials, counter, flag);
+  k_same_state<<<sweep_blocks(G, 1, NBLK), 256, 0, ex.s>>>(G, a[0], a[1], a[2], b[0], b[1], b[2], rel, partials, counter, flag);
   ex.end();
   return cudaGetLastError();
 }
@@ -796,14 +836,14 @@ cudaError_t launch_set_int(int* p, int v, const Exec& ex) {
 cudaError_t launch_ext_start(const Geom& G, const cpx<double>* ring, int s, const ExtHist* hist, cpx<double>* sig,
                              const Exec& ex) {
   ex.begin(PK_KRYLOV);
-  k_ext_start<<<NBLK, 256, 0, ex.s>>>(G, ring, G.nspec(), s, hist, sig);
+  k_ext_start<<<sweep_blocks(G, 1, NBLK), 256, 0, ex.s>>>(G, ring, G.nspec(), s, hist, sig);
   ex.end();
   return cudaGetLastError();
 }
 cudaError_t launch_ext_store(const Geom& G, const cpx<double>* sig, cpx<double>* ring, int s, const ExtHist* hist,
                              const Exec& ex) {
   ex.begin(PK_KRYLOV);
-  k_ext_store<<<NBLK, 256, 0, ex.s>>>(G, sig, ring, G.nspec(), s, hist);
+  k_ext_store<<<sweep_blocks(G, 1, NBLK), 256, 0, ex.s>>>(G, sig, ring, G.nspec(), s, hist);
   ex.end();
   return cudaGetLastError();
 }

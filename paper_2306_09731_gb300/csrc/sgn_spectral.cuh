@@ -1940,7 +1940,7 @@ static cudaError_t launch_rk_update(const Geom& G, const Tables<S>& tbs, cpx<S>*
   a.sig = sig;
   a.rk = rk;
   ex.begin(PK_RK);
-  k_rk_update<T, S><<<NBLK, 256, 0, ex.s>>>(G, a, rk.dt / 6.0, rk.mode == RK_STAGE3 ? rk.dt : 0.5 * rk.dt,
+  k_rk_update<T, S><<<sweep_partials(G), 256, 0, ex.s>>>(G, a, rk.dt / 6.0, rk.mode == RK_STAGE3 ? rk.dt : 0.5 * rk.dt,
                                              rk.krasny_thr * rk.krasny_thr * (double)G.nphys() * (double)G.nphys());
   ex.end();
   return cudaGetLastError();
@@ -2027,7 +2027,7 @@ template <typename T>
 cudaError_t launch_spec_div(const Geom& G, const Tables<T>& tb, const cpx<T>* vx, const cpx<T>* vy, cpx<T>* b,
                             const Exec& ex) {
   ex.begin(PK_KRYLOV);
-  k_spec_div<T><<<NBLK, 256, 0, ex.s>>>(G, tb.kx, tb.ky, vx, vy, b);
+  k_spec_div<T><<<sweep_partials(G), 256, 0, ex.s>>>(G, tb.kx, tb.ky, vx, vy, b);
   ex.end();
   return cudaGetLastError();
 }
@@ -2054,7 +2054,7 @@ template <typename T>
 cudaError_t launch_precond(const Geom& G, const Tables<T>& tb, const cpx<T>* in, cpx<T>* out, double* partials,
                            const Exec& ex) {
   ex.begin(PK_KRYLOV);
-  k_precond<T><<<NBLK, 256, 0, ex.s>>>(G, tb.kx, tb.ky, tb.minv, in, out, partials);
+  k_precond<T><<<sweep_partials(G), 256, 0, ex.s>>>(G, tb.kx, tb.ky, tb.minv, in, out, partials);
   ex.end();
   return cudaGetLastError();
 }
