@@ -22,7 +22,7 @@ static inline void fx_ln(int lN, F&& f) {
 static void fx_x_config(const Geom& G, dim3& grid, dim3& block, size_t& smem, int nf, int extra_per_pair = 0,
                         int tpb = 0) {
   const int Tn = G.Nx >> 3;
-  int P = fx_default_pairs(G);
+  int P = builtin_pairs(G);
   if (tpb > 0 && tpb % Tn == 0) {
     const int q = tpb / Tn;
     if ((q & (q - 1)) == 0 && tpb <= (G.lNx == 12 ? 512 : 256) && q <= (G.Ny >> 1)) P = q;
@@ -33,7 +33,7 @@ static void fx_x_config(const Geom& G, dim3& grid, dim3& block, size_t& smem, in
 }
 static void fx_y_config(const Geom& G, dim3& grid, dim3& block, size_t& smem, int nf, int stash = 0, int tpb = 0) {
   const int Tn = G.Ny >> 3;
-  int C = fx_default_cols(G);
+  int C = builtin_cols(G, TT_F64, 1);
   if (tpb >= 32 && tpb % Tn == 0) {
     const int q = tpb / Tn;
     if ((q & (q - 1)) == 0 && q <= 64 && tpb <= (G.lNy == 12 ? 512 : 256)) C = q;

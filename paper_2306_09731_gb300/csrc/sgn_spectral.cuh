@@ -646,21 +646,24 @@ __device__ __forceinline__ cpx<T> ld_as(const cpx<S>* p) {
 // Column tile: C = blockDim / (Ny/8) neighbouring kx columns, thread index
 // c + C*t. Each input column is transformed in registers; the epilogue gets
 // all NIN results of the thread's 8 rows.
-// Threads of a y-pass block. FP32: 512 (two columns per block at Ny = 2048,
-// twice the bytes per row segment). FP64: 256, the registers of one column per
-// block (measured at 2048^2: inverse 321 against 371 us and forward 327
-// against 386 us with 512). Double-float: 256, one column per block, three
-// blocks per SM for the passes that hold one signal at a time (see
-// ypass_body).
-// At 4096 points (LN = 12) one column takes 512 threads in every type.
-// FP32 passes with at most two inputs (NIN <= 2): 1024 threads, four columns
-// per block at Ny = 2048, so that a warp's access covers 8 rows x 32 bytes (8
-// cache lines) instead of 16 rows x 16 bytes (16 lines): the strided column
-// accesses cost L1 wavefronts per line touched.
+// Threads of a y-pass block.
+// Double-float: 256, one column per block at 2048, three blocks per SM for the
+// passes that hold one signal at a time (see ypass_body); 512 at 4096 points
+// (LN = 12), where one column takes them.
+// FP32 at the compile-time lengths: four columns per block, so that a warp's
+// access covers 8 rows x 32 bytes (8 cache lines) instead of 16 rows x 16
+// bytes (16 lines): the strided column accesses cost L1 wavefronts per line
+// touched (at 2048, matvec y-inverse 41.5 -> 33.4 us against two); fewer where
+// four do not fit 1024 threads (512 with three or more inputs, whose registers
+// do not fit more). Blocks of a fixed 1024 threads would hold 32 columns at 256
+// points, five blocks for a 256^2 grid: matvec y-inverse 12.5 us there against
+// 7.7, RHS y-forward 14.1 against 7.7 (1024 x 512: 14.8 -> 9.3, 12.3 -> 10.0).
+// LN = 0: the most threads a tuned shape may have.
+constexpr int f32_cols(int lN, int nin) { return nin <= 2 ? (lN == 12 ? 2 : 4) : (lN == 12 ? 1 : (lN == 11 ? 2 : 4)); }
 template <typename T, bool INV, int LN = 0, int NIN = 0>
 constexpr int ypass_threads() {
-  if (sizeof(T) == 4 && NIN >= 1 && NIN <= 2) return 1024;
-  return (sizeof(T) == 4 || LN == 12) ? 512 : 256;
+  if (sizeof(T) == 4) return LN > 0 ? (1 << (LN - 3)) * f32_cols(LN, NIN) : (NIN <= 2 ? 1024 : 512);
+  return LN == 12 ? 512 : 256;
 }
 
 constexpr int ilog2c(int n) { return n <= 1 ? 0 : 1 + ilog2c(n / 2); }
@@ -1075,20 +1078,20 @@ __global__ void __launch_bounds__(ypass_threads<T, INV, LN, NIN>()) k_ypass(Geom
   ypass_body<T, INV, NIN, Epi, S, LN, FL, PLAN>(G, tw, ky, in, epi);
 }
 // FP32 passes with at most two transforms per thread: 64 registers, 32 warps
-// per SM (measured with two 512-thread blocks: matvec y-forward 34 against
+// per SM (16 below 2048 points, whose index arithmetic spills at 64; measured with two 512-thread blocks: matvec y-forward 34 against
 // 39 us at 2048^2 with the compiler's choice). The other passes keep the
 // compiler's register choice.
-template <typename T, bool INV, int NIN>
-constexpr int ypass_o2_blocks() { return ypass_threads<T, INV, 0, NIN>() >= 1024 ? 1 : 2; }
+template <typename T, bool INV, int NIN, int LN>
+constexpr int ypass_o2_blocks() { return ((LN >= 8 && LN <= 10) ? 512 : 1024) / ypass_threads<T, INV, LN, NIN>(); }
 template <typename T, bool INV, int NIN, class Epi, typename S = T, int LN = 0, int FL = 0, int PLAN = 0>
-__global__ void __launch_bounds__(ypass_threads<T, INV, LN, NIN>(), ypass_o2_blocks<T, INV, NIN>()) k_ypass_o2(Geom G, const cpx<T>* __restrict__ tw,
+__global__ void __launch_bounds__(ypass_threads<T, INV, LN, NIN>(), ypass_o2_blocks<T, INV, NIN, LN>()) k_ypass_o2(Geom G, const cpx<T>* __restrict__ tw,
                                                                         const T* __restrict__ ky,
                                                                         YIn<T, NIN, S> in, Epi epi) {
   ypass_body<T, INV, NIN, Epi, S, LN, FL, PLAN>(G, tw, ky, in, epi);
 }
 // FP32 passes whose inputs arrive by tensor copies (see yf_tma)
 template <typename T, bool INV, int NIN, class Epi, int LN, int FL, int PLAN = 0>
-__global__ void __launch_bounds__(ypass_threads<T, INV, LN, NIN>(), ypass_o2_blocks<T, INV, NIN>())
+__global__ void __launch_bounds__(ypass_threads<T, INV, LN, NIN>(), ypass_o2_blocks<T, INV, NIN, LN>())
     k_ypass_tma(Geom G, const cpx<T>* __restrict__ tw, const T* __restrict__ ky, YIn<T, NIN, T> in,
                 const __grid_constant__ YTma tm, Epi epi) {
   ypass_body<T, INV, NIN, Epi, T, LN, FL, PLAN>(G, tw, ky, in, epi, &tm);
@@ -1376,18 +1379,32 @@ static inline void dispatch_l12(int lN, F&& f) {
     f(std::integral_constant<int, 0>());
 }
 
-template <typename T>
-static inline int x_pairs_per_block(const Geom& G) {
-  int Tn = G.Nx >> 3;
+// Built-in shapes. Blocks of 256 threads (256 or 512 threads where one
+// transform takes them), fewer where the grid would leave SMs idle (under two
+// blocks each of 152), but at least a warp a block and, for columns, two
+// neighbours (32-byte segments of the 16-byte types). At 256^2 (128 row pairs in
+// 128 blocks instead of 16): double-float matvec x-pass 36.2 -> 30.8 us, FP32
+// RHS x-pass 15.4 -> 12.4; at 1024 x 512 54.5 -> 49.5 and 19.2 -> 18.4.
+static inline int builtin_pairs(const Geom& G) {
+  const int Tn = G.Nx >> 3, half = G.Ny >> 1;
   int P = Tn >= 256 ? 1 : 256 / Tn;
-  int half = G.Ny >> 1;
   if (P > half) P = half;
+  while (P > 1 && (half + P - 1) / P < 304 && Tn * P >= 64) P >>= 1;
   return P;
+}
+// type: TuneType; nin: the pass's inputs (FP32)
+static inline int builtin_cols(const Geom& G, int type, int nin) {
+  if (type == TT_F32 && G.lNy >= 8) return f32_cols(G.lNy, nin);
+  const int Tn = G.Ny >> 3;
+  int C = 256 / Tn;
+  C = C < 1 ? 1 : (C > 64 ? 64 : C);
+  while (C > 2 && (G.Nxh + C - 1) / C < 304 && Tn * C >= 64) C >>= 1;
+  return C;
 }
 template <typename T>
 static inline void x_config(const Geom& G, dim3& grid, dim3& block, size_t& smem, int nf, int tpb = 0,
                             int extra_elems_per_group = 0) {
-  int P = x_pairs_per_block<T>(G);
+  int P = builtin_pairs(G);
   // tuned shape: whole row pairs, a power of two, within the launch bound
   const int Tn = G.Nx >> 3;
   if (tpb > 0 && tpb % Tn == 0) {
@@ -1403,9 +1420,7 @@ static inline void y_config(const Geom& G, dim3& grid, dim3& block, size_t& smem
                             int tpb_tuned = 0, bool* builtin = nullptr) {
   const int Tn = G.Ny >> 3;
   const int bound = G.lNy == 12 ? ypass_threads<T, INV, 12, NIN>() : ypass_threads<T, INV, 0, NIN>();
-  int C = bound / Tn;
-  if (C < 1) C = 1;
-  if (C > 64) C = 64;
+  int C = builtin_cols(G, tune_type<T>(), NIN);
   const int C0 = C;
   // tuned shape: whole columns, a power of two, within the launch bound
   if (tpb_tuned > 0 && tpb_tuned % Tn == 0) {
@@ -1567,37 +1582,9 @@ static int y_bound(const Geom& G, int type, int pass) {
 static bool is_y_pass(int pass) { return pass <= TP_RHS_YFWD; }
 
 #ifdef SGN_SPECTRAL_COMMON
-// Columns (row pairs) per block of the FP64 passes: 256 threads, fewer where
-// the grid would leave SMs idle (fewer than two blocks each), but at least a
-// warp a block and, for columns, two neighbours (32-byte segments).
-static int fx_default_cols(const Geom& G) {
-  const int Tn = G.Ny >> 3;
-  int C = 256 / Tn;
-  C = C < 1 ? 1 : (C > 64 ? 64 : C);
-  while (C > 2 && (G.Nxh + C - 1) / C < 304 && Tn * C >= 64) C >>= 1;
-  return C;
-}
-static int fx_default_pairs(const Geom& G) {
-  const int Tn = G.Nx >> 3, half = G.Ny >> 1;
-  int P = Tn >= 256 ? 1 : 256 / Tn;
-  if (P > half) P = half;
-  while (P > 1 && (half + P - 1) / P < 304 && Tn * P >= 64) P >>= 1;
-  return P;
-}
-
 int pass_default_threads(const Geom& G, int type, int pass) {
-  if (type == TT_F64) return is_y_pass(pass) ? (G.Ny >> 3) * fx_default_cols(G) : (G.Nx >> 3) * fx_default_pairs(G);
-  if (is_y_pass(pass)) {
-    const int Tn = G.Ny >> 3;
-    int C = y_bound(G, type, pass) / Tn;
-    if (C < 1) C = 1;
-    if (C > 64) C = 64;
-    return Tn * C;
-  }
-  const int Tn = G.Nx >> 3;
-  int P = Tn >= 256 ? 1 : 256 / Tn;
-  if (P > (G.Ny >> 1)) P = G.Ny >> 1;
-  return Tn * P;
+  const int nin = (pass == TP_MV_YINV || pass == TP_MV_YFWD) ? 2 : (pass == TP_RHS_YINV ? 4 : 3);
+  return is_y_pass(pass) ? (G.Ny >> 3) * builtin_cols(G, type, nin) : (G.Nx >> 3) * builtin_pairs(G);
 }
 #endif  // SGN_SPECTRAL_COMMON
 
