@@ -41,9 +41,6 @@ __device__ __forceinline__ __nv_bfloat16 tof<__nv_bfloat16>(float v) {
   return __float2bfloat16_rn(v);
 }
 
-constexpr int TILE = 16;   // output tile side of the 3x3 convolution
-constexpr int COT = 8;     // output channels per block
-
 // 3x3 periodic convolution. Forward (TR = false):
 //   out[b][co][y][x] = bias[co] + sum_ci sum_k w[co][ci][k] in[b][ci][y+ky-1][x+kx-1]
 // Transposed (TR = true, the gradient with respect to the input): the output
@@ -51,56 +48,352 @@ constexpr int COT = 8;     // output channels per block
 // channel o, and the kernel is flipped:
 //   out[b][c][y][x] = sum_o sum_k w[o][c][8-k] in[b][o][y+ky-1][x+kx-1]
 // (Cw: the forward input-channel count, the row length of w.) H, W are powers
-// of two; in and out have batch strides ibs, obs (elements).
-template <typename TI, typename TO, bool TR>
-__global__ void __launch_bounds__(TILE* TILE) k_conv3(const TI* __restrict__ in, size_t ibs, int Ci, TO* out,
-                                                      size_t obs, int Co, const float* __restrict__ w,
-                                                      const float* __restrict__ bias, int Cw, int H, int W,
-                                                      int relu) {
-  __shared__ float tile[TILE + 2][TILE + 2];
-  __shared__ float ws[COT][9];
-  const int tx = threadIdx.x, ty = threadIdx.y, tid = ty * TILE + tx;
-  const int tiles_x = (W + TILE - 1) / TILE;
-  const int x0 = (blockIdx.x % tiles_x) * TILE, y0 = (blockIdx.x / tiles_x) * TILE;
+// of two >= 4; in and out have batch strides ibs, obs (elements).
+//
+// FP32-FMA bound in principle (44 of the 65 GFLOP of a training step of the
+// 471,873-parameter network, batch 8 at 128^2). A thread keeps PX pixels x COT
+// channels of sums in registers, as channel pairs for the packed FMA: with 8 x 8
+// an input channel costs 288 packed FMAs (576 issue cycles of an SM quarter)
+// against 27 shared loads (18 of them broadcasts of weights; 432). With 4 x 8 the
+// loads cost more than the FMAs (360 against 288), with one pixel x 8 channels and
+// a load per FMA they were all of it. Each stage of CCK input channels is
+// fetched with every load in flight before the first is stored: a loop of
+// dependent fetch-and-store pairs took 20 us a stage. Loss and gradients of one
+// batch of 8 at 128^2: 11.5 -> 3.0 ms (with the weight gradients below).
+// Each sum runs over (ci, ky, kx) in order, one rounded FMA at a time, whatever
+// the tile: BF16 activations do not depend on it.
+// Tile: TX x TY threads of PX x 1 pixels, TX = min(W / PX, 8),
+// TY = min(H, 128 / TX, 16).
+template <int PX>
+constexpr int conv_cck() { return PX == 8 ? 4 : 8; }  // input channels per stage
+// four consecutive elements as floats
+__device__ __forceinline__ float4 load4(const float* p) { return *reinterpret_cast<const float4*>(p); }
+__device__ __forceinline__ float4 load4(const __nv_bfloat16* p) {
+  const uint2 r = *reinterpret_cast<const uint2*>(p);
+  return make_float4(__uint_as_float(r.x << 16), __uint_as_float(r.x & 0xffff0000u), __uint_as_float(r.y << 16),
+                     __uint_as_float(r.y & 0xffff0000u));
+}
+__device__ __forceinline__ void store4(float* p, float a, float b, float c, float d) {
+  *reinterpret_cast<float4*>(p) = make_float4(a, b, c, d);
+}
+__device__ __forceinline__ void store4(__nv_bfloat16* p, float a, float b, float c, float d) {
+  const __nv_bfloat162 u = __halves2bfloat162(__float2bfloat16_rn(a), __float2bfloat16_rn(b));
+  const __nv_bfloat162 v = __halves2bfloat162(__float2bfloat16_rn(c), __float2bfloat16_rn(d));
+  uint2 r;
+  r.x = *reinterpret_cast<const unsigned*>(&u);
+  r.y = *reinterpret_cast<const unsigned*>(&v);
+  *reinterpret_cast<uint2*>(p) = r;
+}
+
+// Stages rows [0, nrow) of a tile: row r = (channel r / RPC, line r % RPC) at
+// dst + dsto(r), tw interior pixels from element 4 on and the halo at 3 and
+// tw + 4. 16-byte (8-byte) fetches, U in flight per thread.
+template <int U, typename TI, class Src, class Dst>
+__device__ __forceinline__ void stage_rows(int nrow, int ltw, int tid, int nthr, int x0, int W, Src src, Dst dst) {
+  const int lv = ltw - 2, nvec = nrow << lv;  // 4-pixel vectors per row: 2^lv
+  for (int base = 0; base < nvec; base += U * nthr) {
+    float4 q[U];
+#pragma unroll
+    for (int u = 0; u < U; ++u) {
+      const int i = base + u * nthr + tid;
+      if (i < nvec) q[u] = load4(src(i >> lv) + x0 + 4 * (i & ((1 << lv) - 1)));
+    }
+#pragma unroll
+    for (int u = 0; u < U; ++u) {
+      const int i = base + u * nthr + tid;
+      if (i < nvec) *reinterpret_cast<float4*>(dst(i >> lv) + 4 + 4 * (i & ((1 << lv) - 1))) = q[u];
+    }
+  }
+  const int tw = 1 << ltw;
+  for (int base = 0; base < 2 * nrow; base += 4 * nthr) {
+    float q[4];
+#pragma unroll
+    for (int u = 0; u < 4; ++u) {
+      const int i = base + u * nthr + tid;
+      if (i < 2 * nrow) q[u] = ldf(src(i >> 1) + ((x0 + ((i & 1) ? tw : -1)) & (W - 1)));
+    }
+#pragma unroll
+    for (int u = 0; u < 4; ++u) {
+      const int i = base + u * nthr + tid;
+      if (i < 2 * nrow) dst(i >> 1)[(i & 1) ? tw + 4 : 3] = q[u];
+    }
+  }
+}
+
+template <typename TI, typename TO, bool TR, int COT, int PX>
+__global__ void __launch_bounds__(128) k_conv3(const TI* __restrict__ in, size_t ibs, int Ci, TO* out, size_t obs,
+                                               const float* __restrict__ w, const float* __restrict__ bias, int Cw,
+                                               int H, int W, int lTX, int relu) {
+  constexpr int CP = COT / 2, CCK = conv_cck<PX>(), LPX = PX == 8 ? 3 : 2;
+  const int TX = 1 << lTX, TY = blockDim.x >> lTX, RPC = TY + 2;
+  const int tid = threadIdx.x, tx = tid & (TX - 1), ty = tid >> lTX;
+  const int ltw = lTX + LPX, tw = 1 << ltw, RS = tw + 8;
+  extern __shared__ __align__(16) float csm[];
+  float* tile = csm;                             // [CCK][TY + 2][RS]
+  float* ws = csm + (size_t)CCK * RPC * RS;      // [CCK][9][COT]
+  const int tiles_x = W / tw;
+  const int x0 = (blockIdx.x % tiles_x) * tw, y0 = (blockIdx.x / tiles_x) * TY;
   const int co0 = blockIdx.y * COT, b = blockIdx.z;
   const size_t HW = (size_t)H * W;
   const TI* inb = in + (size_t)b * ibs;
-  float acc[COT];
+  // r / RPC for r < 256, RPC in 6..18
+  const unsigned inv = 65536u / (unsigned)RPC + 1u;
+  float2 acc[PX][CP];
 #pragma unroll
-  for (int c = 0; c < COT; ++c) acc[c] = 0.f;
-  for (int ci = 0; ci < Ci; ++ci) {
-    const TI* src = inb + (size_t)ci * HW;
-    for (int i = tid; i < (TILE + 2) * (TILE + 2); i += TILE * TILE) {
-      const int ly = i / (TILE + 2), lx = i % (TILE + 2);
-      const int gy = (y0 + ly - 1) & (H - 1), gx = (x0 + lx - 1) & (W - 1);
-      tile[ly][lx] = ldf(src + (size_t)gy * W + gx);
-    }
-    if (tid < COT * 9) {
-      const int c = tid / 9, k = tid % 9, co = co0 + c;
-      float v = 0.f;
-      if (co < Co) v = TR ? w[((size_t)ci * Cw + co) * 9 + (8 - k)] : w[((size_t)co * Ci + ci) * 9 + k];
-      ws[c][k] = v;
-    }
-    __syncthreads();
+  for (int p = 0; p < PX; ++p)
 #pragma unroll
-    for (int ky = 0; ky < 3; ++ky)
+    for (int c = 0; c < CP; ++c) acc[p][c] = make_float2(0.f, 0.f);
+  for (int c0 = 0; c0 < Ci; c0 += CCK) {
+    const int nc = min(CCK, Ci - c0);
+    if (c0) __syncthreads();
+    stage_rows<9, TI>(
+        nc * RPC, ltw, tid, blockDim.x, x0, W,
+        [&](int r) {
+          const int ci = (int)((unsigned)r * inv >> 16), ly = r - ci * RPC;
+          return inb + (size_t)(c0 + ci) * HW + (size_t)((y0 + ly - 1) & (H - 1)) * W;
+        },
+        [&](int r) { return tile + r * RS; });
+    constexpr int WU = (CCK * 9 * COT + 127) / 128;
+    const int nwt = nc * 9 * COT;
+    for (int base = 0; base < nwt; base += WU * blockDim.x) {
+      float q[WU];
+      int to[WU];
 #pragma unroll
-      for (int kx = 0; kx < 3; ++kx) {
-        const float v = tile[ty + ky][tx + kx];
-#pragma unroll
-        for (int c = 0; c < COT; ++c) acc[c] = fmaf(ws[c][ky * 3 + kx], v, acc[c]);
+      for (int u = 0; u < WU; ++u) {
+        const int i = base + u * (int)blockDim.x + tid;
+        // TR: w[c0 + ci][co0 + c][8 - k], c then ci outermost; else w[co0 + c][c0 + ci][k]
+        const int k = i % 9, m = i / 9, ci = TR ? m / COT : m % nc, c = TR ? m % COT : m / nc;
+        to[u] = (ci * 9 + k) * COT + c;
+        if (i < nwt)
+          q[u] = TR ? w[((size_t)(c0 + ci) * Cw + co0 + c) * 9 + (8 - k)] : w[((size_t)(co0 + c) * Ci + c0 + ci) * 9 + k];
       }
+#pragma unroll
+      for (int u = 0; u < WU; ++u)
+        if (base + u * (int)blockDim.x + tid < nwt) ws[to[u]] = q[u];
+    }
     __syncthreads();
+    for (int ci = 0; ci < nc; ++ci) {
+      const float* wc = ws + ci * 9 * COT;
+#pragma unroll
+      for (int ky = 0; ky < 3; ++ky) {
+        const float* row = tile + (ci * RPC + ty + ky) * RS + 4 + PX * tx;
+        float v[PX + 2];
+        v[0] = row[-1];
+        v[PX + 1] = row[PX];
+#pragma unroll
+        for (int p = 0; p < PX; p += 4) {
+          const float4 q = *reinterpret_cast<const float4*>(row + p);
+          v[p + 1] = q.x;
+          v[p + 2] = q.y;
+          v[p + 3] = q.z;
+          v[p + 4] = q.w;
+        }
+#pragma unroll
+        for (int kx = 0; kx < 3; ++kx) {
+          float2 wv[CP];
+#pragma unroll
+          for (int c = 0; c < CP; c += 2) {
+            const float4 q = *reinterpret_cast<const float4*>(wc + (ky * 3 + kx) * COT + 2 * c);
+            wv[c] = make_float2(q.x, q.y);
+            wv[c + 1] = make_float2(q.z, q.w);
+          }
+#pragma unroll
+          for (int p = 0; p < PX; ++p) {
+            const float2 vv = make_float2(v[p + kx], v[p + kx]);
+#pragma unroll
+            for (int c = 0; c < CP; ++c) acc[p][c] = __ffma2_rn(wv[c], vv, acc[p][c]);
+          }
+        }
+      }
+    }
   }
-  const int y = y0 + ty, x = x0 + tx;
-  if (y >= H || x >= W) return;
+  const int y = y0 + ty, x = x0 + PX * tx;
 #pragma unroll
   for (int c = 0; c < COT; ++c) {
-    const int co = co0 + c;
-    if (co >= Co) break;
-    float v = acc[c] + (bias ? bias[co] : 0.f);
-    if (relu) v = fmaxf(v, 0.f);
-    out[(size_t)b * obs + (size_t)co * HW + (size_t)y * W + x] = tof<TO>(v);
+    const float bb = bias ? bias[co0 + c] : 0.f;
+    float o[PX];
+#pragma unroll
+    for (int p = 0; p < PX; ++p) {
+      o[p] = ((c & 1) ? acc[p][c >> 1].y : acc[p][c >> 1].x) + bb;
+      if (relu) o[p] = fmaxf(o[p], 0.f);
+    }
+    TO* dst = out + (size_t)b * obs + (size_t)(co0 + c) * HW + (size_t)y * W + x;
+#pragma unroll
+    for (int p = 0; p < PX; p += 4) store4(dst + p, o[p], o[p + 1], o[p + 2], o[p + 3]);
+  }
+}
+
+// Weight gradients dw[co][ci][k] = sum_{b,y,x} dp[b][co][y][x] in[b][ci][y+ky-1][x+kx-1]
+// and db[co] = sum dp[b][co], as partial sums of a split of the pixels.
+// A block takes 16 input x 32 output channels and the chunks z, z + splits, ...
+// of up to 128 pixels (R rows x CW columns); a thread one input channel and 4
+// output channels: 36 sums in registers, fed by 10 vector loads per 4 pixels and
+// 72 packed FMAs: 71 us a layer on average in the step above. (One block per
+// channel pair read every activation 9 Co times.) A chunk is summed on its own before it is added, so that no sum
+// runs over more than 128 terms. Fixed order: deterministic.
+constexpr int DWPX = 128;
+__host__ __device__ inline void dw_chunk(int H, int W, int* R, int* CW) {
+  *CW = W < 64 ? W : 64;
+  const int r = DWPX / *CW;
+  *R = r < H ? r : H;
+}
+__host__ __device__ inline int dw_row_stride(int CW) { return CW + 8; }
+// words per input channel of the staged tile, = 4 mod 32 (conflict-free 16-byte loads)
+__host__ __device__ inline int dw_in_stride(int R, int CW) {
+  const int n = (R + 2) * dw_row_stride(CW);
+  return (n + 27) / 32 * 32 + 4;
+}
+template <typename TI>
+__global__ void __launch_bounds__(128, 4) k_conv3_dw(const TI* __restrict__ in, size_t ibs, int Ci,
+                                                  const float* __restrict__ dp, size_t dbs, int Co, int H, int W,
+                                                  int B, float* part) {
+  extern __shared__ __align__(16) float csm[];
+  int R, CW;
+  dw_chunk(H, W, &R, &CW);
+  const int RS = dw_row_stride(CW), IS = dw_in_stride(R, CW);
+  float* ti = csm;            // [16][IS]
+  float* tg = csm + 16 * IS;  // [R * CW][32 + 4]
+  constexpr int GS = 36;
+  const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+  const int cl = tid & 15, cg = tid >> 4;
+  const int ci0 = blockIdx.x * 16, co0 = blockIdx.y * 32, splits = gridDim.z;
+  const size_t HW = (size_t)H * W;
+  const int cpr = W / CW, chunks = B * (H / R) * cpr;
+  const int lCW = 31 - __clz(CW), nin = min(16, Ci - ci0);
+  const unsigned inv = 65536u / (unsigned)(R + 2) + 1u;  // r / (R + 2), r < 16 (R + 2) <= 288
+  // channels past Ci contribute zeros
+  for (int i = nin * IS + tid; i < 16 * IS; i += 128) ti[i] = 0.f;
+  float2 acc[9][2];
+  float2 ab[2];
+#pragma unroll
+  for (int k = 0; k < 9; ++k) acc[k][0] = acc[k][1] = make_float2(0.f, 0.f);
+  ab[0] = ab[1] = make_float2(0.f, 0.f);
+  for (int ch = blockIdx.z; ch < chunks; ch += splits) {
+    const int b = ch / ((H / R) * cpr), rem = ch - b * (H / R) * cpr;
+    const int y0 = rem / cpr * R, x0 = (rem % cpr) * CW;
+    __syncthreads();
+    stage_rows<9, TI>(
+        nin * (R + 2), lCW, tid, 128, x0, W,
+        [&](int r) {
+          const int c = (int)((unsigned)r * inv >> 16), ly = r - c * (R + 2);
+          return in + (size_t)b * ibs + (size_t)(ci0 + c) * HW + (size_t)((y0 + ly - 1) & (H - 1)) * W;
+        },
+        [&](int r) {
+          const int c = (int)((unsigned)r * inv >> 16);
+          return ti + c * IS + (r - c * (R + 2)) * RS;
+        });
+    // lane = output channel: conflict-free transposed stores
+    const int nv = R * CW / 4;
+    const bool gok = co0 + lane < Co;
+    const float* gsrc = dp + (size_t)b * dbs + (size_t)(gok ? co0 + lane : 0) * HW + (size_t)y0 * W + x0;
+    float4 q[8];
+#pragma unroll
+    for (int u = 0; u < 8; ++u) {
+      const int i = 4 * u + warp;
+      if (i < nv) {
+        const int ly = 4 * i >> lCW;
+        q[u] = gok ? load4(gsrc + (size_t)ly * W + (4 * i - (ly << lCW))) : make_float4(0.f, 0.f, 0.f, 0.f);
+      }
+    }
+#pragma unroll
+    for (int u = 0; u < 8; ++u) {
+      const int i = 4 * u + warp;
+      if (i < nv) {
+        float* t = tg + 4 * i * GS + lane;
+        t[0] = q[u].x;
+        t[GS] = q[u].y;
+        t[2 * GS] = q[u].z;
+        t[3 * GS] = q[u].w;
+      }
+    }
+    __syncthreads();
+    float2 s[9][2], sb[2];
+#pragma unroll
+    for (int k = 0; k < 9; ++k) s[k][0] = s[k][1] = make_float2(0.f, 0.f);
+    sb[0] = sb[1] = make_float2(0.f, 0.f);
+    for (int r = 0; r < R; ++r) {
+      for (int x = 0; x < CW; x += 4) {
+        float2 g[4][2];
+#pragma unroll
+        for (int p = 0; p < 4; ++p) {
+          const float4 q = *reinterpret_cast<const float4*>(tg + (r * CW + x + p) * GS + 4 * cg);
+          g[p][0] = make_float2(q.x, q.y);
+          g[p][1] = make_float2(q.z, q.w);
+        }
+#pragma unroll
+        for (int ky = 0; ky < 3; ++ky) {
+          const float* row = ti + cl * IS + (r + ky) * RS + 4 + x;
+          const float4 ra = *reinterpret_cast<const float4*>(row);
+          const float v[6] = {row[-1], ra.x, ra.y, ra.z, ra.w, row[4]};
+#pragma unroll
+          for (int kx = 0; kx < 3; ++kx)
+#pragma unroll
+            for (int p = 0; p < 4; ++p) {
+              const float2 vv = make_float2(v[p + kx], v[p + kx]);
+              s[ky * 3 + kx][0] = __ffma2_rn(g[p][0], vv, s[ky * 3 + kx][0]);
+              s[ky * 3 + kx][1] = __ffma2_rn(g[p][1], vv, s[ky * 3 + kx][1]);
+            }
+        }
+        if (cl == 0) {
+#pragma unroll
+          for (int p = 0; p < 4; ++p) {
+            sb[0] = __fadd2_rn(sb[0], g[p][0]);
+            sb[1] = __fadd2_rn(sb[1], g[p][1]);
+          }
+        }
+      }
+    }
+#pragma unroll
+    for (int k = 0; k < 9; ++k) {
+      acc[k][0] = __fadd2_rn(acc[k][0], s[k][0]);
+      acc[k][1] = __fadd2_rn(acc[k][1], s[k][1]);
+    }
+    ab[0] = __fadd2_rn(ab[0], sb[0]);
+    ab[1] = __fadd2_rn(ab[1], sb[1]);
+  }
+  // this split's sums: [Co][Ci][9], then [Co]
+  float* o = part + (size_t)blockIdx.z * ((size_t)Co * Ci * 9 + Co);
+  const int ci = ci0 + cl;
+#pragma unroll
+  for (int c = 0; c < 4; ++c) {
+    const int co = co0 + 4 * cg + c;
+    if (co >= Co) continue;
+    if (ci < Ci) {
+#pragma unroll
+      for (int k = 0; k < 9; ++k)
+        o[((size_t)co * Ci + ci) * 9 + k] = (c & 1) ? acc[k][c >> 1].y : acc[k][c >> 1].x;
+    }
+    if (ci0 == 0 && cl == 0) o[(size_t)Co * Ci * 9 + co] = (c & 1) ? ab[c >> 1].y : ab[c >> 1].x;
+  }
+}
+// blocks of pixel chunks a weight gradient is split into: about 600 blocks in all
+inline int dw_splits(int Ci, int Co, int H, int W, int B) {
+  int R, CW;
+  dw_chunk(H, W, &R, &CW);
+  const int tiles = ((Ci + 15) / 16) * ((Co + 31) / 32), chunks = B * (H / R) * (W / CW);
+  const int s = (600 + tiles - 1) / tiles;
+  return s < chunks ? s : chunks;
+}
+// out[i] = sum of the splits' partial sums: 8 threads a sum, each over every
+// 8th split, then in order (32 x 8 threads)
+__global__ void __launch_bounds__(256) k_part_sum(const float* __restrict__ part, int n, int splits, float* out) {
+  __shared__ float red[8][32];
+  const int i = blockIdx.x * 32 + threadIdx.x;
+  float s[4] = {0.f, 0.f, 0.f, 0.f};
+  if (i < n) {
+    int z = threadIdx.y;
+    for (; z + 24 < splits; z += 32)
+#pragma unroll
+      for (int u = 0; u < 4; ++u) s[u] += part[(size_t)(z + 8 * u) * n + i];
+    for (; z < splits; z += 8) s[0] += part[(size_t)z * n + i];
+  }
+  red[threadIdx.y][threadIdx.x] = (s[0] + s[1]) + (s[2] + s[3]);
+  __syncthreads();
+  if (threadIdx.y == 0 && i < n) {
+    float t = 0.f;
+#pragma unroll
+    for (int z = 0; z < 8; ++z) t += red[z][threadIdx.x];
+    out[i] = t;
   }
 }
 
@@ -122,38 +415,6 @@ __device__ __forceinline__ void block_sum(float (&v)[K], float* red /* K * 32 */
     }
 }
 
-// dw[co][ci][k] = sum_{b,y,x} dp[b][co][y][x] in[b][ci][y+ky-1][x+kx-1];
-// db[co] = sum dp[b][co] (blocks with ci = 0). One block per (co, ci).
-template <typename TI>
-__global__ void __launch_bounds__(256) k_conv3_dw(const TI* __restrict__ in, size_t ibs, int Ci,
-                                                  const float* __restrict__ dp, size_t dbs, int Co, int H, int W,
-                                                  int B, float* dw, float* db) {
-  __shared__ float red[10 * 32];
-  const int co = blockIdx.x, ci = blockIdx.y;
-  const size_t HW = (size_t)H * W;
-  float acc[10];
-#pragma unroll
-  for (int k = 0; k < 10; ++k) acc[k] = 0.f;
-  for (size_t p = threadIdx.x; p < (size_t)B * HW; p += blockDim.x) {
-    const int b = (int)(p / HW);
-    const int yx = (int)(p % HW), y = yx / W, x = yx % W;
-    const float g = dp[(size_t)b * dbs + (size_t)co * HW + yx];
-    const TI* src = in + (size_t)b * ibs + (size_t)ci * HW;
-#pragma unroll
-    for (int ky = 0; ky < 3; ++ky) {
-      const int gy = (y + ky - 1) & (H - 1);
-#pragma unroll
-      for (int kx = 0; kx < 3; ++kx) acc[ky * 3 + kx] = fmaf(g, ldf(src + (size_t)gy * W + ((x + kx - 1) & (W - 1))), acc[ky * 3 + kx]);
-    }
-    acc[9] += g;
-  }
-  block_sum<10>(acc, red);
-  if (threadIdx.x == 0) {
-    for (int k = 0; k < 9; ++k) dw[((size_t)co * Ci + ci) * 9 + k] = acc[k];
-    if (ci == 0) db[co] = acc[9];
-  }
-}
-
 // 1x1 convolution C -> 1 (the output layer), FP32 output
 template <typename T>
 __global__ void k_conv1_fwd(const T* __restrict__ in, size_t ibs, int C, const float* __restrict__ w,
@@ -166,27 +427,21 @@ __global__ void k_conv1_fwd(const T* __restrict__ in, size_t ibs, int C, const f
   out[i] = v;
 }
 
-// gradients of the output layer: dw[c] = sum dout in[c], db = sum dout
-// (block c < C: dw[c]; block C: db) and din[c] = w[c] dout masked by in > 0
-// (the ReLU of the layer before).
+// gradients of the output layer: dw[c] = sum dout in[c], db = sum dout (block
+// c < C: dw[c]; block C: db), as partial sums part[z][c] of gridDim.y ranges of
+// the pixels; din[c] = w[c] dout masked by in > 0 (the ReLU of the layer before).
 template <typename T>
 __global__ void __launch_bounds__(256) k_conv1_dw(const T* __restrict__ in, size_t ibs, int C,
-                                                  const float* __restrict__ dout, int HW, int B, float* dw,
-                                                  float* db) {
+                                                  const float* __restrict__ dout, int HW, int B, float* part) {
   __shared__ float red[32];
   const int c = blockIdx.x;
   float acc[1] = {0.f};
-  for (int i = threadIdx.x; i < B * HW; i += blockDim.x) {
+  for (int i = blockIdx.y * blockDim.x + threadIdx.x; i < B * HW; i += gridDim.y * blockDim.x) {
     const int b = i / HW, yx = i % HW;
     acc[0] += dout[i] * (c < C ? ldf(in + (size_t)b * ibs + (size_t)c * HW + yx) : 1.f);
   }
   block_sum<1>(acc, red);
-  if (threadIdx.x == 0) {
-    if (c < C)
-      dw[c] = acc[0];
-    else
-      db[0] = acc[0];
-  }
+  if (threadIdx.x == 0) part[(size_t)blockIdx.y * (C + 1) + c] = acc[0];
 }
 
 template <typename T>
@@ -256,25 +511,38 @@ __global__ void k_up_bwd(const float* __restrict__ dout, size_t obs, float* din,
   din[(size_t)b * ibs + r] = (s[0] + s[1]) + (s[2 * W] + s[2 * W + 1]);
 }
 
-// dout = 2 (out - target) / n; loss = sum (out - target)^2 / n (one block)
-__global__ void __launch_bounds__(1024) k_mse(const float* __restrict__ out, const float* __restrict__ target,
-                                              float* dout, int n, double* loss) {
+// dout = 2 (out - target) / n; loss = sum (out - target)^2 / n: block sums in
+// part, added in order by the last block to finish (ticket: zeroed, left zeroed)
+constexpr int MSE_BLOCKS = 128;
+__global__ void __launch_bounds__(256) k_mse(const float* __restrict__ out, const float* __restrict__ target,
+                                             float* dout, int n, double* loss, double* part, unsigned* ticket) {
   __shared__ double red[32];
+  __shared__ int s_last;
   double acc = 0.0;
   const float s = 2.f / (float)n;
-  for (int i = threadIdx.x; i < n; i += blockDim.x) {
+  for (int i = blockIdx.x * blockDim.x + threadIdx.x; i < n; i += gridDim.x * blockDim.x) {
     const float d = out[i] - target[i];
     dout[i] = s * d;
     acc += (double)d * d;
   }
+  if (!loss) return;
   for (int o = 16; o > 0; o >>= 1) acc += __shfl_xor_sync(0xffffffffu, acc, o);
   if ((threadIdx.x & 31) == 0) red[threadIdx.x >> 5] = acc;
   __syncthreads();
-  if (threadIdx.x == 0 && loss) {
+  if (threadIdx.x == 0) {
     double t = 0.0;
     for (int i = 0; i < (int)(blockDim.x >> 5); ++i) t += red[i];
-    *loss = t / (double)n;
+    part[blockIdx.x] = t;
+    __threadfence();
+    s_last = atomicAdd(ticket, 1u) == gridDim.x - 1;
+    if (s_last) *ticket = 0u;
   }
+  __syncthreads();
+  if (!s_last || threadIdx.x >= 32) return;
+  double t = 0.0;
+  for (int i = threadIdx.x; i < (int)gridDim.x; i += 32) t += __ldcg(part + i);
+  for (int o = 16; o > 0; o >>= 1) t += __shfl_xor_sync(0xffffffffu, t, o);
+  if (threadIdx.x == 0) *loss = t / (double)n;
 }
 
 __global__ void k_adam(float* p, const float* __restrict__ g, float* m, float* v, long long n, float lr, float b1,
@@ -292,6 +560,7 @@ __global__ void k_adam(float* p, const float* __restrict__ g, float* m, float* v
 inline unsigned blocks_for(size_t n, int t = 256) { return (unsigned)((n + t - 1) / t); }
 
 constexpr int kMaxLevels = 6;
+constexpr int kConv1Splits = 16;  // ranges of pixels in the output layer's gradient
 
 struct Layer {
   int Ci, Co, k;
@@ -320,6 +589,10 @@ struct sgn_unet_ctx {
   //   U[l]   w_l channels: d_l's output (l < D-1), b1's output (l = D-1)
   void *A[kMaxLevels] = {}, *CAT[kMaxLevels] = {}, *Q[kMaxLevels] = {}, *U[kMaxLevels] = {};
   float *OUT = nullptr, *gOUT = nullptr;
+  // partial sums of the weight gradients and of the loss
+  float* part = nullptr;
+  double* mse_part = nullptr;
+  unsigned* ticket = nullptr;
   // FP32 gradients: two scratch tensors of wmax channels per level, and the
   // concatenation's gradient per level
   float *G[kMaxLevels][2] = {}, *gCAT[kMaxLevels] = {};
@@ -395,27 +668,55 @@ void init_params(sgn_unet_ctx* net, unsigned long long seed) {
   UCK(cudaMemset(net->grads, 0, sizeof(float) * (size_t)net->P));
 }
 
+template <typename TI, typename TO, bool TR, int COT, int PX>
+void conv3_tile(sgn_unet_ctx* net, const TI* in, size_t ibs, int Ci, TO* out, size_t obs, int Co, const float* w,
+                const float* bias, int Cw, int H, int B, bool relu) {
+  int lTX = 0;
+  while (lTX < 3 && (2 * PX << lTX) <= H) ++lTX;
+  const int TX = 1 << lTX;
+  int TY = 128 / TX;
+  TY = TY < 16 ? TY : 16;
+  TY = TY < H ? TY : H;
+  const dim3 grid((unsigned)((H / (PX * TX)) * (H / TY)), Co / COT, B);
+  const size_t smem =
+      sizeof(float) * conv_cck<PX>() * ((size_t)(TY + 2) * (PX * TX + 8) + 9 * (size_t)COT);
+  k_conv3<TI, TO, TR, COT, PX><<<grid, TX * TY, smem, net->stream>>>(in, ibs, Ci, out, obs, w, bias, Cw, H, H, lTX,
+                                                                    relu ? 1 : 0);
+  UCK(cudaGetLastError());
+}
+// Ci input and Co output channels (Co a multiple of 16): 8 pixels x 8 channels
+// a thread where that leaves two blocks per SM (64 x 16 pixels each), else 4 x 8
+template <typename TI, typename TO, bool TR>
+void conv3_launch(sgn_unet_ctx* net, const TI* in, size_t ibs, int Ci, TO* out, size_t obs, int Co, const float* w,
+                  const float* bias, int Cw, int H, int B, bool relu) {
+  if (H >= 64 && (long long)(H / 64) * (H / 16) * (Co / 8) * B >= 256)
+    conv3_tile<TI, TO, TR, 8, 8>(net, in, ibs, Ci, out, obs, Co, w, bias, Cw, H, B, relu);
+  else
+    conv3_tile<TI, TO, TR, 8, 4>(net, in, ibs, Ci, out, obs, Co, w, bias, Cw, H, B, relu);
+}
 template <typename TI, typename TO>
 void conv3(sgn_unet_ctx* net, const TI* in, size_t ibs, int li, TO* out, size_t obs, int H, int B, bool relu) {
   const Layer& l = net->L[li];
-  dim3 grid(((H + TILE - 1) / TILE) * ((H + TILE - 1) / TILE), (l.Co + COT - 1) / COT, B);
-  k_conv3<TI, TO, false><<<grid, dim3(TILE, TILE), 0, net->stream>>>(
-      in, ibs, l.Ci, out, obs, l.Co, net->params + l.woff, net->params + l.boff, l.Ci, H, H, relu ? 1 : 0);
-  UCK(cudaGetLastError());
+  conv3_launch<TI, TO, false>(net, in, ibs, l.Ci, out, obs, l.Co, net->params + l.woff, net->params + l.boff, l.Ci, H,
+                              B, relu);
 }
 // gradient with respect to the layer input (channels Ci) from dp (channels Co)
 void conv3_dx(sgn_unet_ctx* net, const float* dp, size_t dbs, int li, float* dx, size_t xbs, int H, int B) {
   const Layer& l = net->L[li];
-  dim3 grid(((H + TILE - 1) / TILE) * ((H + TILE - 1) / TILE), (l.Ci + COT - 1) / COT, B);
-  k_conv3<float, float, true><<<grid, dim3(TILE, TILE), 0, net->stream>>>(
-      dp, dbs, l.Co, dx, xbs, l.Ci, net->params + l.woff, nullptr, l.Ci, H, H, 0);
-  UCK(cudaGetLastError());
+  conv3_launch<float, float, true>(net, dp, dbs, l.Co, dx, xbs, l.Ci, net->params + l.woff, nullptr, l.Ci, H, B,
+                                   false);
 }
 template <typename TI>
 void conv3_dw(sgn_unet_ctx* net, const TI* in, size_t ibs, const float* dp, size_t dbs, int li, int H, int B) {
   const Layer& l = net->L[li];
-  k_conv3_dw<TI><<<dim3(l.Co, l.Ci), 256, 0, net->stream>>>(in, ibs, l.Ci, dp, dbs, l.Co, H, H, B,
-                                                             net->grads + l.woff, net->grads + l.boff);
+  int R, CW;
+  dw_chunk(H, H, &R, &CW);
+  const int splits = dw_splits(l.Ci, l.Co, H, H, B), n = l.Co * l.Ci * 9 + l.Co;
+  const size_t smem = sizeof(float) * (16 * (size_t)dw_in_stride(R, CW) + (size_t)R * CW * 36);
+  k_conv3_dw<TI><<<dim3((l.Ci + 15) / 16, (l.Co + 31) / 32, splits), 128, smem, net->stream>>>(
+      in, ibs, l.Ci, dp, dbs, l.Co, H, H, B, net->part);
+  UCK(cudaGetLastError());
+  k_part_sum<<<blocks_for(n, 32), dim3(32, 8), 0, net->stream>>>(net->part, n, splits, net->grads + l.woff);
   UCK(cudaGetLastError());
 }
 template <typename T>
@@ -480,12 +781,15 @@ void backward_impl(sgn_unet_ctx* net, const float* target, double* loss) {
   const int D = net->D, B = net->lastB;
   const int* w = net->w;
   const size_t N0 = npix(net, 0);
-  k_mse<<<1, 1024, 0, net->stream>>>(net->OUT, target, net->gOUT, (int)(B * N0), loss);
+  k_mse<<<MSE_BLOCKS, 256, 0, net->stream>>>(net->OUT, target, net->gOUT, (int)(B * N0), loss, net->mse_part,
+                                              net->ticket);
   UCK(cudaGetLastError());
   // output layer w_0 -> 1, then the ReLU of d_0
   const Layer& lo = net->L[iOut(net)];
-  k_conv1_dw<T><<<w[0] + 1, 256, 0, net->stream>>>((const T*)net->U[0], (size_t)w[0] * N0, w[0], net->gOUT, (int)N0,
-                                                   B, net->grads + lo.woff, net->grads + lo.boff);
+  k_conv1_dw<T><<<dim3(w[0] + 1, kConv1Splits), 256, 0, net->stream>>>((const T*)net->U[0], (size_t)w[0] * N0, w[0],
+                                                                       net->gOUT, (int)N0, B, net->part);
+  UCK(cudaGetLastError());
+  k_part_sum<<<blocks_for(w[0] + 1, 32), dim3(32, 8), 0, net->stream>>>(net->part, w[0] + 1, kConv1Splits, net->grads + lo.woff);
   UCK(cudaGetLastError());
   k_conv1_dx_relu<T><<<blocks_for((size_t)B * w[0] * N0), 256, 0, net->stream>>>(
       (const T*)net->U[0], (size_t)w[0] * N0, w[0], net->params + lo.woff, net->gOUT, net->G[0][0],
@@ -759,6 +1063,17 @@ sgn_status create_impl(int n, int max_batch, int act_bf16, unsigned long long se
     const size_t N0 = npix(net, 0);
     net->OUT = (float*)ualloc(net, sizeof(float) * B * N0);
     net->gOUT = (float*)ualloc(net, sizeof(float) * B * N0);
+    size_t npart = (size_t)kConv1Splits * (w[0] + 1);
+    for (const Layer& l : net->L) {
+      if (l.k != 3) continue;
+      const int H = n >> l.level;
+      const size_t np = (size_t)dw_splits(l.Ci, l.Co, H, H, max_batch) * ((size_t)l.Co * l.Ci * 9 + l.Co);
+      npart = np > npart ? np : npart;
+    }
+    net->part = (float*)ualloc(net, sizeof(float) * npart);
+    net->mse_part = (double*)ualloc(net, sizeof(double) * MSE_BLOCKS);
+    net->ticket = (unsigned*)ualloc(net, sizeof(unsigned));
+    UCK(cudaMemset(net->ticket, 0, sizeof(unsigned)));
     net->wimg = (__nv_bfloat16*)ualloc(net, bf * (size_t)(ioff > 0 ? ioff : 1));
     net->dev_err = (int*)ualloc(net, sizeof(int));
     UCK(cudaMemset(net->dev_err, 0, sizeof(int)));
