@@ -43,22 +43,34 @@ static void fx_y_config(const Geom& G, dim3& grid, dim3& block, size_t& smem, in
   smem = (size_t)C * ((size_t)G.Ny * (1 + stash) * sizeof(cpx<fx>) + kFxSlots * sizeof(unsigned) + sizeof(cpx<double>));
 }
 
+// Whether a pass of `blocks` blocks of `threads` threads runs its transforms side
+// by side in `phases` groups (PAR, see k_fx_mv_x): the groups must be whole
+// warps and fit the kernel's threads, and the GPU must have room, under two
+// blocks per SM.
+static bool fx_parallel(const dim3& grid, const dim3& block, int phases, int most = 384) {
+  return block.x % 32 == 0 && (int)block.x * phases <= most && grid.x < 304;
+}
+
 template <int L>
 static void fx_attrs() {
   set_smem<double>((const void*)k_fx_r2c<L>);
   set_smem<double>((const void*)k_fx_c2r<L>);
   set_smem<double>((const void*)k_fx_coef_x<L>);
-  set_smem<double>((const void*)k_fx_mv_x<L>);
-  set_smem<double>((const void*)k_fx_rhs_x<L>);
+  set_smem<double>((const void*)k_fx_mv_x<L, false>);
+  set_smem<double>((const void*)k_fx_rhs_x<L, false>);
   set_smem<double>((const void*)k_fx_y<true, L>);
   set_smem<double>((const void*)k_fx_y<false, L>);
-  set_smem<double>((const void*)k_fx_yfwd<2, L>);
-  set_smem<double>((const void*)k_fx_yfwd<3, L>);
+  set_smem<double>((const void*)k_fx_yfwd<2, L, false>);
+  set_smem<double>((const void*)k_fx_yfwd<3, L, false>);
 }
 template <>
 void init_kernel_attributes<double>() {
   fx_attrs<0>();
   fx_attrs<12>();
+  set_smem<double>((const void*)k_fx_mv_x<0, true>);
+  set_smem<double>((const void*)k_fx_rhs_x<0, true>);
+  set_smem<double>((const void*)k_fx_yfwd<2, 0, true>);
+  set_smem<double>((const void*)k_fx_yfwd<3, 0, true>);
   cudaGetLastError();
 }
 
@@ -148,6 +160,27 @@ cudaError_t launch_coef_x<double>(const Geom& G, const Tables<double>& tb, const
   return cudaGetLastError();
 }
 
+// the forward column transforms of NIN inputs and their epilogue
+template <int NIN>
+static void fx_yfwd(const Geom& G, const Tables<double>& tb, const FxYFwdArgs& a, int pass, int kind, const Exec& ex) {
+  dim3 grid, block;
+  size_t smem;
+  const int plan = ex.plan(TT_F64, pass);
+  fx_y_config(G, grid, block, smem, 1, NIN - 1, ex.tpb(TT_F64, pass));
+  ex.begin(kind);
+  if (fx_parallel(grid, block, NIN)) {
+    // a buffer and a stash per transform, slots and scales per group
+    const size_t C = block.x / (G.Ny >> 3);
+    smem = NIN * C * (2 * (size_t)G.Ny * sizeof(cpx<fx>) + kFxSlots * sizeof(unsigned) + sizeof(cpx<double>));
+    k_fx_yfwd<NIN, 0, true><<<grid, NIN * block.x, smem, ex.s>>>(G, tb.twy, a, plan);
+  } else {
+    fx_ln(G.lNy, [&](auto ln) {
+      k_fx_yfwd<NIN, decltype(ln)::value, false><<<grid, block, smem, ex.s>>>(G, tb.twy, a, plan);
+    });
+  }
+  ex.end();
+}
+
 template <>
 cudaError_t launch_matvec<double>(const Geom& G, const Tables<double>& tb, const cpx<double>* sig, const double* cr,
                                   const double* cc, cpx<double>* w, cpx<double>* const* tmp, bool precond,
@@ -164,10 +197,17 @@ cudaError_t launch_matvec<double>(const Geom& G, const Tables<double>& tb, const
   fx_y(G, tb, true, a, 2, 0.0, ex.plan(TT_F64, TP_MV_YINV), ex.tpb(TT_F64, TP_MV_YINV), PK_MV_YINV, ex);
   fx_x_config(G, grid, block, smem, 1, 10 * (G.Nx >> 3), ex.tpb(TT_F64, TP_MV_X));
   ex.begin(PK_MV_X);
-  fx_ln(G.lNx, [&](auto ln) {
-    k_fx_mv_x<decltype(ln)::value><<<grid, block, smem, ex.s>>>(G, tb.twx, tb.k2x, tmp[0], tmp[1], cr, cc, tmp[0],
-                                                                tmp[1], ex.plan(TT_F64, TP_MV_X));
-  });
+  if (fx_parallel(grid, block, 3)) {
+    const int P = (int)block.x / (G.Nx >> 3);
+    smem += (size_t)2 * P * (G.Nx * sizeof(cpx<fx>) + kFxSlots * sizeof(unsigned));
+    k_fx_mv_x<0, true><<<grid, 3 * block.x, smem, ex.s>>>(G, tb.twx, tb.k2x, tmp[0], tmp[1], cr, cc, tmp[0], tmp[1],
+                                                          ex.plan(TT_F64, TP_MV_X));
+  } else {
+    fx_ln(G.lNx, [&](auto ln) {
+      k_fx_mv_x<decltype(ln)::value, false><<<grid, block, smem, ex.s>>>(G, tb.twx, tb.k2x, tmp[0], tmp[1], cr, cc,
+                                                                         tmp[0], tmp[1], ex.plan(TT_F64, TP_MV_X));
+    });
+  }
   ex.end();
   FxYFwdArgs f{};
   f.src[0] = tmp[0];
@@ -175,12 +215,7 @@ cudaError_t launch_matvec<double>(const Geom& G, const Tables<double>& tb, const
   f.dst[0] = w;
   f.kr = tb.k2y;
   f.minv = precond ? tb.minv : nullptr;
-  fx_y_config(G, grid, block, smem, 1, 1, ex.tpb(TT_F64, TP_MV_YFWD));
-  ex.begin(PK_MV_YFWD);
-  fx_ln(G.lNy, [&](auto ln) {
-    k_fx_yfwd<2, decltype(ln)::value><<<grid, block, smem, ex.s>>>(G, tb.twy, f, ex.plan(TT_F64, TP_MV_YFWD));
-  });
-  ex.end();
+  fx_yfwd<2>(G, tb, f, TP_MV_YFWD, PK_MV_YFWD, ex);
   return cudaGetLastError();
 }
 
@@ -203,23 +238,27 @@ cudaError_t launch_rhs<double, double>(const Geom& G, const Tables<double>& tb, 
   // may overwrite the inputs
   fx_x_config(G, grid, block, smem, 1, 2 * G.Nx, ex.tpb(TT_F64, TP_RHS_X));
   ex.begin(PK_RHS_X);
-  fx_ln(G.lNx, [&](auto ln) {
-    k_fx_rhs_x<decltype(ln)::value><<<grid, block, smem, ex.s>>>(G, tb.twx, tb.kx, tmp[0], tmp[1], tmp[2], tmp[3], h,
-                                                                 cr, rk.g, kTwoPi / G.Lx, kTwoPi / G.Ly, tmp[0],
-                                                                 tmp[1], tmp[2], ex.plan(TT_F64, TP_RHS_X));
-  });
+  const double alx = kTwoPi / G.Lx, aly = kTwoPi / G.Ly;
+  const int xplan = ex.plan(TT_F64, TP_RHS_X);
+  if (fx_parallel(grid, block, 5, 640)) {
+    const size_t P = block.x / (G.Nx >> 3);
+    smem = 5 * P * (2 * (size_t)G.Nx * sizeof(cpx<fx>) + kFxSlots * sizeof(unsigned) + sizeof(cpx<double>));
+    k_fx_rhs_x<0, true><<<grid, 5 * block.x, smem, ex.s>>>(G, tb.twx, tb.kx, tmp[0], tmp[1], tmp[2], tmp[3], h, cr,
+                                                           rk.g, alx, aly, tmp[0], tmp[1], tmp[2], xplan);
+  } else {
+    fx_ln(G.lNx, [&](auto ln) {
+      k_fx_rhs_x<decltype(ln)::value, false><<<grid, block, smem, ex.s>>>(G, tb.twx, tb.kx, tmp[0], tmp[1], tmp[2],
+                                                                          tmp[3], h, cr, rk.g, alx, aly, tmp[0],
+                                                                          tmp[1], tmp[2], xplan);
+    });
+  }
   ex.end();
   FxYFwdArgs f{};
   for (int i = 0; i < 3; ++i) f.src[i] = f.dst[i] = tmp[i];
   f.kr = tb.ky;
   f.kx = tb.kx;
   f.dealias = rk.dealias;
-  fx_y_config(G, grid, block, smem, 1, 2, ex.tpb(TT_F64, TP_RHS_YFWD));
-  ex.begin(PK_RHS_YFWD);
-  fx_ln(G.lNy, [&](auto ln) {
-    k_fx_yfwd<3, decltype(ln)::value><<<grid, block, smem, ex.s>>>(G, tb.twy, f, ex.plan(TT_F64, TP_RHS_YFWD));
-  });
-  ex.end();
+  fx_yfwd<3>(G, tb, f, TP_RHS_YFWD, PK_RHS_YFWD, ex);
   return launch_rk_update<double, double>(G, tbs, U, sig, tmp, Un, Unext, acc, bhat, rk, ex);
 }
 
