@@ -88,6 +88,8 @@ struct sgn_ctx {
   GmresReadback* rb_host = nullptr;  // pinned
   double* inv_host = nullptr;        // pinned, 4 doubles
   int* flags = nullptr;
+  bool ortho = false;                      // Arnoldi steps orthogonalise in one launch (ortho_fits)
+  unsigned long long* bar_count = nullptr;  // its grid barrier
   unsigned* counters = nullptr;  // last-block reduction tickets (zeroed, self-resetting)
   Prof prof;
   // graph mode (opt.graph = 1): one RK4 step as an instantiated graph
@@ -478,7 +480,7 @@ void check_flags(sgn_ctx* ctx, int flags) {
     throw Fail{SGN_ECAVITATION};
   }
   if (flags & FLAG_WAIT) {
-    ctx->err = "a y-pass stopped waiting for its tensor copies (bounded wait ran out)";
+    ctx->err = "a kernel stopped waiting for its tensor copies or its grid (bounded wait ran out)";
     throw Fail{SGN_ECUDA};
   }
 }
@@ -494,6 +496,16 @@ void coef_from_spectral(sgn_ctx* ctx, const C64* hh) {
   CK(launch_y_fft<double>(ctx->G, ctx->tb, true, &hh, nullptr, 1, ctx->tmp, EX(ctx, PK_COEF)));
   CK(launch_coef_x<double>(ctx->G, ctx->tb, ctx->tmp[0], ctx->h, ctx->cr, ctx->cc, ctx->flags, coef_copy(ctx),
                             EX(ctx)));
+}
+
+// Whether Arnoldi steps on vectors of type T take the one-launch form: the FP64
+// ones, whose second pass nearly always runs (four kernels to one). The FP32
+// step has two to save, a wash for one solver at a time, and the cooperative
+// launches of an ensemble's members keep one another waiting (12 members: 42 ms
+// with two kernels, 58 with one).
+template <typename T>
+bool use_ortho(const sgn_ctx* ctx) {
+  return ctx->ortho && sizeof(T) == 8;
 }
 
 // One Arnoldi step of the inner or outer GMRES on the basis V (type T):
@@ -513,15 +525,21 @@ void arnoldi_step(sgn_ctx* ctx, const Tables<T>& tb, const T* cr, const T* cc, c
   // pass: it only has to reduce its residual by 1e-6 and the FP64 refinement
   // checks the result (measured: same iteration and refinement counts, 4% faster)
   const bool dgks = sizeof(T) == 8;
-  // the FP32 basis is stored unnormalised (GmresDev::vscl): the update writes
-  // the next basis vector itself, with no scaling pass
-  const double* vscl = dgks ? nullptr : ctx->gst->vscl;
+  // the basis is stored unnormalised (GmresDev::vscl): the update writes the
+  // next basis vector itself, with no scaling pass
+  const double* vscl = ctx->gst->vscl;
+  if (use_ortho<T>(ctx)) {
+    CK(launch_ortho<T>(G, V, vs, w, ctx->partials, ctx->gst, j, dgks, ctx->bar_count, ctx->rb_dev, ctx->flags,
+                       EX(ctx)));
+    sync_read(ctx);
+    return;
+  }
   CK(launch_dots<T>(G, V, vs, nv, w, ctx->partials, nullptr, ctx->gst->h1, cnt + 0, EX(ctx), nullptr, vscl));
   CK(launch_cgs_update<T>(G, V, vs, nv, ctx->gst->h1, w, ctx->partials, nullptr, ctx->gst, j, dgks ? 1 : 3,
-                          cnt + 1, ctx->rb_dev, ctx->flags, EX(ctx), nullptr, nullptr, !dgks));
+                          cnt + 1, ctx->rb_dev, ctx->flags, EX(ctx)));
   if (dgks) {
-    CK(launch_dots<T>(G, V, vs, nv, w, ctx->partials, gate, ctx->gst->h2, cnt + 2, EX(ctx)));
-    CK(launch_cgs_update<T>(G, V, vs, nv, ctx->gst->h2, w, ctx->partials, gate, ctx->gst, j, 2, cnt + 3,
+    CK(launch_dots<T>(G, V, vs, nv, nullptr, ctx->partials, gate, ctx->gst->h2, cnt + 2, EX(ctx), nullptr, vscl));
+    CK(launch_cgs_update<T>(G, V, vs, nv, ctx->gst->h2, nullptr, ctx->partials, gate, ctx->gst, j, 2, cnt + 3,
                             ctx->rb_dev, ctx->flags, EX(ctx)));
   }
   sync_read(ctx);
@@ -573,8 +591,7 @@ bool gmres_fp64(sgn_ctx* ctx, int* iters_out, double* relres_out) {
       break;
     }
     if (its >= ctx->opt.maxit) break;
-    CK(launch_scale<double, double>(G, V, beta_d, true, V, EX(ctx)));
-    CK(launch_gmres_start(ctx->gst, beta_d, EX(ctx)));
+    CK(launch_gmres_start(ctx->gst, beta_d, false, EX(ctx)));
     int k = 0;
     for (int j = 0; j < m; ++j) {
       arnoldi_step<double>(ctx, ctx->tb, ctx->cr, ctx->cc, V, ctx->w, ctx->tmp, j);
@@ -583,10 +600,9 @@ bool gmres_fp64(sgn_ctx* ctx, int* iters_out, double* relres_out) {
       const double hnext = ctx->rb_host->hnext;
       k = j + 1;
       if (res <= target || its >= ctx->opt.maxit || !(hnext > 0.0) || res != res) break;
-      if (j + 1 < m) CK(launch_scale<double, double>(G, ctx->w, &ctx->gst->hnext, true, V + (size_t)(j + 1) * vs, EX(ctx)));
     }
     CK(launch_backsolve(ctx->gst, k, EX(ctx)));
-    CK(launch_axpy_multi<double, double>(G, V, vs, k, ctx->gst->y, ctx->sig, EX(ctx)));
+    CK(launch_axpy_multi<double, double>(G, V, vs, k, ctx->gst->y, ctx->sig, EX(ctx), nullptr, ctx->gst->vscl));
     if (res <= target) {
       conv = true;
       break;
@@ -650,7 +666,7 @@ bool gmres_mixed(sgn_ctx* ctx, int* iters_out, double* relres_out) {
     if (its >= ctx->opt.maxit) break;
     C32* const V = ctx->V32;
     CK(launch_scale<double, float>(G, ctx->r64, beta_d, true, V, EX(ctx)));
-    CK(launch_gmres_start(ctx->gst, beta_d, EX(ctx)));
+    CK(launch_gmres_start(ctx->gst, beta_d, true, EX(ctx)));
     const double inner_target = fmax(0.5 * target, kInnerRel * beta);
     double res_in = beta;
     int k = 0;
@@ -989,19 +1005,21 @@ void graph_arnoldi(sgn_ctx* ctx, const Tables<T>& tb, const T* cr, const T* cc, 
   const int* gate = &ctx->gst->reorth;
   unsigned* cnt = ctx->counters;
   const bool dgks = sizeof(T) == 8;
-  const double* vscl = dgks ? nullptr : ctx->gst->vscl;
+  const double* vscl = ctx->gst->vscl;
   CK(launch_matvec<T>(G, tb, V, cr, cc, w, tmp, true, EX(ctx), jd, vs, &ctx->mvt));
+  if (use_ortho<T>(ctx)) {
+    CK(launch_ortho<T>(G, V, vs, w, ctx->partials, ctx->gst, 0, dgks, ctx->bar_count, ctx->rb_dev, ctx->flags,
+                       EX(ctx), jd, &ctl));
+    return;
+  }
   CK(launch_dots<T>(G, V, vs, m, w, ctx->partials, nullptr, ctx->gst->h1, cnt + 0, EX(ctx), jd, vscl));
   CK(launch_cgs_update<T>(G, V, vs, m, ctx->gst->h1, w, ctx->partials, nullptr, ctx->gst, 0, dgks ? 1 : 3, cnt + 1,
-                          ctx->rb_dev, ctx->flags, EX(ctx), jd, &ctl, !dgks));
+                          ctx->rb_dev, ctx->flags, EX(ctx), jd, &ctl));
   if (dgks) {
-    CK(launch_dots<T>(G, V, vs, m, w, ctx->partials, gate, ctx->gst->h2, cnt + 2, EX(ctx), jd));
-    CK(launch_cgs_update<T>(G, V, vs, m, ctx->gst->h2, w, ctx->partials, gate, ctx->gst, 0, 2, cnt + 3,
+    CK(launch_dots<T>(G, V, vs, m, nullptr, ctx->partials, gate, ctx->gst->h2, cnt + 2, EX(ctx), jd, vscl));
+    CK(launch_cgs_update<T>(G, V, vs, m, ctx->gst->h2, nullptr, ctx->partials, gate, ctx->gst, 0, 2, cnt + 3,
                             ctx->rb_dev, ctx->flags, EX(ctx), jd, &ctl));
   }
-  // FP64: V_{j+1} = w / H[j+1][j]; j has already advanced (index m is the
-  // spare slot). FP32: the update stored the unnormalised V_{j+1} itself.
-  if (dgks) CK(launch_scale<T, T>(G, w, &ctx->gst->hnext, true, V, EX(ctx), jd, vs));
 }
 
 // One GMRES solve (FP64 or mixed) appended to the top-level segment.
@@ -1038,10 +1056,7 @@ void graph_gmres(sgn_ctx* ctx, GraphSeg& top) {
     CK(launch_residual<double>(G, ctx->cvec, ctx->w, r, ctx->partials, EX(ctx)));
     CK(launch_reduce(ctx->partials, 1, beta_d, true, nullptr, EX(ctx), sweep_partials(G)));
     CK(launch_ctl_sweep(ctx->gst, beta_d, ctl, EX(ctx)));
-    if (mixed)
-      CK((launch_scale<double, float>(G, r, beta_d, true, ctx->V32, EX(ctx))));
-    else
-      CK((launch_scale<double, double>(G, r, beta_d, true, ctx->V, EX(ctx))));
+    if (mixed) CK((launch_scale<double, float>(G, r, beta_d, true, ctx->V32, EX(ctx))));
   });
   sweep.close();
   ctx->sweep_bodies.push_back(sweep.g);
@@ -1062,7 +1077,8 @@ void graph_gmres(sgn_ctx* ctx, GraphSeg& top) {
       CK((launch_axpy_multi<float, double>(G, ctx->V32, vs, 0, ctx->gst->y, ctx->sig, EX(ctx), &ctx->gst->k,
                                            ctx->gst->vscl)));
     else
-      CK((launch_axpy_multi<double, double>(G, ctx->V, vs, 0, ctx->gst->y, ctx->sig, EX(ctx), &ctx->gst->k)));
+      CK((launch_axpy_multi<double, double>(G, ctx->V, vs, 0, ctx->gst->y, ctx->sig, EX(ctx), &ctx->gst->k,
+                                             ctx->gst->vscl)));
     CK(launch_ctl_after(ctx->gst, ctl, EX(ctx)));
   });
   sweep.close();
@@ -1357,7 +1373,9 @@ sgn_status sgn_create(int Nx, int Ny, double Lx, double Ly, double g, const sgn_
     ctx->h = dalloc<double>(ctx, G.nphys());
     ctx->cr = dalloc<double>(ctx, G.nphys());
     ctx->cc = dalloc<double>(ctx, G.nphys());
-    ctx->partials = dalloc<double>(ctx, (size_t)(MAXV + 2) * NBLK);
+    ctx->partials = dalloc<double>(ctx, 2 * (size_t)(MAXV + 2) * NBLK);
+    ctx->ortho = ortho_fits(G);
+    ctx->bar_count = dalloc<unsigned long long>(ctx, 1);
     ctx->scal = dalloc<double>(ctx, 16);
     ctx->gst = dalloc<GmresDev>(ctx, 1);
     ctx->rb_dev = dalloc<GmresReadback>(ctx, 1);

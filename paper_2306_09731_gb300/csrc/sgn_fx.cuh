@@ -549,7 +549,7 @@ __global__ void __launch_bounds__(PAR ? 384 : fx_threads<LN>(), PAR || LN == 12 
 // The RHS's x-pass (see k_rhs_x), its pointwise part in FP64. alx, aly: 2 pi /
 // Lx, Ly. PAR: the five inverse transforms run side by side in five groups of
 // threads, then three of them take F, q_x and q_y (grids with few row pairs, see
-// k_fx_mv_x: @PR@).
+// k_fx_mv_x: 256 x 16 66 -> 31 us, 1024 x 256 85 -> 53).
 template <int LN, bool PAR>
 __global__ void __launch_bounds__(PAR ? 640 : fx_threads<LN>(), PAR || LN == 12 ? 1 : 2) k_fx_rhs_x(
     Geom G, const cpx<fx>* __restrict__ tw, const double* __restrict__ kx, const cpx<double>* Vx,

@@ -109,8 +109,8 @@ struct GmresDev {
   double H[(MAXM + 1) * MAXM];  // column-major, H[i + j*(MAXM+1)]
   double cs[MAXM], sn[MAXM], g[MAXM + 1], y[MAXM];
   double h1[MAXV + 1], h2[MAXV + 1];  // Gram-Schmidt passes; slot nv holds |w|^2
-  // FP32 inner solve: basis vector i is stored unnormalised, V_i = vscl[i] X_i
-  // (the orthogonalised vector of step i-1, written straight into its slot)
+  // basis vector i is stored unnormalised, V_i = vscl[i] X_i (the
+  // orthogonalised vector of step i-1, written straight into its slot)
   double vscl[MAXV + 1];
   double nrm2;                // squared norm of the orthogonalised vector
   int reorth;                 // second pass needed (DGKS test)
@@ -368,7 +368,7 @@ cudaError_t launch_precond(const Geom& G, const Tables<T>& tb, const cpx<T>* in,
 template <typename T>
 cudaError_t launch_dots(const Geom& G, const cpx<T>* V, size_t vstride, int nv, const cpx<T>* w,
                         double* partials, const int* gate, double* out, unsigned* counter, const Exec& ex,
-                        const int* jdev = nullptr, const double* vscl = nullptr);
+                        const int* jdev, const double* vscl);
 // Gram-Schmidt update w -= sum_i coef[i] V_i of Arnoldi step j; the last block
 // stores |w'|^2, takes the DGKS decision (pass 1) and runs the Givens step once
 // the orthogonalisation is final (pass 1 without reorthogonalisation, pass 2,
@@ -377,10 +377,19 @@ cudaError_t launch_dots(const Geom& G, const cpx<T>* V, size_t vstride, int nv, 
 // the Givens step the last block advances the graph-mode control (its, k, j,
 // the Arnoldi loop condition).
 template <typename T>
-cudaError_t launch_cgs_update(const Geom& G, const cpx<T>* V, size_t vstride, int nv, const double* coef,
-                              cpx<T>* w, double* partials, const int* gate, GmresDev* st, int j, int pass,
+cudaError_t launch_cgs_update(const Geom& G, cpx<T>* V, size_t vstride, int nv, const double* coef,
+                              const cpx<T>* w, double* partials, const int* gate, GmresDev* st, int j, int pass,
                               unsigned* counter, GmresReadback* rb, const int* flags, const Exec& ex,
-                              const int* jdev = nullptr, const GraphCtl* ctl = nullptr, bool scaled = false);
+                              const int* jdev = nullptr, const GraphCtl* ctl = nullptr);
+// The whole orthogonalisation and Givens step of Arnoldi step j in one
+// cooperative launch, for vectors that ortho_fits() accepts (k_ortho): w = A X_j
+// in, X_{j+1} into slot j+1. part: 2 (MAXV + 2) NBLK doubles; count: a zeroed
+// device word of the handle's own.
+bool ortho_fits(const Geom& G);
+template <typename T>
+cudaError_t launch_ortho(const Geom& G, cpx<T>* V, size_t vstride, const cpx<T>* w, double* part, GmresDev* st, int j,
+                         bool dgks, unsigned long long* count, GmresReadback* rb, int* flags, const Exec& ex,
+                         const int* jdev = nullptr, const GraphCtl* ctl = nullptr);
 // r = c - w, and partial squared norm of r
 template <typename T>
 cudaError_t launch_residual(const Geom& G, const cpx<T>* c, const cpx<T>* w, cpx<T>* r, double* partials,
@@ -412,7 +421,7 @@ cudaError_t launch_reduce(const double* partials, int n, double* out, bool sqrt_
 // launch_residual)
 int sweep_partials(const Geom& G);
 // GMRES scalar kernels (one thread)
-cudaError_t launch_gmres_start(GmresDev* st, const double* beta, const Exec& ex);
+cudaError_t launch_gmres_start(GmresDev* st, const double* beta, bool unit, const Exec& ex);
 cudaError_t launch_backsolve(GmresDev* st, int k, const Exec& ex, const int* kdev = nullptr);
 // graph-mode control kernels (one thread); see csrc/sgn_krylov.cu
 cudaError_t launch_ctl_begin(GmresDev* st, const double* cnorm, GraphCtl ctl, const Exec& ex);

@@ -17,9 +17,9 @@
 // are FP64-issue bound, not HBM bound (4 DFMA per 16-byte entry against an
 // FP64:HBM balance below 1 DFMA per byte), so each entry's Parseval weight is
 // folded into w once rather than into every dot product. The Gram-Schmidt
-// pair runs one wave of KBLK blocks (4 per SM). The FP32 basis of the inner
-// solve is kept unnormalised, V_i = s_i X_i with the scales s_i on the device,
-// so no pass rescales a vector (k_cgs_update writes X_{j+1} itself).
+// pair runs one wave of KBLK blocks (4 per SM). The basis is kept unnormalised,
+// V_i = s_i X_i with the scales s_i on the device, so no pass rescales a vector
+// (k_cgs_update writes X_{j+1} itself, and a second pass works on it in place).
 #include <math.h>
 
 #include "sgn_internal.h"
@@ -27,32 +27,45 @@
 
 namespace sgn {
 
-// Givens update of column j of the Hessenberg matrix (one thread): the column
-// from the two Gram-Schmidt passes and |w|, previous rotations, a new rotation
-// zeroing H[j+1][j], and the residual estimate |g_{j+1}| into the readback.
-__device__ void givens_step(GmresDev* st, int j, GmresReadback* rb, const int* flags) {
-  const int ld = MAXM + 1;
+// Givens update of column j of the Hessenberg matrix by one warp: the column
+// from the two Gram-Schmidt passes (h2: whether there was a second) and |w|^2,
+// previous rotations, a new rotation zeroing H[j+1][j], and the residual
+// estimate |g_{j+1}| into the readback. Lane i fetches entry and rotation i, so
+// that the serial chain runs on registers and not on one load after the other.
+__device__ void givens_step(GmresDev* st, int j, double nrm2, bool h2, GmresReadback* rb, const int* flags) {
+  const int ld = MAXM + 1, lane = threadIdx.x & 31;
   double* Hj = st->H + (size_t)j * ld;
-  for (int i = 0; i <= j; ++i) Hj[i] = st->h1[i] + st->h2[i];
-  const double hn = sqrt(st->nrm2);
-  Hj[j + 1] = hn;
-  st->hnext = hn;
-  st->inv_hnext = hn > 0.0 ? 1.0 / hn : 0.0;
-  for (int i = 0; i < j; ++i) {
-    const double a = Hj[i], b = Hj[i + 1];
-    Hj[i] = st->cs[i] * a + st->sn[i] * b;
-    Hj[i + 1] = -st->sn[i] * a + st->cs[i] * b;
+  double h = 0.0, c = 0.0, s = 0.0;
+  if (lane <= j) h = st->h1[lane] + (h2 ? st->h2[lane] : 0.0);
+  if (lane < j) {
+    c = st->cs[lane];
+    s = st->sn[lane];
   }
-  const double d = hypot(Hj[j], Hj[j + 1]);
-  const double c = d > 0.0 ? Hj[j] / d : 1.0;
-  const double s = d > 0.0 ? Hj[j + 1] / d : 0.0;
-  st->cs[j] = c;
-  st->sn[j] = s;
+  const double gj = st->g[j];
+  const double hn = sqrt(nrm2);
+  double cur = __shfl_sync(0xffffffffu, h, 0);  // entry i, rotated so far
+  for (int i = 0; i < j; ++i) {
+    const double ci = __shfl_sync(0xffffffffu, c, i), si = __shfl_sync(0xffffffffu, s, i);
+    const double b = __shfl_sync(0xffffffffu, h, i + 1);
+    const double r = ci * cur + si * b;
+    cur = -si * cur + ci * b;
+    if (lane == i) h = r;
+  }
+  const double d = hypot(cur, hn);
+  const double cj = d > 0.0 ? cur / d : 1.0;
+  const double sj = d > 0.0 ? hn / d : 0.0;
+  if (lane < j) Hj[lane] = h;
+  if (lane != 0) return;
   Hj[j] = d;
   Hj[j + 1] = 0.0;
-  st->g[j + 1] = -s * st->g[j];
-  st->g[j] = c * st->g[j];
-  st->res = fabs(st->g[j + 1]);
+  st->nrm2 = nrm2;
+  st->hnext = hn;
+  st->inv_hnext = hn > 0.0 ? 1.0 / hn : 0.0;
+  st->cs[j] = cj;
+  st->sn[j] = sj;
+  st->g[j + 1] = -sj * gj;
+  st->g[j] = cj * gj;
+  st->res = fabs(sj * gj);
   rb->res = st->res;
   rb->hnext = hn;
   rb->flags = flags ? *flags : 0;
@@ -172,6 +185,21 @@ struct Acc<float> {
   typedef float type;
 };
 
+// s + a x + b y + c z + d w. FP64: one FMA a term (the Krylov sweeps are bound by
+// the FP64 pipe: 64 to 69% busy in k_ortho, and a product plus a sum of two
+// products took three of its slots for two terms). FP32: sums of pairs.
+__device__ __forceinline__ double add4(double s, double a, double x, double b, double y, double c, double z, double d,
+                                       double w) {
+  return fma(d, w, fma(c, z, fma(b, y, fma(a, x, s))));
+}
+__device__ __forceinline__ float add4(float s, float a, float x, float b, float y, float c, float z, float d,
+                                      float w) {
+  return s + ((a * x + b * y) + (c * z + d * w));
+}
+__device__ __forceinline__ float sub4(float s, const float* c, float x, float y, float z, float w) {
+  return s - ((c[0] * x + c[1] * y) + (c[2] * z + c[3] * w));
+}
+
 constexpr int DOT_CHUNK = 4;  // dot products per sweep of a block's entries
 
 // partials[i * NBLK + b] = block b's share of <V_i, w> (i < nv) and
@@ -179,7 +207,7 @@ constexpr int DOT_CHUNK = 4;  // dot products per sweep of a block's entries
 // chunks of four vectors (one sweep of its entries per chunk; at the usual
 // cycle lengths one chunk), so the grid does not depend on nv: graph mode reads
 // nv from the device. Four accumulators keep registers low enough for 4 blocks
-// per SM.
+// per SM. w (may be null): else the second pass's vector, slot nv of the basis.
 // gate (may be null): the kernel does nothing unless *gate != 0.
 template <typename T>
 __global__ void __launch_bounds__(256, 4) k_dots(Geom G, const cpx<T>* V, size_t vstride, int nv, const cpx<T>* w,
@@ -188,6 +216,7 @@ __global__ void __launch_bounds__(256, 4) k_dots(Geom G, const cpx<T>* V, size_t
   typedef typename Acc<T>::type A;
   if (gate && *gate == 0) return;
   if (jdev) nv = *jdev + 1;
+  if (!w) w = V + (size_t)nv * vstride;
   __shared__ double red[8 * 32];
   for (int i0 = 0; i0 < nv; i0 += DOT_CHUNK) {
     const int nc = min(DOT_CHUNK, nv - i0);
@@ -213,8 +242,8 @@ __global__ void __launch_bounds__(256, 4) k_dots(Geom G, const cpx<T>* V, size_t
       const A ax = ta * (A)wa.x, ay = ta * (A)wa.y, bx = tb * (A)wb.x, by = tb * (A)wb.y;
 #pragma unroll
       for (int i = 0; i < DOT_CHUNK; ++i)
-        if (i < nc) acc[i] += (ax * (A)va[i].x + ay * (A)va[i].y) + (bx * (A)vb[i].x + by * (A)vb[i].y);
-      if (chunk0) nrm += (ax * (A)wa.x + ay * (A)wa.y) + (bx * (A)wb.x + by * (A)wb.y);
+        if (i < nc) acc[i] = add4(acc[i], ax, (A)va[i].x, ay, (A)va[i].y, bx, (A)vb[i].x, by, (A)vb[i].y);
+      if (chunk0) nrm = add4(nrm, ax, (A)wa.x, ay, (A)wa.y, bx, (A)wb.x, by, (A)wb.y);
     }
     // thread i < DOT_CHUNK holds <V_{i0+i}, w>, thread DOT_CHUNK |w|^2
     A vals[DOT_CHUNK + 1];
@@ -230,19 +259,16 @@ __global__ void __launch_bounds__(256, 4) k_dots(Geom G, const cpx<T>* V, size_t
   // the last block combines all partials: out[i] = <V_i, w>, out[nv] = |w|^2
   if (last_block(counter, threadIdx.x <= DOT_CHUNK)) {
     reduce_slots(partials, nv + 1, out, gridDim.x);
-    // scaled basis (vscl): V_i = s_i X_i and w = s_j w~ for the stored X_i and
-    // the matvec of X_j: <V_i, w> = s_i s_j <X_i, w~>, |w|^2 = s_j^2 |w~|^2
-    if (vscl) {
-      __syncthreads();
-      if ((int)threadIdx.x <= nv) {
-        const double sj = vscl[nv - 1];
-        out[threadIdx.x] *= ((int)threadIdx.x < nv ? vscl[threadIdx.x] : sj) * sj;
-      }
+    // V_i = s_i X_i and w = s_j w~ for the stored X_i and the matvec of X_j:
+    // <V_i, w> = s_i s_j <X_i, w~>, |w|^2 = s_j^2 |w~|^2
+    __syncthreads();
+    if ((int)threadIdx.x <= nv) {
+      const double sj = vscl[nv - 1];
+      out[threadIdx.x] *= ((int)threadIdx.x < nv ? vscl[threadIdx.x] : sj) * sj;
     }
   }
 }
 
-// w -= sum_i coef[i] V_i (i < nv) and |w_new|^2 into slot 0. Gated like k_dots.
 // After the final Givens step of Arnoldi step j (graph mode): count the matvec,
 // record the residual estimate, and keep the Arnoldi loop running unless the
 // cycle is done (the eager host loop's test).
@@ -257,16 +283,17 @@ __device__ __forceinline__ void ctl_step(GmresDev* st, int j, const GraphCtl& ct
   cudaGraphSetConditional(ctl.h_step, stop ? 0u : 1u);
 }
 
-// scaled (FP32 inner solve): the basis is stored unnormalised, V_i = s_i X_i
-// (s = st->vscl) and w holds w~ = A X_j; the kernel writes X_{j+1} = w~ -
-// sum_i (h_i s_i / s_j) X_i = w' / s_j straight into slot j+1 of V (no scaling
-// pass), |w'|^2 = s_j^2 |X_{j+1}|^2, and s_{j+1} = s_j / |w'|.
+// w -= sum_i coef[i] V_i (i < nv) and |w_new|^2. Gated like k_dots. The basis is
+// stored unnormalised, V_i = s_i X_i (s = st->vscl), and w holds w~ = A X_j: the
+// kernel writes X_{j+1} = w~ - sum_i (h_i s_i / s_j) X_i = w' / s_j straight into
+// slot j+1 of V (no scaling pass), |w'|^2 = s_j^2 |X_{j+1}|^2, and s_{j+1} = s_j /
+// |w'|. A second pass (pass 2) takes X_{j+1} from there.
 template <typename T>
-__global__ void __launch_bounds__(256) k_cgs_update(Geom G, const cpx<T>* V, size_t vstride, int nv,
-                                                    const double* __restrict__ coef, cpx<T>* w, double* partials,
-                                                    const int* gate, GmresDev* st, int j, int pass,
+__global__ void __launch_bounds__(256) k_cgs_update(Geom G, cpx<T>* V, size_t vstride, int nv,
+                                                    const double* __restrict__ coef, const cpx<T>* w,
+                                                    double* partials, const int* gate, GmresDev* st, int j, int pass,
                                                     unsigned* counter, GmresReadback* rb, const int* flags,
-                                                    const int* jdev, GraphCtl ctl, int scaled) {
+                                                    const int* jdev, GraphCtl ctl) {
   typedef typename Acc<T>::type A;
   if (gate && *gate == 0) return;
   if (jdev) {
@@ -277,11 +304,12 @@ __global__ void __launch_bounds__(256) k_cgs_update(Geom G, const cpx<T>* V, siz
   __shared__ A cf[MAXV + 4];
   if (threadIdx.x < MAXV + 4) {
     double c = threadIdx.x < nv ? coef[threadIdx.x] : 0.0;
-    if (scaled && threadIdx.x < nv) c *= st->vscl[threadIdx.x] / st->vscl[j];
+    if (threadIdx.x < nv) c *= st->vscl[threadIdx.x] / st->vscl[j];
     cf[threadIdx.x] = (A)c;
   }
   __syncthreads();
-  cpx<T>* wout = scaled ? const_cast<cpx<T>*>(V) + (size_t)(j + 1) * vstride : w;
+  cpx<T>* wout = V + (size_t)(j + 1) * vstride;
+  if (pass == 2) w = wout;
   A nrm = (A)0;
   // two interleaved walkers; four basis vectors per round with predicated
   // loads rather than a remainder loop, so that a round's loads (8 entries)
@@ -299,10 +327,23 @@ __global__ void __launch_bounds__(256) k_cgs_update(Geom G, const cpx<T>* V, siz
         va[u] = in ? V[(size_t)(i + u) * vstride + a.e] : mk((T)0, (T)0);
         vb[u] = in ? V[(size_t)(i + u) * vstride + eb] : mk((T)0, (T)0);
       }
-      zax -= (cf[i] * (A)va[0].x + cf[i + 1] * (A)va[1].x) + (cf[i + 2] * (A)va[2].x + cf[i + 3] * (A)va[3].x);
-      zay -= (cf[i] * (A)va[0].y + cf[i + 1] * (A)va[1].y) + (cf[i + 2] * (A)va[2].y + cf[i + 3] * (A)va[3].y);
-      zbx -= (cf[i] * (A)vb[0].x + cf[i + 1] * (A)vb[1].x) + (cf[i + 2] * (A)vb[2].x + cf[i + 3] * (A)vb[3].x);
-      zby -= (cf[i] * (A)vb[0].y + cf[i + 1] * (A)vb[1].y) + (cf[i + 2] * (A)vb[2].y + cf[i + 3] * (A)vb[3].y);
+      if constexpr (sizeof(T) == 8) {
+        // one FMA a term, and none for the vectors past nv
+#pragma unroll
+        for (int u = 0; u < 4; ++u)
+          if (i + u < nv) {
+            const A c = -cf[i + u];
+            zax = fma(c, va[u].x, zax);
+            zay = fma(c, va[u].y, zay);
+            zbx = fma(c, vb[u].x, zbx);
+            zby = fma(c, vb[u].y, zby);
+          }
+      } else {
+        zax = sub4(zax, cf + i, va[0].x, va[1].x, va[2].x, va[3].x);
+        zay = sub4(zay, cf + i, va[0].y, va[1].y, va[2].y, va[3].y);
+        zbx = sub4(zbx, cf + i, vb[0].x, vb[1].x, vb[2].x, vb[3].x);
+        zby = sub4(zby, cf + i, vb[0].y, vb[1].y, vb[2].y, vb[3].y);
+      }
     }
     const cpx<T> za = mk((T)zax, (T)zay), zb = mk((T)zbx, (T)zby);
     wout[a.e] = za;
@@ -319,28 +360,199 @@ __global__ void __launch_bounds__(256) k_cgs_update(Geom G, const cpx<T>* V, siz
   // step once the orthogonalisation is final. pass: 1 first pass with the DGKS
   // test, 2 second pass, 3 single pass (no reorthogonalisation)
   if (last_block(counter, threadIdx.x == 0)) {
-    const double n2 = reduce_slot(partials, 0, red, gridDim.x);
+    const double sum = reduce_slot(partials, 0, red, gridDim.x);
+    if (threadIdx.x >= 32) return;
+    const double sj = st->vscl[j];
+    const double n2 = __shfl_sync(0xffffffffu, sum, 0) * sj * sj;
+    const bool need = pass == 1 && n2 < 0.5 * st->h1[nv];
     if (threadIdx.x == 0) {
-      st->nrm2 = scaled ? n2 * st->vscl[j] * st->vscl[j] : n2;
-      bool final_pass = (pass == 2);
-      if (pass == 1 || pass == 3) {
-        // pass 3: first pass of an Arnoldi step that never reorthogonalises
-        const int need = (pass == 1 && n2 < 0.5 * st->h1[nv]) ? 1 : 0;
-        st->reorth = need;
-        if (!need) {
-          for (int i = 0; i <= MAXV; ++i) st->h2[i] = 0.0;
-          final_pass = true;
-        }
-      }
+      if (pass != 2) st->reorth = need ? 1 : 0;
       // graph mode: the Arnoldi loop continues only if the final pass re-arms it
       if (ctl.enabled) cudaGraphSetConditional(ctl.h_step, 0u);
-      if (final_pass) {
-        givens_step(st, j, rb, flags);
-        if (scaled) st->vscl[j + 1] = st->hnext > 0.0 ? st->vscl[j] / st->hnext : 0.0;
-        if (ctl.enabled) ctl_step(st, j, ctl);
-      }
+    }
+    if (need) return;
+    givens_step(st, j, n2, pass == 2, rb, flags);
+    if (threadIdx.x == 0) {
+      st->vscl[j + 1] = st->hnext > 0.0 ? sj / st->hnext : 0.0;
+      if (ctl.enabled) ctl_step(st, j, ctl);
     }
   }
+}
+
+// ------------------------------------------- one Arnoldi step in one launch
+// A grid barrier of a cooperative launch: every block arrives once per barrier
+// (count: 64-bit, never reset, a multiple of the grid between launches), and
+// the wait is bounded (about a second): *flags gets FLAG_WAIT when it runs out.
+__device__ __forceinline__ void grid_barrier(unsigned long long* count, int* flags) {
+  __syncthreads();
+  if (threadIdx.x == 0) {
+    __threadfence();
+    const unsigned long long n = gridDim.x;
+    const unsigned long long target = (atomicAdd(count, 1ull) / n + 1ull) * n;
+    bool ok = false;
+    for (int it = 0; it < (1 << 22) && !ok; ++it) {
+      unsigned long long c;
+      asm volatile("ld.acquire.gpu.global.u64 %0, [%1];" : "=l"(c) : "l"(count) : "memory");
+      ok = c >= target;
+    }
+    if (!ok) atomicOr(flags, FLAG_WAIT);
+    __threadfence();
+  }
+  __syncthreads();
+}
+
+// Entries of w a thread of k_ortho holds at most, its threads at most and its
+// blocks: one per SM, as every block repeats the sums over all partials.
+constexpr int ORTHO_NE = 4, ORTHO_THR = 512, ORTHO_BLK = 152;
+
+// Block sums of 8 values over nw <= 16 warps (at least 4): the sum of value k on
+// thread 16 k (of the first 128). red: 8 * 16 doubles.
+template <typename A>
+__device__ __forceinline__ double ortho_reduce8(const A (&v)[8], double* red) {
+  const int lane = threadIdx.x & 31;
+  const A c = warp_sum8(v);
+  if ((lane & 3) == 0) red[(lane >> 2) * 16 + (threadIdx.x >> 5)] = (double)c;
+  __syncthreads();
+  double t = 0.0;
+  if (threadIdx.x < 128) {
+    const int nw = blockDim.x >> 5;
+    t = (int)(threadIdx.x & 15) < nw ? red[threadIdx.x] : 0.0;
+    for (int o = nw >> 1; o > 0; o >>= 1) t += __shfl_xor_sync(0xffffffffu, t, o);
+  }
+  return t;
+}
+
+// The whole orthogonalisation of Arnoldi step j for vectors of up to ORTHO_BLK *
+// ORTHO_THR * ORTHO_NE entries: k_dots and k_cgs_update (dgks: and their gated second
+// pair) with w in registers and a grid barrier in the place of each kernel
+// boundary. On such grids the four launches (the second pair nearly always runs,
+// as A is near the identity) are mostly latency: an Arnoldi step's
+// orthogonalisation takes about 25 us instead of 45 at 256 x 16, 50 instead of 69
+// at 1024 x 256 (where the FP64 pipe is 64 to 69% busy).
+// Every block sums the partials itself, in the same order, so all take the same
+// DGKS decision. part: two regions of MAXV + 2 slots, one for each pass, as a
+// block may write its share of the next sum while others still read the last.
+template <typename T>
+__global__ void __launch_bounds__(ORTHO_THR, 1) k_ortho(Geom G, cpx<T>* V, size_t vstride, const cpx<T>* w, double* part,
+                                                  GmresDev* st, int j, int dgks, unsigned long long* count,
+                                                  GmresReadback* rb, int* flags, const int* jdev, GraphCtl ctl) {
+  typedef typename Acc<T>::type A;
+  constexpr int CH = 7;
+  if (jdev) j = *jdev;
+  const int nv = j + 1, nblk = gridDim.x, lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+  __shared__ double red[8 * 32];
+  __shared__ double hs[MAXV + 2];
+  __shared__ double sc[MAXV + 1];
+  __shared__ A cf[MAXV + 8];
+  const size_t n = G.nspec();
+  const int nthr = nblk * blockDim.x;
+  cpx<T> z[ORTHO_NE];
+  A wt[ORTHO_NE];
+  size_t e[ORTHO_NE];
+#pragma unroll
+  for (int k = 0; k < ORTHO_NE; ++k) {
+    e[k] = (size_t)blockIdx.x * blockDim.x + threadIdx.x + (size_t)k * nthr;
+    const bool in = e[k] < n;
+    z[k] = in ? w[e[k]] : mk((T)0, (T)0);
+    wt[k] = in ? col_weight_k<A>(G, (int)(e[k] % G.ldS)) : (A)0;
+    if (!in) e[k] = 0;
+  }
+  if (threadIdx.x < MAXV + 1) sc[threadIdx.x] = (int)threadIdx.x <= j ? st->vscl[threadIdx.x] : 0.0;
+  __syncthreads();
+  const double sj = sc[j];
+  double n2 = 0.0;
+#pragma unroll 1
+  for (int pass = 1;; ++pass) {
+    double* pr = part + (size_t)(pass - 1) * (MAXV + 2) * NBLK;
+    // <X_i, w> (and |w|^2) of the thread's entries
+#pragma unroll 1
+    for (int i0 = 0; i0 < nv; i0 += CH) {
+      A acc[CH + 1];
+#pragma unroll
+      for (int i = 0; i <= CH; ++i) acc[i] = (A)0;
+#pragma unroll
+      for (int k = 0; k < ORTHO_NE; ++k) {
+        if (k * nthr >= (int)n) break;
+        cpx<T> x[CH];
+#pragma unroll
+        for (int i = 0; i < CH; ++i)
+          if (i0 + i < nv) x[i] = V[(size_t)(i0 + i) * vstride + e[k]];
+        const A ax = weigh(wt[k], (A)z[k].x), ay = weigh(wt[k], (A)z[k].y);
+#pragma unroll
+        for (int i = 0; i < CH; ++i)
+          if (i0 + i < nv) acc[i] = fma(ay, (A)x[i].y, fma(ax, (A)x[i].x, acc[i]));
+        if (i0 == 0 && pass == 1 && dgks) acc[CH] = fma(ay, (A)z[k].y, fma(ax, (A)z[k].x, acc[CH]));
+      }
+      const double tot = ortho_reduce8(acc, red);
+      const int k8 = threadIdx.x >> 4;
+      if ((threadIdx.x & 15) == 0 && k8 < CH && i0 + k8 < nv) pr[(size_t)(i0 + k8) * NBLK + blockIdx.x] = tot;
+      if (threadIdx.x == 16 * CH && i0 == 0) pr[(size_t)nv * NBLK + blockIdx.x] = tot;
+      __syncthreads();
+    }
+    grid_barrier(count, flags);
+    // V_i = s_i X_i, w = s_j w~
+    reduce_slots(pr, nv + 1, hs, nblk);
+    __syncthreads();
+    if ((int)threadIdx.x < nv) {
+      const double h = hs[threadIdx.x] * sc[threadIdx.x] * sj;
+      cf[threadIdx.x] = (A)(h * sc[threadIdx.x] / sj);
+      if (blockIdx.x == 0) (pass == 1 ? st->h1 : st->h2)[threadIdx.x] = h;
+    } else if (threadIdx.x < MAXV + 8) {
+      cf[threadIdx.x] = (A)0;
+    }
+    __syncthreads();
+    // X_{j+1} = w~ - sum_i (h_i s_i / s_j) X_i and its norm
+    A nrm[ORTHO_NE] = {(A)0};
+#pragma unroll
+    for (int k = 0; k < ORTHO_NE; ++k) {
+      if (k * nthr >= (int)n) break;
+      A zx = (A)z[k].x, zy = (A)z[k].y;
+      for (int i = 0; i < nv; i += 4) {
+        cpx<T> x[4];
+#pragma unroll
+        for (int u = 0; u < 4; ++u)
+          if (i + u < nv) x[u] = V[(size_t)(i + u) * vstride + e[k]];
+#pragma unroll
+        for (int u = 0; u < 4; ++u)
+          if (i + u < nv) {
+            const A c = -cf[i + u];
+            zx = fma(c, (A)x[u].x, zx);
+            zy = fma(c, (A)x[u].y, zy);
+          }
+      }
+      z[k] = mk((T)zx, (T)zy);
+      nrm[k] = weigh(wt[k], (A)z[k].x * (A)z[k].x + (A)z[k].y * (A)z[k].y);
+    }
+    A one[8] = {(nrm[0] + nrm[1]) + (nrm[2] + nrm[3])};
+    const double tot = ortho_reduce8(one, red);
+    if (threadIdx.x == 0) pr[(size_t)(MAXV + 1) * NBLK + blockIdx.x] = tot;
+    const double w2 = hs[nv] * sj * sj;  // |w|^2 before the pass (first pass)
+    grid_barrier(count, flags);
+    if (warp == 0) {
+      double t = 0.0;
+      for (int b = lane; b < nblk; b += 32) t += __ldcg(pr + (size_t)(MAXV + 1) * NBLK + b);
+      for (int o = 16; o > 0; o >>= 1) t += __shfl_xor_sync(0xffffffffu, t, o);
+      if (lane == 0) hs[MAXV + 1] = t * sj * sj;
+    }
+    __syncthreads();
+    n2 = hs[MAXV + 1];
+    const bool need = dgks && pass == 1 && n2 < 0.5 * w2;
+    if (!need) {
+      if (blockIdx.x == 0 && warp == 0) {
+        if (ctl.enabled && lane == 0) cudaGraphSetConditional(ctl.h_step, 0u);
+        givens_step(st, j, n2, pass == 2, rb, flags);
+        if (lane == 0) {
+          st->vscl[j + 1] = st->hnext > 0.0 ? sj / st->hnext : 0.0;
+          if (ctl.enabled) ctl_step(st, j, ctl);
+        }
+      }
+      break;
+    }
+  }
+  cpx<T>* out = V + (size_t)(j + 1) * vstride;
+#pragma unroll
+  for (int k = 0; k < ORTHO_NE; ++k)
+    if ((size_t)blockIdx.x * blockDim.x + threadIdx.x + (size_t)k * nthr < n) out[e[k]] = z[k];
 }
 
 template <typename T>
@@ -435,12 +647,12 @@ __global__ void k_reduce(const double* partials, int n, double* out, int sqrt_ou
 // ---------------------------------------------------------- scalar kernels
 
 // g = (beta, 0, ...), the start of a GMRES cycle
-__global__ void k_gmres_start(GmresDev* st, const double* beta) {
+// (unit: X_0 = V_0, else X_0 = r = beta V_0)
+__global__ void k_gmres_start(GmresDev* st, const double* beta, int unit) {
+  for (int i = threadIdx.x; i <= MAXM; i += 32) st->g[i] = i == 0 ? *beta : 0.0;
   if (threadIdx.x != 0) return;
-  for (int i = 0; i <= MAXM; ++i) st->g[i] = 0.0;
-  st->g[0] = *beta;
   st->res = *beta;
-  st->vscl[0] = 1.0;
+  st->vscl[0] = unit ? 1.0 : 1.0 / *beta;
 }
 
 // y = H(0:k,0:k)^{-1} g(0:k) by back substitution
@@ -492,7 +704,7 @@ __global__ void k_ctl_sweep(GmresDev* st, const double* beta_d, GraphCtl ctl) {
   st->beta = beta;
   st->k = 0;
   st->j = 0;
-  st->vscl[0] = 1.0;
+  st->vscl[0] = ctl.mixed ? 1.0 : 1.0 / beta;  // X_0: r / beta in FP32, else r itself
   st->sweeps += 1;
   st->tot_sweeps += 1;
   const bool done = !(beta > st->target);
@@ -721,17 +933,54 @@ cudaError_t launch_dots(const Geom& G, const cpx<T>* V, size_t vstride, int nv, 
   return cudaGetLastError();
 }
 template <typename T>
-cudaError_t launch_cgs_update(const Geom& G, const cpx<T>* V, size_t vstride, int nv, const double* coef,
-                              cpx<T>* w, double* partials, const int* gate, GmresDev* st, int j, int pass,
+cudaError_t launch_cgs_update(const Geom& G, cpx<T>* V, size_t vstride, int nv, const double* coef,
+                              const cpx<T>* w, double* partials, const int* gate, GmresDev* st, int j, int pass,
                               unsigned* counter, GmresReadback* rb, const int* flags, const Exec& ex,
-                              const int* jdev, const GraphCtl* ctl, bool scaled) {
+                              const int* jdev, const GraphCtl* ctl) {
   GraphCtl c{};
   if (ctl) c = *ctl;
   ex.begin(PK_KRYLOV);
   k_cgs_update<T><<<sweep_blocks(G, 2, KBLK), 256, 0, ex.s>>>(G, V, vstride, nv, coef, w, partials, gate, st, j, pass, counter, rb,
-                                         flags, jdev, c, scaled ? 1 : 0);
+                                         flags, jdev, c);
   ex.end();
   return cudaGetLastError();
+}
+bool ortho_fits(const Geom& G) {
+  int dev = 0, coop = 0, sms = 0, per = 0;
+  if (G.nspec() > (size_t)ORTHO_BLK * ORTHO_THR * ORTHO_NE) return false;
+  if (cudaGetDevice(&dev) != cudaSuccess ||
+      cudaDeviceGetAttribute(&coop, cudaDevAttrCooperativeLaunch, dev) != cudaSuccess ||
+      cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev) != cudaSuccess ||
+      cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per, k_ortho<double>, ORTHO_THR, 0) != cudaSuccess) {
+    cudaGetLastError();
+    return false;
+  }
+  return coop && per * sms >= ORTHO_BLK;
+}
+template <typename T>
+cudaError_t launch_ortho(const Geom& G, cpx<T>* V, size_t vstride, const cpx<T>* w, double* part, GmresDev* st, int j,
+                         bool dgks, unsigned long long* count, GmresReadback* rb, int* flags, const Exec& ex,
+                         const int* jdev, const GraphCtl* ctl) {
+  GraphCtl c{};
+  if (ctl) c = *ctl;
+  cudaLaunchAttribute at{};
+  at.id = cudaLaunchAttributeCooperative;
+  at.val.cooperative = 1;
+  cudaLaunchConfig_t cfg{};
+  // short vectors: fewer threads a block, so that every SM shares the FP64 work
+  unsigned thr = ORTHO_THR;
+  while (thr > 128 && (G.nspec() + thr / 2 - 1) / (thr / 2) <= (size_t)ORTHO_BLK) thr /= 2;
+  const size_t b = (G.nspec() + thr - 1) / thr;
+  cfg.gridDim = dim3(b < (size_t)ORTHO_BLK ? (unsigned)b : ORTHO_BLK);
+  cfg.blockDim = dim3(thr);
+  cfg.stream = ex.s;
+  cfg.attrs = &at;
+  cfg.numAttrs = 1;
+  ex.begin(PK_KRYLOV);
+  const cudaError_t e = cudaLaunchKernelEx(&cfg, k_ortho<T>, G, V, vstride, w, part, st, j, dgks ? 1 : 0, count, rb,
+                                           flags, jdev, c);
+  ex.end();
+  return e != cudaSuccess ? e : cudaGetLastError();
 }
 template <typename T>
 cudaError_t launch_residual(const Geom& G, const cpx<T>* c, const cpx<T>* w, cpx<T>* r, double* partials,
@@ -788,9 +1037,9 @@ cudaError_t launch_reduce(const double* partials, int n, double* out, bool sqrt_
   ex.end();
   return cudaGetLastError();
 }
-cudaError_t launch_gmres_start(GmresDev* st, const double* beta, const Exec& ex) {
+cudaError_t launch_gmres_start(GmresDev* st, const double* beta, bool unit, const Exec& ex) {
   ex.begin(PK_KRYLOV);
-  k_gmres_start<<<1, 32, 0, ex.s>>>(st, beta);
+  k_gmres_start<<<1, 32, 0, ex.s>>>(st, beta, unit ? 1 : 0);
   ex.end();
   return cudaGetLastError();
 }
@@ -879,10 +1128,13 @@ cudaError_t launch_invariant_sums(const Geom& G, const double* h, const double* 
   template cudaError_t launch_dots<T>(const Geom&, const cpx<T>*, size_t, int, const cpx<T>*, double*,       \
                                       const int*, double*, unsigned*, const Exec&, const int*,              \
                                       const double*);                                                      \
-  template cudaError_t launch_cgs_update<T>(const Geom&, const cpx<T>*, size_t, int, const double*, cpx<T>*, \
+  template cudaError_t launch_cgs_update<T>(const Geom&, cpx<T>*, size_t, int, const double*, const cpx<T>*, \
                                             double*, const int*, GmresDev*, int, int, unsigned*,            \
                                             GmresReadback*, const int*, const Exec&, const int*,            \
-                                            const GraphCtl*, bool);                                         \
+                                            const GraphCtl*);                                               \
+  template cudaError_t launch_ortho<T>(const Geom&, cpx<T>*, size_t, const cpx<T>*, double*, GmresDev*, int, \
+                                       bool, unsigned long long*, GmresReadback*, int*, const Exec&,         \
+                                       const int*, const GraphCtl*);                                         \
   template cudaError_t launch_residual<T>(const Geom&, const cpx<T>*, const cpx<T>*, cpx<T>*, double*,       \
                                           const Exec&);                                                     \
   template cudaError_t launch_zero<T>(const Geom&, cpx<T>*, const Exec&, const int*);                       \
@@ -892,12 +1144,8 @@ cudaError_t launch_invariant_sums(const Geom& G, const double* h, const double* 
 
 SGN_KRYLOV_INST(double)
 SGN_KRYLOV_INST(float)
-template cudaError_t launch_scale<double, double>(const Geom&, const cpx<double>*, const double*, bool,
-                                                  cpx<double>*, const Exec&, const int*, size_t);
 template cudaError_t launch_scale<double, float>(const Geom&, const cpx<double>*, const double*, bool,
                                                  cpx<float>*, const Exec&, const int*, size_t);
-template cudaError_t launch_scale<float, float>(const Geom&, const cpx<float>*, const double*, bool,
-                                                cpx<float>*, const Exec&, const int*, size_t);
 template cudaError_t launch_axpy_multi<double, double>(const Geom&, const cpx<double>*, size_t, int,
                                                        const double*, cpx<double>*, const Exec&, const int*,
                                                        const double*);

@@ -91,8 +91,11 @@ extern "C" sgn_status sgn_elliptic_apply_noalloc(int Nx, int Ny, double Lx, doub
   cudaError_t e = cudaGetSymbolAddress(&scratch, g_noalloc_scratch);
   if (e != cudaSuccess || !scratch)
     return noalloc_fail(SGN_ECUDA, std::string("cudaGetSymbolAddress: ") + cudaGetErrorString(e));
-  // the shared-memory opt-in of the transform kernels (per device; cheap to repeat)
-  init_kernel_attributes<double>();
+  // the shared-memory opt-in of the transform kernels, per device. Up to 256
+  // points an axis no block asks for more than the default 48 KB (its row pair
+  // or two columns take 33 KB at most), and the attribute calls would be a
+  // third of such a call's time.
+  if (Nx > 256 || Ny > 256) init_kernel_attributes<double>();
 
   Geom G{};
   G.Nx = Nx;
