@@ -48,6 +48,15 @@ __device__ __forceinline__ cpx<T> mk(T a, T b) {
   r.y = b;
   return r;
 }
+// real and imaginary part (cpx<dfl> keeps its parts otherwise, see dfloat.cuh)
+template <typename T>
+__host__ __device__ __forceinline__ T re(cpx<T> a) { return a.x; }
+template <typename T>
+__host__ __device__ __forceinline__ T im(cpx<T> a) { return a.y; }
+// (a Re z, b Im z)
+template <typename T>
+__device__ __forceinline__ cpx<T> mul_xy(T a, T b, cpx<T> z) { return mk(a * z.x, b * z.y); }
+
 template <typename T>
 __device__ __forceinline__ cpx<T> operator+(cpx<T> a, cpx<T> b) { return mk(a.x + b.x, a.y + b.y); }
 template <typename T>

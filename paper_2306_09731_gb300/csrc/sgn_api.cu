@@ -310,8 +310,8 @@ void build_tables(sgn_ctx* ctx) {
   if (ctx->opt.precision >= 2) {
     // double-float copies: nearest FP32 pair of each FP64 entry
     std::vector<CDF> dx(tx.size()), dy(ty.size());
-    for (size_t k = 0; k < tx.size(); ++k) dx[k] = CDF{dfl(tx[k].x), dfl(tx[k].y)};
-    for (size_t k = 0; k < ty.size(); ++k) dy[k] = CDF{dfl(ty[k].x), dfl(ty[k].y)};
+    for (size_t k = 0; k < tx.size(); ++k) dx[k] = mk_df(dfl(tx[k].x), dfl(tx[k].y));
+    for (size_t k = 0; k < ty.size(); ++k) dy[k] = mk_df(dfl(ty[k].x), dfl(ty[k].y));
     std::vector<dfl> kxd(kx.begin(), kx.end()), kyd(ky.begin(), ky.end()), md(minv.begin(), minv.end());
     ctx->tbd.twx = dalloc<CDF>(ctx, dx.size());
     ctx->tbd.twy = dalloc<CDF>(ctx, dy.size());

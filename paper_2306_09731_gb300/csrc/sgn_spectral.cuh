@@ -60,14 +60,14 @@ __device__ __forceinline__ void load_packed(cpx<T> (&v)[8], const cpx<T>* S0, co
       B = mul_ik(B, kv);
     }
     if (kk == 0 || kk == half) {
-      A.y = (T)0;
-      B.y = (T)0;
+      A = mk(re(A), (T)0);
+      B = mk(re(B), (T)0);
     }
     if (k > half) {
-      A.y = -A.y;
-      B.y = -B.y;
+      A = conjg(A);
+      B = conjg(B);
     }
-    v[s] = mk(A.x - B.y, A.y + B.x);
+    v[s] = A + mul_i(B);
   }
 }
 
@@ -197,8 +197,8 @@ __global__ void k_x_c2r(Geom G, const cpx<T>* __restrict__ tw, const T* __restri
 #pragma unroll
   for (int s = 0; s < 8; ++s) {
     const int x = L.t + s * T_;
-    o[(size_t)L.y0 * N + x] = to_f64<T>(v[s].x) * scale;
-    o[(size_t)L.y1 * N + x] = to_f64<T>(v[s].y) * scale;
+    o[(size_t)L.y0 * N + x] = to_f64<T>(re(v[s])) * scale;
+    o[(size_t)L.y1 * N + x] = to_f64<T>(im(v[s])) * scale;
   }
 }
 
@@ -292,8 +292,8 @@ __global__ void k_coef_x(Geom G, const cpx<T>* __restrict__ tw, const T* __restr
   for (int s = 0; s < 8; ++s) {
     const int x = L.t + s * T_;
     const cpx<T> z = sm[sidx<T>(x, 0)];
-    coef_point_df(scale_pow2(z.x, fN), fN, h, cr, cc, (size_t)L.y0 * N + x, flags, cp);
-    coef_point_df(scale_pow2(z.y, fN), fN, h, cr, cc, (size_t)L.y1 * N + x, flags, cp);
+    coef_point_df(scale_pow2(re(z), fN), fN, h, cr, cc, (size_t)L.y0 * N + x, flags, cp);
+    coef_point_df(scale_pow2(im(z), fN), fN, h, cr, cc, (size_t)L.y1 * N + x, flags, cp);
   }
 }
 
@@ -367,7 +367,7 @@ __global__ void __launch_bounds__(xpass_threads<LN>(), mv_min_blocks<T, LN>()) k
 #pragma unroll
     for (int s = 0; s < 8; ++s) {
       const int x = L.t + s * T_;
-      Z[s] = mk(cf[p0 + x] * Z[s].x, cf[p1 + x] * Z[s].y);
+      Z[s] = mul_xy(cf[p0 + x], cf[p1 + x], Z[s]);
     }
     fft_regs<false>(Z, sm, tw, L.t, lN, 0, PLAN);
     split_pair(Z, sm, L.t, lN, b0, b1);
@@ -462,7 +462,7 @@ __global__ void __launch_bounds__(xpass_threads<LN>(), rhs_min_blocks<T, LN>()) 
         const int x = L.t + s * T_;
         cpx<T>* qx = acc + (size_t)s * T_ + L.t;
         cpx<T>* qy = acc + (size_t)(8 + s) * T_ + L.t;
-        const T z0 = Z[s].x * n, z1 = Z[s].y * n;
+        const T z0 = re(Z[s]) * n, z1 = im(Z[s]) * n;
         if (i == 0) {
           *qx = mk(-z0, -z1);  // -sigma_x
         } else if (i == 1) {
@@ -470,23 +470,20 @@ __global__ void __launch_bounds__(xpass_threads<LN>(), rhs_min_blocks<T, LN>()) 
           const T r0 = cr[p0 + x] * twoN, r1 = cr[p1 + x] * twoN;
           const cpx<T> q = *qx;
           *qy = mk(-z0, -z1);
-          F[s] = mk((T)-0.5 * r0 * r0 * (q.x * q.x + z0 * z0), (T)-0.5 * r1 * r1 * (q.y * q.y + z1 * z1));
+          F[s] = mk((T)-0.5 * r0 * r0 * (re(q) * re(q) + z0 * z0), (T)-0.5 * r1 * r1 * (im(q) * im(q) + z1 * z1));
         } else if (i == 2) {
           // sigma: -9 sigma^2 / (2 h^4)
           const T r0 = cr[p0 + x] * twoN, r1 = cr[p1 + x] * twoN;
           const T q0 = z0 * r0 * r0, q1 = z1 * r1 * r1;
-          F[s].x -= (T)4.5 * q0 * q0;
-          F[s].y -= (T)4.5 * q1 * q1;
+          F[s] = mk(re(F[s]) - (T)4.5 * q0 * q0, im(F[s]) - (T)4.5 * q1 * q1);
         } else {
           // vx, vy: h v and |v|^2/2; with vy also g (h - 1) (see below)
           const T a0 = hh[p0 + x], a1 = hh[p1 + x];  // h - 1
           cpx<T>* q = i == 3 ? qx : qy;
           cpx<T> w = *q;
-          w.x += z0 + a0 * z0;
-          w.y += z1 + a1 * z1;
+          w = mk(re(w) + (z0 + a0 * z0), im(w) + (z1 + a1 * z1));
           const T gh0 = i == 4 ? g * a0 : (T)0, gh1 = i == 4 ? g * a1 : (T)0;
-          F[s].x += (T)0.5 * z0 * z0 + gh0;
-          F[s].y += (T)0.5 * z1 * z1 + gh1;
+          F[s] = mk(re(F[s]) + ((T)0.5 * z0 * z0 + gh0), im(F[s]) + ((T)0.5 * z1 * z1 + gh1));
           // the split returns twice the half spectra: pre-scale by 1/2
           *q = scl(w, (T)0.5);
           if (i == 4) F[s] = scl(F[s], (T)0.5);
@@ -526,8 +523,7 @@ __global__ void __launch_bounds__(xpass_threads<LN>(), rhs_min_blocks<T, LN>()) 
       }
       __syncthreads();
     }
-    return;
-  }
+  } else {
   cpx<T> QX[8], QY[8], F[8], Z[8];
   // grad sigma
   load_packed(QX, S + o0, S + o1, true, kx, L.t, lN);
@@ -619,6 +615,7 @@ __global__ void __launch_bounds__(xpass_threads<LN>(), rhs_min_blocks<T, LN>()) 
     Fh[o0 + k] = f0[s];
     Fh[o1 + k] = f1[s];
   }
+  }
 }
 
 // ------------------------------------------------------------------ y-pass
@@ -639,6 +636,8 @@ __device__ __forceinline__ cpx<T> ld_as(const cpx<S>* p) {
   // the issue-bound RHS y-inverse than the FP64-pipe conversion saves)
   if constexpr (std::is_same<T, dfl>::value && std::is_same<S, double>::value)
     return mk(dfl_from_f64(v.x), dfl_from_f64(v.y));
+  else if constexpr (std::is_same<T, S>::value)
+    return v;
   else
     return mk((T)v.x, (T)v.y);
 }
@@ -1101,8 +1100,9 @@ constexpr int FL_MV_FWD_TMA = yf_tma(0) | yf_tma(1);
 
 // Double-float passes of two or more inputs with one signal live at a time
 // (see ypass_body): the y-inverses that only store and the y-forward passes,
-// 256 threads, MINB blocks per SM: three, two for the three-input y-forward
-// (its stash of two transforms leaves room for two). One input keeps k_ypass:
+// 256 threads, MINB blocks per SM: three, two from three inputs on (the
+// y-forward's stash of two transforms leaves room for two, and the four-input
+// y-inverse spills 308 bytes at three). One input keeps k_ypass:
 // 107 registers there, against 80 with 36 bytes spilled.
 template <int MINB, typename T, bool INV, int NIN, class Epi, typename S = T, int LN = 0, int FL = 0, int PLAN = 0>
 __global__ void __launch_bounds__(256, MINB) k_ypass_df(Geom G, const cpx<T>* __restrict__ tw,
@@ -1123,7 +1123,7 @@ constexpr auto ypass_fn() {
   else if constexpr (sizeof(T) == 4 && INV && is_epi_store<Epi>::value && LN != 12)
     return &k_ypass_f2<T, INV, NIN, Epi, S, LN, FL, PLAN>;
   else if constexpr (std::is_same<T, dfl>::value && (!INV || is_epi_store<Epi>::value) && NIN >= 2 && LN != 12)
-    return &k_ypass_df<(!INV && NIN >= 3) ? 2 : 3, T, INV, NIN, Epi, S, LN, FL, PLAN>;
+    return &k_ypass_df<NIN >= 3 ? 2 : 3, T, INV, NIN, Epi, S, LN, FL, PLAN>;
   else
     return &k_ypass<T, INV, NIN, Epi, S, LN, FL, PLAN>;
 }
@@ -1166,7 +1166,7 @@ struct EpiStoreF64 {
                                              const T* ky) const {
     if (!valid) return;
 #pragma unroll
-    for (int s = 0; s < 8; ++s) dst[(size_t)(t + s * T_) * G.ldS + col] = mk(to_f64<T>(r[0][s].x), to_f64<T>(r[0][s].y));
+    for (int s = 0; s < 8; ++s) dst[(size_t)(t + s * T_) * G.ldS + col] = mk(to_f64<T>(re(r[0][s])), to_f64<T>(im(r[0][s])));
   }
 };
 
@@ -1189,9 +1189,9 @@ struct EpiMatvec {
     cpx<T> z = v[0] - mul_ik(v[1], kyv);
     if (precond) z = scl(z, minv ? ldr(minv + e) : (T)1 / ((T)3 + kxv * kxv + kyv * kyv));
     if constexpr (std::is_same<T, dfl>::value && std::is_same<SO, double>::value)
-      w[e] = mk(dfl_to_f64(z.x), dfl_to_f64(z.y));
+      w[e] = mk(dfl_to_f64(re(z)), dfl_to_f64(im(z)));
     else
-      w[e] = mk((SO)z.x, (SO)z.y);
+      w[e] = mk((SO)re(z), (SO)im(z));
   }
   __device__ __forceinline__ void operator()(cpx<T> (&r)[2][8], int col, int t, int T_, bool valid,
                                              const Geom& G, const T* ky) const {
@@ -1269,7 +1269,7 @@ __global__ void k_rk_update(Geom G, RkK<T, S> a, double c6d, double cdtd, double
     const size_t e = it.e;
     cpx<S> kk[3];
 #pragma unroll
-    for (int f = 0; f < 3; ++f) kk[f] = mk(cvt<S>(a.K[f][e].x), cvt<S>(a.K[f][e].y));
+    for (int f = 0; f < 3; ++f) kk[f] = mk(cvt<S>(re(a.K[f][e])), cvt<S>(im(a.K[f][e])));
     if (rhs_lin_split<T>()) {
       const int my = it.row <= (G.Ny >> 1) ? it.row : G.Ny - it.row;
       const bool keep = it.col < G.Nxh && (!rk.dealias || (3 * it.col <= G.Nx && 3 * my <= G.Ny));
