@@ -295,12 +295,24 @@ void build_tables(sgn_ctx* ctx) {
   std::vector<double> k2x(kx), k2y(ky);
   for (double& k : k2x) k *= two_pi / G.Lx;
   for (double& k : k2y) k *= two_pi / G.Ly;
+  auto upload = [&](const std::vector<double>& v) {
+    double* d = dalloc<double>(ctx, v.size());
+    CK(cudaMemcpy(d, v.data(), v.size() * sizeof(double), cudaMemcpyHostToDevice));
+    return d;
+  };
+  std::vector<double> gkx(kx), gky(ky), kx2(kx), ky2(ky);
+  for (double& k : gkx) k *= ctx->g;
+  for (double& k : gky) k *= ctx->g;
+  for (double& k : kx2) k *= k;
+  for (double& k : ky2) k *= k;
+  ctx->tb.gkx = upload(gkx);
+  ctx->tb.gky = upload(gky);
+  ctx->tb.kx2 = upload(kx2);
+  ctx->tb.ky2 = upload(ky2);
   ctx->tb.twx = dalloc<cpx<fx>>(ctx, qx.size());
   ctx->tb.twy = dalloc<cpx<fx>>(ctx, qy.size());
-  ctx->tb.k2x = dalloc<double>(ctx, G.Nxh);
-  ctx->tb.k2y = dalloc<double>(ctx, G.Ny);
-  CK(cudaMemcpy(ctx->tb.k2x, k2x.data(), G.Nxh * sizeof(double), cudaMemcpyHostToDevice));
-  CK(cudaMemcpy(ctx->tb.k2y, k2y.data(), G.Ny * sizeof(double), cudaMemcpyHostToDevice));
+  ctx->tb.k2x = upload(k2x);
+  ctx->tb.k2y = upload(k2y);
   ctx->tb.kx = dalloc<double>(ctx, G.Nxh);
   ctx->tb.ky = dalloc<double>(ctx, G.Ny);
   CK(cudaMemcpy(ctx->tb.twx, qx.data(), qx.size() * sizeof(qx[0]), cudaMemcpyHostToDevice));
@@ -556,7 +568,6 @@ bool gmres_fp64(sgn_ctx* ctx, int* iters_out, double* relres_out) {
   const size_t vs = G.nspec();
   double* cnorm_d = ctx->scal + 0;
   double* beta_d = ctx->scal + 1;
-  CK(launch_hermitian_fix<double>(G, ctx->bh, EX(ctx)));
   CK(launch_precond<double>(G, ctx->tb, ctx->bh, ctx->cvec, ctx->partials, EX(ctx)));
   CK(launch_reduce(ctx->partials, 1, cnorm_d, true, nullptr, EX(ctx), sweep_partials(G)));
   CK(launch_readback_scalar(cnorm_d, ctx->flags, ctx->rb_dev, EX(ctx)));
@@ -629,7 +640,6 @@ bool gmres_mixed(sgn_ctx* ctx, int* iters_out, double* relres_out) {
   const size_t vs = G.nspec();
   double* cnorm_d = ctx->scal + 0;
   double* beta_d = ctx->scal + 1;
-  CK(launch_hermitian_fix<double>(G, ctx->bh, EX(ctx)));
   CK(launch_precond<double>(G, ctx->tb, ctx->bh, ctx->cvec, ctx->partials, EX(ctx)));
   CK(launch_reduce(ctx->partials, 1, cnorm_d, true, nullptr, EX(ctx), sweep_partials(G)));
   CK(launch_readback_scalar(cnorm_d, ctx->flags, ctx->rb_dev, EX(ctx)));
@@ -800,13 +810,13 @@ void coarse_alloc(sgn_ctx* ctx, int n, float2** tw, float2** Y) {
 void launch_rhs_ctx(sgn_ctx* ctx, C64* const* U, C64* bnext, const RkArgs& rk) {
   if (ctx->opt.precision == 3)
     CK((launch_rhs<dfl, double>(ctx->G, ctx->tbd, ctx->tb, U, ctx->sig, ctx->hd, ctx->crd, tmp_df(ctx), ctx->Un,
-                                ctx->Us, ctx->acc, bnext, rk, EX(ctx))));
+                                ctx->Us, ctx->acc, ctx->bh, bnext, rk, EX(ctx))));
   else if (ctx->opt.precision >= 1)
     CK((launch_rhs<float, double>(ctx->G, ctx->tb32, ctx->tb, U, ctx->sig, ctx->h32, ctx->cr32, ctx->tmp32, ctx->Un,
-                                  ctx->Us, ctx->acc, bnext, rk, EX(ctx))));
+                                  ctx->Us, ctx->acc, ctx->bh, bnext, rk, EX(ctx))));
   else
     CK((launch_rhs<double, double>(ctx->G, ctx->tb, ctx->tb, U, ctx->sig, ctx->h, ctx->cr, ctx->tmp, ctx->Un,
-                                   ctx->Us, ctx->acc, bnext, rk, EX(ctx))));
+                                   ctx->Us, ctx->acc, ctx->bh, bnext, rk, EX(ctx))));
 }
 
 // one RK4 stage (s = 1..4) or a plain RHS evaluation (mode RK_STORE_K)
@@ -1040,8 +1050,7 @@ void graph_gmres(sgn_ctx* ctx, GraphSeg& top) {
   ctl.h_sweep = top.handle();
   top.open();
   long long fixed = count_launches(ctx, [&] {
-    CK(launch_hermitian_fix<double>(G, ctx->bh, EX(ctx)));
-    CK(launch_precond<double>(G, ctx->tb, ctx->bh, ctx->cvec, ctx->partials, EX(ctx)));
+      CK(launch_precond<double>(G, ctx->tb, ctx->bh, ctx->cvec, ctx->partials, EX(ctx)));
     CK(launch_reduce(ctx->partials, 1, cnorm_d, true, nullptr, EX(ctx), sweep_partials(G)));
     CK(launch_ctl_begin(ctx->gst, cnorm_d, ctl, EX(ctx)));
     CK(launch_zero<double>(G, ctx->sig, EX(ctx), &ctx->gst->zero_sigma));

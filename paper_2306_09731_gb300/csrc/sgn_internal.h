@@ -99,6 +99,10 @@ struct Tables {
   cpx<typename tw_type<T>::type>* twy = nullptr;  // W_Ny^k
   T* k2x = nullptr;       // FP64: (2 pi / Lx) kx [Nxh] and (2 pi / Ly) ky [Ny] (see k_fx_mv_x)
   T* k2y = nullptr;
+  T* gkx = nullptr;       // FP64: g kx, g ky, kx^2, ky^2 (see k_rk_update)
+  T* gky = nullptr;
+  T* kx2 = nullptr;
+  T* ky2 = nullptr;
   T* kx = nullptr;        // 2 pi m / Lx, m = 0..Nx/2, Nyquist 0   [Nxh]
   T* ky = nullptr;        // 2 pi m / Ly, m = 0..Ny/2-1, -Ny/2..-1, Nyquist 0 [Ny]
   T* minv = nullptr;      // 1 / (3 + kx^2 + ky^2) per half-spectrum entry [Ny][ldS] (FP64, double-float)
@@ -332,29 +336,33 @@ struct RkK {
   cpx<S>* b;
   const S* kxs;
   const S* kys;
-  // stage state and sigma_hat of the right-hand side (its linear part, added
-  // by the update when the passes run in FP32)
-  const cpx<S>* Y[3];
+  // the right-hand side's linear part, added by the update when the passes run
+  // in FP32: the stage's h_hat, sigma_hat and b_hat, g k and k^2 per column and row
+  const cpx<S>* Yh;
   const cpx<S>* sig;
+  const cpx<S>* bcur;
+  const S* gkx;
+  const S* gky;
+  const S* kx2;
+  const S* ky2;
   RkArgs rk;
 };
 
 // T: compute type of the passes (tmp, h, cr); S: storage type of the state,
-// sigma_hat and b_hat (FP64 in both modes).
+// sigma_hat and b_hat (FP64 in both modes). bcur: the stage's own b_hat (may be
+// bhat, the next stage's).
 template <typename T, typename S>
 cudaError_t launch_rhs(const Geom& G, const Tables<T>& tb, const Tables<S>& tbs, cpx<S>* const* U,
                        const cpx<S>* sig, const T* h, const T* cr, cpx<T>* const* tmp, cpx<S>* const* Un,
-                       cpx<S>* const* Unext, cpx<S>* const* acc, cpx<S>* bhat, const RkArgs& rk,
-                       const Exec& ex);
+                       cpx<S>* const* Unext, cpx<S>* const* acc, const cpx<S>* bcur, cpx<S>* bhat,
+                       const RkArgs& rk, const Exec& ex);
 
 // b_hat = -(i kx vx_hat + i ky vy_hat)
 template <typename T>
 cudaError_t launch_spec_div(const Geom& G, const Tables<T>& tb, const cpx<T>* vx, const cpx<T>* vy,
                             cpx<T>* b, const Exec& ex);
-// project the kx = 0 and kx = Nx/2 columns onto their Hermitian part (in place)
-template <typename T>
-cudaError_t launch_hermitian_fix(const Geom& G, cpx<T>* x, const Exec& ex);
-// out = M^-1 in (spectral), and the weighted squared norm into partials
+// out = M^-1 in (spectral; in's kx = 0 and kx = Nx/2 columns projected onto their
+// Hermitian part), and the weighted squared norm into partials
 template <typename T>
 cudaError_t launch_precond(const Geom& G, const Tables<T>& tb, const cpx<T>* in, cpx<T>* out,
                            double* partials, const Exec& ex);

@@ -447,14 +447,14 @@ __global__ void __launch_bounds__(ORTHO_THR, 1) k_ortho(Geom G, cpx<T>* V, size_
   const size_t n = G.nspec();
   const int nthr = nblk * blockDim.x;
   cpx<T> z[ORTHO_NE];
-  A wt[ORTHO_NE];
+  int wt[ORTHO_NE];
   size_t e[ORTHO_NE];
 #pragma unroll
   for (int k = 0; k < ORTHO_NE; ++k) {
     e[k] = (size_t)blockIdx.x * blockDim.x + threadIdx.x + (size_t)k * nthr;
     const bool in = e[k] < n;
     z[k] = in ? w[e[k]] : mk((T)0, (T)0);
-    wt[k] = in ? col_weight_k<A>(G, (int)(e[k] % G.ldS)) : (A)0;
+    wt[k] = in ? col_weight_i(G, (int)(e[k] % G.ldS)) : 0;
     if (!in) e[k] = 0;
   }
   if (threadIdx.x < MAXV + 1) sc[threadIdx.x] = (int)threadIdx.x <= j ? st->vscl[threadIdx.x] : 0.0;
@@ -563,7 +563,9 @@ __global__ void __launch_bounds__(256) k_residual(Geom G, const cpx<T>* c, const
   for (Walk it(G); it.ok(); it.next()) {
     const cpx<T> z = c[it.e] - w[it.e];
     r[it.e] = z;
-    acc += col_weight_k(G, it.col) * wdot(z, z);
+    const int wt = col_weight_i(G, it.col);
+    const double x = (double)z.x, y = (double)z.y;
+    acc = fma(weigh(wt, x), x, fma(weigh(wt, y), y, acc));
   }
   const double tot = block_reduce(acc, red);
   if (threadIdx.x == 0) partials[blockIdx.x] = tot;
@@ -770,7 +772,8 @@ __global__ void k_ext_start(Geom G, const cpx<double>* ring, size_t vs, int s, c
     const cpx<double>* p3 = ext_slot(ring, vs, head - 4, s);
     for (Walk it(G); it.ok(); it.next()) {
       const cpx<double> a = p0[it.e], b = p1[it.e], c = p2[it.e], d = p3[it.e];
-      sig[it.e] = mk(4.0 * a.x - 6.0 * b.x + 4.0 * c.x - d.x, 4.0 * a.y - 6.0 * b.y + 4.0 * c.y - d.y);
+      // three FP64 instructions a component, not four
+      sig[it.e] = mk(fma(-6.0, b.x, fma(4.0, a.x + c.x, -d.x)), fma(-6.0, b.y, fma(4.0, a.y + c.y, -d.y)));
     }
   } else {
     for (Walk it(G); it.ok(); it.next()) {

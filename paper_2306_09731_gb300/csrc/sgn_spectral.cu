@@ -223,8 +223,9 @@ template <>
 cudaError_t launch_rhs<double, double>(const Geom& G, const Tables<double>& tb, const Tables<double>& tbs,
                                        cpx<double>* const* U, const cpx<double>* sig, const double* h,
                                        const double* cr, cpx<double>* const* tmp, cpx<double>* const* Un,
-                                       cpx<double>* const* Unext, cpx<double>* const* acc, cpx<double>* bhat,
-                                       const RkArgs& rk, const Exec& ex) {
+                                       cpx<double>* const* Unext, cpx<double>* const* acc,
+                                       const cpx<double>* bcur, cpx<double>* bhat, const RkArgs& rk,
+                                       const Exec& ex) {
   dim3 grid, block;
   size_t smem;
   FxYArgs a{};
@@ -259,7 +260,7 @@ cudaError_t launch_rhs<double, double>(const Geom& G, const Tables<double>& tb, 
   f.kx = tb.kx;
   f.dealias = rk.dealias;
   fx_yfwd<3>(G, tb, f, TP_RHS_YFWD, PK_RHS_YFWD, ex);
-  return launch_rk_update<double, double>(G, tbs, U, sig, tmp, Un, Unext, acc, bhat, rk, ex);
+  return launch_rk_update<double, double>(G, tbs, U, sig, tmp, Un, Unext, acc, bcur, bhat, rk, ex);
 }
 
 template cudaError_t launch_coef_phys<double>(const Geom&, const double*, double*, double*, double*, int*,
@@ -268,6 +269,5 @@ template cudaError_t launch_spec_div<double>(const Geom&, const Tables<double>&,
                                              const cpx<double>*, cpx<double>*, const Exec&);
 template cudaError_t launch_precond<double>(const Geom&, const Tables<double>&, const cpx<double>*, cpx<double>*,
                                             double*, const Exec&);
-template cudaError_t launch_hermitian_fix<double>(const Geom&, cpx<double>*, const Exec&);
 
 }  // namespace sgn

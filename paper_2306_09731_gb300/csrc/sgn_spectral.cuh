@@ -1255,7 +1255,11 @@ struct EpiK {
 // With an FP32 right-hand side (rhs_lin_split), K holds only its nonlinear
 // part; the linear part comes from the stage state Y and sigma_hat here:
 //   h_t += -i kx vx - i ky vy - (kx^2 + ky^2) sigma,  v_t += -i k g h,
-// with the zeroed-Nyquist wavenumbers and the 2/3 mask of the FP32 pass.
+// with the zeroed-Nyquist wavenumbers and the 2/3 mask of the FP32 pass. Its
+// first two terms are the stage's own b_hat (a.bcur), which the update before
+// left; g k and k^2 come per column and row from tables: 25 FP64
+// instructions an entry on average instead of 31, and one spectrum less to read
+// (2048^2: 125 -> 112 us; the 580 MB an entry's arrays come to take 85).
 // c6 = dt/6, cdt = the stage's dt (dt/2 or dt) and thr2 = the squared Krasny
 // threshold times (Nx Ny)^2 come from the host (in every thread they would
 // cost an FP64 division and products on the slow FP64 pipe).
@@ -1264,7 +1268,6 @@ __global__ void k_rk_update(Geom G, RkK<T, S> a, double c6d, double cdtd, double
   const RkArgs rk = a.rk;
   const S c6 = (S)c6d;
   const S cdt = (S)cdtd;
-  const S g = (S)rk.g;
   for (Walk it(G); it.ok(); it.next()) {
     const size_t e = it.e;
     cpx<S> kk[3];
@@ -1274,12 +1277,12 @@ __global__ void k_rk_update(Geom G, RkK<T, S> a, double c6d, double cdtd, double
       const int my = it.row <= (G.Ny >> 1) ? it.row : G.Ny - it.row;
       const bool keep = it.col < G.Nxh && (!rk.dealias || (3 * it.col <= G.Nx && 3 * my <= G.Ny));
       if (keep) {
-        const S kxv = __ldg(a.kxs + it.col);
-        const S kyv = __ldg(a.kys + it.row);
-        const cpx<S> yh = a.Y[0][e], yx = a.Y[1][e], yy = a.Y[2][e], sg = a.sig[e];
-        kk[0] = kk[0] - mul_ik(yx, kxv) - mul_ik(yy, kyv) - scl(sg, kxv * kxv + kyv * kyv);
-        kk[1] = kk[1] - mul_ik(yh, g * kxv);
-        kk[2] = kk[2] - mul_ik(yh, g * kyv);
+        const S gkx = __ldg(a.gkx + it.col), gky = __ldg(a.gky + it.row);
+        const S k2 = __ldg(a.kx2 + it.col) + __ldg(a.ky2 + it.row);
+        const cpx<S> yh = a.Yh[e], bc = a.bcur[e], sg = a.sig[e];
+        kk[0] = mk(fma(-k2, sg.x, kk[0].x + bc.x), fma(-k2, sg.y, kk[0].y + bc.y));
+        kk[1] = mk(fma(gkx, yh.y, kk[1].x), fma(-gkx, yh.x, kk[1].y));
+        kk[2] = mk(fma(gky, yh.y, kk[2].x), fma(-gky, yh.x, kk[2].y));
       }
     }
     if (rk.mode == RK_STORE_K) {
@@ -1309,41 +1312,6 @@ __global__ void k_rk_update(Geom G, RkK<T, S> a, double c6d, double cdtd, double
       a.b[e] = mul_ik(u[1], -kxv) - mul_ik(u[2], __ldg(a.kys + it.row));
     }
   }
-}
-
-// The kx = 0 and kx = Nx/2 columns of the half spectrum of a real field are
-// Hermitian in ky: x(-ky) = conj(x(ky)), real at ky = 0 and ky = Ny/2. The
-// inverse transforms read only that part, so an anti-Hermitian remainder (FP32
-// rounding of RK4 increments leaves one in the state) lies in the null space
-// of the discrete operator; left in b_hat it would stall GMRES at its size.
-// This projects both columns onto their Hermitian part, in place.
-template <typename T>
-__global__ void k_hermitian_fix(Geom G, cpx<T>* x) {
-  const int i = blockIdx.x * blockDim.x + threadIdx.x;  // 0 .. Ny/2 for each of the 2 columns
-  const int half = G.Ny >> 1;
-  if (i > 2 * half + 1) return;
-  const int col = (i <= half) ? 0 : (G.Nx >> 1);
-  const int ky = (i <= half) ? i : i - half - 1;
-  const int kn = (G.Ny - ky) & (G.Ny - 1);
-  cpx<T>* a = x + (size_t)ky * G.ldS + col;
-  cpx<T>* b = x + (size_t)kn * G.ldS + col;
-  if (ky == kn) {
-    a->y = (T)0;
-  } else {
-    const cpx<T> va = *a, vb = *b;
-    const cpx<T> h = mk((T)0.5 * (va.x + vb.x), (T)0.5 * (va.y - vb.y));
-    *a = h;
-    *b = conjg(h);
-  }
-}
-
-template <typename T>
-cudaError_t launch_hermitian_fix(const Geom& G, cpx<T>* x, const Exec& ex) {
-  const int n = 2 * ((G.Ny >> 1) + 1);
-  ex.begin(PK_KRYLOV);
-  k_hermitian_fix<T><<<(n + 127) / 128, 128, 0, ex.s>>>(G, x);
-  ex.end();
-  return cudaGetLastError();
 }
 
 // ------------------------------------------------------------ launchers
@@ -1912,7 +1880,7 @@ void init_kernel_attributes_df() {
 template <typename T, typename S>
 static cudaError_t launch_rk_update(const Geom& G, const Tables<S>& tbs, cpx<S>* const* U, const cpx<S>* sig,
                                     cpx<T>* const* tmp, cpx<S>* const* Un, cpx<S>* const* Unext, cpx<S>* const* acc,
-                                    cpx<S>* bhat, const RkArgs& rk, const Exec& ex) {
+                                    const cpx<S>* bcur, cpx<S>* bhat, const RkArgs& rk, const Exec& ex) {
   RkK<T, S> a{};
   for (int f = 0; f < 3; ++f) {
     a.K[f] = tmp[f];
@@ -1923,8 +1891,13 @@ static cudaError_t launch_rk_update(const Geom& G, const Tables<S>& tbs, cpx<S>*
   a.b = bhat;
   a.kxs = tbs.kx;
   a.kys = tbs.ky;
-  for (int f = 0; f < 3; ++f) a.Y[f] = U[f];
+  a.Yh = U[0];
   a.sig = sig;
+  a.bcur = bcur;
+  a.gkx = tbs.gkx;
+  a.gky = tbs.gky;
+  a.kx2 = tbs.kx2;
+  a.ky2 = tbs.ky2;
   a.rk = rk;
   ex.begin(PK_RK);
   k_rk_update<T, S><<<sweep_partials(G), 256, 0, ex.s>>>(G, a, rk.dt / 6.0, rk.mode == RK_STAGE3 ? rk.dt : 0.5 * rk.dt,
@@ -1936,7 +1909,8 @@ static cudaError_t launch_rk_update(const Geom& G, const Tables<S>& tbs, cpx<S>*
 template <typename T, typename S>
 cudaError_t launch_rhs(const Geom& G, const Tables<T>& tb, const Tables<S>& tbs, cpx<S>* const* U,
                        const cpx<S>* sig, const T* h, const T* cr, cpx<T>* const* tmp, cpx<S>* const* Un,
-                       cpx<S>* const* Unext, cpx<S>* const* acc, cpx<S>* bhat, const RkArgs& rk, const Exec& ex) {
+                       cpx<S>* const* Unext, cpx<S>* const* acc, const cpx<S>* bcur, cpx<S>* bhat, const RkArgs& rk,
+                       const Exec& ex) {
   dim3 grid, block;
   size_t smem;
   bool bi = true;
@@ -1996,7 +1970,7 @@ cudaError_t launch_rhs(const Geom& G, const Tables<T>& tb, const Tables<S>& tbs,
     });
     ex.end();
   });
-  return launch_rk_update<T, S>(G, tbs, U, sig, tmp, Un, Unext, acc, bhat, rk, ex);
+  return launch_rk_update<T, S>(G, tbs, U, sig, tmp, Un, Unext, acc, bcur, bhat, rk, ex);
 }
 
 // ------------------------------------------------ spectral pointwise kernels
@@ -2019,19 +1993,28 @@ cudaError_t launch_spec_div(const Geom& G, const Tables<T>& tb, const cpx<T>* vx
   return cudaGetLastError();
 }
 
+// out = M^-1 in and its norm, with the kx = 0 and kx = Nx/2 columns of `in`
+// projected onto their Hermitian part. Those columns of the half spectrum of a
+// real field are Hermitian in ky: x(-ky) = conj(x(ky)), real at ky = 0 and ky =
+// Ny/2. The inverse transforms read only that part, so an anti-Hermitian remainder
+// (FP32 rounding of RK4 increments leaves one in the state) lies in the null space
+// of the discrete operator; left in b_hat it would stall GMRES at its size.
 template <typename T>
-__global__ void __launch_bounds__(256) k_precond(Geom G, const T* __restrict__ kx, const T* __restrict__ ky,
-                                                 const T* __restrict__ minv, const cpx<T>* in, cpx<T>* out,
+__global__ void __launch_bounds__(256) k_precond(Geom G, const T* __restrict__ minv, const cpx<T>* in, cpx<T>* out,
                                                  double* partials) {
   __shared__ double red[32];
   double acc = 0.0;
   for (Walk it(G); it.ok(); it.next()) {
-    const T kxv = it.col < G.Nxh ? __ldg(kx + it.col) : (T)0;
-    const T kyv = __ldg(ky + it.row);
-    const T m = minv ? __ldg(minv + it.e) : (T)1 / ((T)3 + kxv * kxv + kyv * kyv);
-    const cpx<T> z = scl(in[it.e], m);
+    cpx<T> b = in[it.e];
+    if (it.col == 0 || it.col == (G.Nx >> 1)) {
+      const int rn = (G.Ny - it.row) & (G.Ny - 1);
+      const cpx<T> c = in[(size_t)rn * G.ldS + it.col];
+      b = mk((T)0.5 * (b.x + c.x), rn == it.row ? (T)0 : (T)0.5 * (b.y - c.y));
+    }
+    const cpx<T> z = scl(b, __ldg(minv + it.e));
     out[it.e] = z;
-    acc += col_weight_k(G, it.col) * ((double)z.x * z.x + (double)z.y * z.y);
+    const int w = col_weight_i(G, it.col);
+    acc = fma(weigh(w, z.x), z.x, fma(weigh(w, z.y), z.y, acc));
   }
   const double tot = block_reduce(acc, red);
   if (threadIdx.x == 0) partials[blockIdx.x] = tot;
@@ -2041,7 +2024,7 @@ template <typename T>
 cudaError_t launch_precond(const Geom& G, const Tables<T>& tb, const cpx<T>* in, cpx<T>* out, double* partials,
                            const Exec& ex) {
   ex.begin(PK_KRYLOV);
-  k_precond<T><<<sweep_partials(G), 256, 0, ex.s>>>(G, tb.kx, tb.ky, tb.minv, in, out, partials);
+  k_precond<T><<<sweep_partials(G), 256, 0, ex.s>>>(G, tb.minv, in, out, partials);
   ex.end();
   return cudaGetLastError();
 }

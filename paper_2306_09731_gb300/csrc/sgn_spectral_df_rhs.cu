@@ -9,7 +9,8 @@ namespace sgn {
 template cudaError_t launch_rhs<dfl, double>(const Geom&, const Tables<dfl>&, const Tables<double>&,
                                              cpx<double>* const*, const cpx<double>*, const dfl*,
                                              const dfl*, cpx<dfl>* const*, cpx<double>* const*,
-                                             cpx<double>* const*, cpx<double>* const*, cpx<double>*,
+                                             cpx<double>* const*, cpx<double>* const*, const cpx<double>*,
+                                             cpx<double>*,
                                              const RkArgs&, const Exec&);
 
 }  // namespace sgn

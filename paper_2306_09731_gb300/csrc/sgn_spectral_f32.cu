@@ -12,7 +12,8 @@ template cudaError_t launch_matvec<float>(const Geom&, const Tables<float>&, con
 template cudaError_t launch_rhs<float, double>(const Geom&, const Tables<float>&, const Tables<double>&,
                                                cpx<double>* const*, const cpx<double>*, const float*,
                                                const float*, cpx<float>* const*, cpx<double>* const*,
-                                               cpx<double>* const*, cpx<double>* const*, cpx<double>*,
+                                               cpx<double>* const*, cpx<double>* const*, const cpx<double>*,
+                                               cpx<double>*,
                                                const RkArgs&, const Exec&);
 
 }  // namespace sgn

@@ -42,13 +42,17 @@ __device__ __forceinline__ A col_weight_k(const Geom& G, int col) {
   return (col == 0 || col == (G.Nx >> 1)) ? (A)1 : (col < G.Nxh ? (A)2 : (A)0);
 }
 
-// x times the Parseval weight `wt` (0, 1 or 2). In FP64 by the exponent: a
-// product costs a warp 77 issue cycles, this 5.
-__device__ __forceinline__ float weigh(float wt, float x) { return wt * x; }
-__device__ __forceinline__ double weigh(double wt, double x) {
+// x times the Parseval weight wt = 0, 1 or 2 (col_weight_i). In FP64 by the
+// exponent: a product, or a comparison, costs a warp 77 issue cycles, this 5.
+__device__ __forceinline__ int col_weight_i(const Geom& G, int col) {
+  return (col == 0 || col == (G.Nx >> 1)) ? 1 : (col < G.Nxh ? 2 : 0);
+}
+__device__ __forceinline__ float weigh(int wt, float x) { return (float)wt * x; }
+__device__ __forceinline__ double weigh(int wt, double x) {
   const int hi = __double2hiint(x), e = (hi >> 20) & 0x7ff;
-  const bool dbl = wt == 2.0 && e > 0 && e < 0x7ff;
-  return wt == 0.0 ? 0.0 : __hiloint2double(hi + (dbl ? 1 << 20 : 0), __double2loint(x));
+  const bool dbl = wt == 2 && e > 0 && e < 0x7ff;
+  const int h = hi + (dbl ? 1 << 20 : 0);
+  return wt == 0 ? 0.0 : __hiloint2double(h, __double2loint(x));
 }
 
 template <typename T>
