@@ -878,7 +878,7 @@ void tc_conv(sgn_unet_ctx* net, int li, const __nv_bfloat16* src0, int C0, int u
   a.err = net->dev_err;
   const unsigned grid = (unsigned)((a.npix + unet_tc::kM - 1) / unet_tc::kM);
   if (L.row)
-    unet_tc::k_conv3_tc_row<<<grid, unet_tc::kThreads, L.smem, net->stream>>>(a);
+    unet_tc::k_conv3_tc_row<<<grid, unet_tc::kRowThreads, L.smem, net->stream>>>(a);
   else
     unet_tc::k_conv3_tc<<<grid, unet_tc::kThreads, L.smem, net->stream>>>(a);
   UCK(cudaGetLastError());
@@ -887,18 +887,15 @@ void tc_conv(sgn_unet_ctx* net, int li, const __nv_bfloat16* src0, int C0, int u
 void infer_impl(sgn_unet_ctx* net, const float* in, float* out, int B) {
   const int D = net->D;
   const int* w = net->w;
-  {
-    const unsigned nb = (unsigned)((net->wtab.total + 255) / 256);
-    unet_tc::k_wimg<<<nb, 256, 0, net->stream>>>(net->wtab, net->params, net->wimg);
-    UCK(cudaGetLastError());
-  }
   int lg0 = 0;
   while ((1 << lg0) < net->n) ++lg0;
   {
     const Layer& L = net->L[iE(0)];
-    const int np = B * (int)npix(net, 0);
-    unet_tc::k_conv_in_nhwc<<<(np + 127) / 128, 128, sizeof(float) * L.Co * 37, net->stream>>>(
-        in, lg0, lg0, np, net->params + L.woff, net->params + L.boff, L.Co, net->tA[0]);
+    const int np = B * (int)npix(net, 0), nconv = (np + 31) / 32;
+    unet_tc::k_conv_in_wimg<<<nconv + unet_tc::wimg_blocks(net->wtab.total), unet_tc::kInThreads,
+                              sizeof(float) * L.Co * 36, net->stream>>>(
+        in, lg0, lg0, np, net->params + L.woff, net->params + L.boff, L.Co, net->tA[0], nconv, net->wtab, net->params,
+        net->wimg);
     UCK(cudaGetLastError());
   }
   for (int l = 0; l < D - 1; ++l) {
@@ -1263,10 +1260,10 @@ sgn_status conv3_tc_run(int batch, int H, int W, const void* src0, int C0, int u
                            cudaFuncAttributeMaxDynamicSharedMemorySize, sm) != cudaSuccess ||
       cudaMemsetAsync(err, 0, sizeof(int), st) != cudaSuccess)
     return SGN_ECUDA;
-  unet_tc::k_wimg<<<(unsigned)((t.total + 255) / 256), 256, 0, st>>>(t, weight, wimg);
+  unet_tc::k_wimg<<<unet_tc::wimg_blocks(t.total), unet_tc::kInThreads, 0, st>>>(t, weight, wimg);
   const unsigned grid = (unsigned)((a.npix + unet_tc::kM - 1) / unet_tc::kM);
   if (row)
-    unet_tc::k_conv3_tc_row<<<grid, unet_tc::kThreads, sm, st>>>(a);
+    unet_tc::k_conv3_tc_row<<<grid, unet_tc::kRowThreads, sm, st>>>(a);
   else
     unet_tc::k_conv3_tc<<<grid, unet_tc::kThreads, sm, st>>>(a);
   int h = 0;

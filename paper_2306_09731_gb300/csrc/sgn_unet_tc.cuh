@@ -35,7 +35,8 @@
 namespace unet_tc {
 
 constexpr int kM = 128;           // output pixels per CTA = TMEM lanes
-constexpr int kThreads = 128;     // one thread per pixel row
+constexpr int kThreads = 128;     // the step kernel: one thread per pixel row
+constexpr int kRowThreads = 256;  // the row kernel: two threads per pixel row, each half the columns
 constexpr int kStageMax = 56 * 1024;
 constexpr int kMaxKC = 128;       // channels per K step at most (the gather's registers)
 constexpr int kStages = 3;        // shared-memory stages of the K loop
@@ -154,13 +155,19 @@ __host__ __device__ constexpr uint32_t stage_bytes(int Co, int KC) { return a_by
 // The epilogue of both kernels, after the last MMA completed: this thread's
 // TMEM lane (its pixel) read back 16 columns at a time, bias, ReLU, BF16
 // store of the NHWC row; with a head, the 1x1 output convolution of the BF16
-// values in FP32. Every thread of the CTA calls it (tcgen05.ld is warp-wide);
-// valid: whether the pixel exists (a ragged last tile).
-__device__ __forceinline__ void tc_epilogue(const ConvArgs& p, uint32_t tmem, int warp, int pix, bool valid) {
+// values in FP32. A warp reads the 32 lanes of its index modulo 4; of nw > 4
+// warps, those of one lane quarter share its columns in turn - not with a
+// head, whose sum over the columns stays one chain of one thread. Every thread
+// of the CTA calls it (tcgen05.ld is warp-wide); valid: whether the pixel
+// exists (a ragged last tile).
+__device__ __forceinline__ void tc_epilogue(const ConvArgs& p, uint32_t tmem, int warp, int nw, int pix,
+                                            bool valid) {
   tc_fence_after();
-  const uint32_t lane_addr = tmem + ((uint32_t)(warp * 32) << 16);
+  const uint32_t lane_addr = tmem + ((uint32_t)((warp & 3) * 32) << 16);
+  const int step = p.head_w ? 1 : nw >> 2;
+  if (p.head_w && warp >= 4) return;
   float head = 0.f;
-  for (int q = 0; q < p.Co / 16; ++q) {
+  for (int q = warp >> 2; q < p.Co / 16; q += step) {
     float v[16];
     tmem_ld16(lane_addr + (uint32_t)(q * 16), v);
     __align__(16) __nv_bfloat16 o[16];
@@ -292,7 +299,7 @@ __global__ void __launch_bounds__(kThreads) k_conv3_tc(ConvArgs p) {
   }
   ok = __syncthreads_and(ok ? 1 : 0) != 0;
   if (ok) {
-    tc_epilogue(p, tmem, warp, pix, valid);
+    tc_epilogue(p, tmem, warp, kThreads / 32, pix, valid);
   } else if (tid == 0) {
     atomicOr(p.err, SGN_TC_WAIT);
     // let what this CTA still has in flight finish before its memory goes
@@ -308,41 +315,7 @@ __global__ void __launch_bounds__(kThreads) k_conv3_tc(ConvArgs p) {
 
 namespace unet_tc {
 
-// The first layer (4 FP32 NCHW input channels -> Co, ReLU) on CUDA cores: its
-// K = 36 is too short for the tensor cores. One thread per pixel; weights
-// [Co][4][3][3] and biases in shared memory; BF16 NHWC out, 8 channels per
-// 16-byte store.
-__global__ void __launch_bounds__(128) k_conv_in_nhwc(const float* __restrict__ x, int lH, int lW, int npix,
-                                                      const float* __restrict__ w, const float* __restrict__ bias,
-                                                      int Co, __nv_bfloat16* out) {
-  extern __shared__ float ws[];  // Co * 36 weights, then Co biases
-  for (int i = threadIdx.x; i < Co * 37; i += blockDim.x) ws[i] = i < Co * 36 ? w[i] : bias[i - Co * 36];
-  __syncthreads();
-  const int pix = blockIdx.x * blockDim.x + threadIdx.x;
-  if (pix >= npix) return;
-  const int W = 1 << lW, H = 1 << lH;
-  const int xq = pix & (W - 1), yq = (pix >> lW) & (H - 1), b = pix >> (lH + lW);
-  float in[36];
-#pragma unroll
-  for (int ci = 0; ci < 4; ++ci)
-#pragma unroll
-    for (int t = 0; t < 9; ++t) {
-      const int yy = (yq + t / 3 - 1) & (H - 1), xx = (xq + t % 3 - 1) & (W - 1);
-      in[ci * 9 + t] = __ldg(x + (((size_t)(b * 4 + ci)) << (lH + lW)) + ((size_t)yy << lW) + xx);
-    }
-  for (int c8 = 0; c8 < Co / 8; ++c8) {
-    __align__(16) __nv_bfloat16 o[8];
-#pragma unroll
-    for (int j = 0; j < 8; ++j) {
-      const float* wr = ws + (c8 * 8 + j) * 36;
-      float acc = 0.f;
-#pragma unroll
-      for (int k = 0; k < 36; ++k) acc = fmaf(wr[k], in[k], acc);
-      o[j] = __float2bfloat16_rn(fmaxf(acc + ws[Co * 36 + c8 * 8 + j], 0.f));
-    }
-    *reinterpret_cast<uint4*>(out + (size_t)pix * Co + c8 * 8) = *reinterpret_cast<const uint4*>(o);
-  }
-}
+constexpr int kInThreads = 128;
 
 // 2x2 average pool of an NHWC BF16 tensor on a 2^lH x 2^lW grid (C channels,
 // a multiple of 8): one thread per output pixel and 8-channel group, summed in
@@ -388,21 +361,96 @@ struct WImgTable {
   long long total;
 };
 
-__global__ void k_wimg(WImgTable t, const float* __restrict__ params, __nv_bfloat16* img) {
-  const long long i = (long long)blockIdx.x * blockDim.x + threadIdx.x;
-  if (i >= t.total) return;
+// One thread per 8 input channels of one (co, tap), the taps of neighbouring
+// threads: the loads of nine threads are consecutive, and each stores 16 bytes.
+__device__ __forceinline__ void wimg_body(const WImgTable& t, int blk, const float* __restrict__ params,
+                                          __nv_bfloat16* img) {
+  const int i = (blk * kInThreads + (int)threadIdx.x) * 8;
+  if (i >= (int)t.total) return;
   int li = 0;
-  while (li + 1 < t.nl && i >= t.l[li + 1].ioff) ++li;
+  while (li + 1 < t.nl && i >= (int)t.l[li + 1].ioff) ++li;
   const WImgLayer L = t.l[li];
-  const long long r = i - L.ioff;
-  const int blk = L.Co * L.KC;
-  const int step = (int)(r / blk), e = (int)(r % blk);
-  const int cg = L.Co >> 3;
-  const int c = e / (cg * 64), rem = e % (cg * 64);
-  const int co = (rem / 64) * 8 + (rem % 64) / 8, k = c * 8 + (rem & 7);
-  const int tap = L.kb_major ? step % 9 : step / L.nkb, kb = L.kb_major ? step / 9 : step % L.nkb;
-  const int ci = kb * L.KC + k;
-  img[i] = __float2bfloat16_rn(params[L.woff + ((long long)co * L.Ci + ci) * 9 + tap]);
+  const int r = (i - (int)L.ioff) >> 3, tap = r % 9, cc = r / 9, g8 = L.Ci >> 3;
+  const int co = cc / g8, g = cc - co * g8;
+  const float* w = params + L.woff + ((long long)co * L.Ci + g * 8) * 9 + tap;
+  float v[8];
+#pragma unroll
+  for (int k = 0; k < 8; ++k) v[k] = __ldg(w + k * 9);
+  const int c8 = L.KC >> 3, kb = g / c8, c = g - kb * c8;
+  const int step = L.kb_major ? kb * 9 + tap : tap * L.nkb + kb;
+  __align__(16) __nv_bfloat16 o[8];
+#pragma unroll
+  for (int k = 0; k < 8; ++k) o[k] = __float2bfloat16_rn(v[k]);
+  *reinterpret_cast<uint4*>(img + L.ioff + (long long)step * L.Co * L.KC + (c * (L.Co >> 3) + (co >> 3)) * 64 +
+                            (co & 7) * 8) = *reinterpret_cast<const uint4*>(o);
+}
+__host__ __device__ constexpr int wimg_blocks(long long total) {
+  return (int)((total / 8 + kInThreads - 1) / kInThreads);
+}
+
+__global__ void __launch_bounds__(kInThreads) k_wimg(WImgTable t, const float* __restrict__ params,
+                                                     __nv_bfloat16* img) {
+  wimg_body(t, blockIdx.x, params, img);
+}
+
+// The first layer (4 FP32 NCHW input channels -> Co, ReLU) on CUDA cores: its
+// K = 36 is too short for the tensor cores. A warp computes 32 pixels of 8
+// output channels at a time, one pixel a thread; weights [Co][4][3][3] in
+// shared memory, read as vectors of four that the warp shares, and eight
+// independent sums a thread.
+__device__ __forceinline__ void conv_in_body(float4* ws, int blk, const float* __restrict__ x, int lH, int lW,
+                                             int npix, const float* __restrict__ w, const float* __restrict__ bias,
+                                             int Co, __nv_bfloat16* out) {
+  float* wf = reinterpret_cast<float*>(ws);
+  for (int i = threadIdx.x; i < Co * 36; i += kInThreads) wf[i] = __ldg(w + i);
+  const int pix = blk * 32 + (threadIdx.x & 31);
+  const int pq = pix < npix ? pix : npix - 1;
+  const int W = 1 << lW, H = 1 << lH;
+  const int xq = pq & (W - 1), yq = (pq >> lW) & (H - 1), b = pq >> (lH + lW);
+  float in[36];
+#pragma unroll
+  for (int ci = 0; ci < 4; ++ci)
+#pragma unroll
+    for (int t = 0; t < 9; ++t) {
+      const int yy = (yq + t / 3 - 1) & (H - 1), xx = (xq + t % 3 - 1) & (W - 1);
+      in[ci * 9 + t] = __ldg(x + (((size_t)(b * 4 + ci)) << (lH + lW)) + ((size_t)yy << lW) + xx);
+    }
+  __syncthreads();
+  for (int c8 = threadIdx.x >> 5; c8 < Co / 8; c8 += kInThreads / 32) {
+    float acc[8];
+#pragma unroll
+    for (int j = 0; j < 8; ++j) acc[j] = 0.f;
+#pragma unroll
+    for (int k = 0; k < 9; ++k)
+#pragma unroll
+      for (int j = 0; j < 8; ++j) {
+        const float4 v = ws[(c8 * 8 + j) * 9 + k];
+        acc[j] = fmaf(v.x, in[4 * k], acc[j]);
+        acc[j] = fmaf(v.y, in[4 * k + 1], acc[j]);
+        acc[j] = fmaf(v.z, in[4 * k + 2], acc[j]);
+        acc[j] = fmaf(v.w, in[4 * k + 3], acc[j]);
+      }
+    __align__(16) __nv_bfloat16 o[8];
+#pragma unroll
+    for (int j = 0; j < 8; ++j) o[j] = __float2bfloat16_rn(fmaxf(acc[j] + __ldg(bias + c8 * 8 + j), 0.f));
+    if (pix < npix) *reinterpret_cast<uint4*>(out + (size_t)pix * Co + c8 * 8) = *reinterpret_cast<const uint4*>(o);
+  }
+}
+
+// The first launch of a forward pass: the first layer by the blocks below
+// nconv, the weight images of the other layers, which it does not need, by the
+// rest. Both are short and latency-bound, 8.5 and 5.7 us as two launches (one
+// thread per pixel and all channels, one per image element) at 128^2.
+__global__ void __launch_bounds__(kInThreads) k_conv_in_wimg(const float* __restrict__ x, int lH, int lW, int npix,
+                                                             const float* __restrict__ w,
+                                                             const float* __restrict__ bias, int Co,
+                                                             __nv_bfloat16* out, int nconv, WImgTable t,
+                                                             const float* __restrict__ params, __nv_bfloat16* img) {
+  extern __shared__ float4 ws[];  // Co * 9
+  if ((int)blockIdx.x < nconv)
+    conv_in_body(ws, blockIdx.x, x, lH, lW, npix, w, bias, Co, out);
+  else
+    wimg_body(t, blockIdx.x - nconv, params, img);
 }
 
 }  // namespace unet_tc
@@ -441,14 +489,14 @@ __host__ __device__ constexpr uint32_t row_smem_bytes(int Co, int KC, int nkb, i
   return (nkb > 1 ? 2u : 1u) * (halo_bytes(KC, W) + 9u * b_bytes(Co, KC));
 }
 
-__device__ __forceinline__ void cp_async16(void* dst, const void* src) {
-  asm volatile("cp.async.cg.shared.global [%0], [%1], 16;\n" ::"r"(smem_addr(dst)), "l"(src) : "memory");
+__device__ __forceinline__ void cp_async16(uint32_t dst, const void* src) {
+  asm volatile("cp.async.cg.shared.global [%0], [%1], 16;\n" ::"r"(dst), "l"(src) : "memory");
 }
 __device__ __forceinline__ void cp_async_commit() { asm volatile("cp.async.commit_group;\n" ::: "memory"); }
 __device__ __forceinline__ void cp_async_wait1() { asm volatile("cp.async.wait_group 1;\n" ::: "memory"); }
 __device__ __forceinline__ void cp_async_wait0() { asm volatile("cp.async.wait_group 0;\n" ::: "memory"); }
 
-__global__ void __launch_bounds__(kThreads) k_conv3_tc_row(ConvArgs p) {
+__global__ void __launch_bounds__(kRowThreads) k_conv3_tc_row(ConvArgs p) {
   extern __shared__ __align__(1024) unsigned char sm[];
   __shared__ __align__(8) uint64_t bar_w[2], bar_mma[2];
   __shared__ uint32_t tmem_slot;
@@ -486,39 +534,44 @@ __global__ void __launch_bounds__(kThreads) k_conv3_tc_row(ConvArgs p) {
     y = (tile % tiles_img) * rows;
     b = tile / tiles_img;
   }
-  const int pix = tile * kM + tid;
+  const int pix = tile * kM + (tid & (kM - 1));
   const uint32_t idesc = instr_desc_bf16(kM, Co);
 
-  // channel block kb's halo (cp.async, piece i = (position, chunk), chunk
-  // fastest) and its nine taps' weights (one bulk copy, thread 0) into buffer bf
+  // channel block kb's halo and its nine taps' weights (one bulk copy, thread
+  // 0) into buffer bf. A thread keeps one 16-byte chunk of the channels, so
+  // its source tensor and channel are fixed for the block, and walks the input
+  // pixels: an address is a few shifts, and in narrow grids it serves all
+  // three copies.
+  const int chunks = KC >> 3, per = kRowThreads / chunks;
+  const int lc = tid % chunks, lp = tid / chunks;
   auto load_block = [&](int kb, int bf) {
     unsigned char* dst = sm + (size_t)bf * bufbytes;
     if (tid == 0)
       bulk_g2s(dst + hbytes, p.wimg + (size_t)kb * 9 * Co * KC, wbytes, &bar_w[bf], (p.stall && kb == 0) ? 16u : 0u);
-    const int chunks = KC >> 3, pieces = halo_copies(W) * P * chunks;
-    for (int i = tid; i < pieces; i += kThreads) {
-      const int kx = i / (P * chunks), rem = i - kx * P * chunks;
-      const int pos = rem / chunks, c = rem - pos * chunks;
-      int gy, gx;
-      if (wide) {
-        const int r = pos / (kM + 2), col = pos - r * (kM + 2);
-        gy = (y + r - 1) & (H - 1);
-        gx = (x0 + col - 1) & (W - 1);
-      } else {
-        const int r = pos >> p.lW, xx = pos & (W - 1);
-        gy = (y + r - 1) & (H - 1);
-        gx = (xx + kx - 1) & (W - 1);
+    if (lp >= per) return;
+    const int ch = kb * KC + 8 * lc;
+    const bool first = ch < p.C0;
+    const int up = first && p.up0 ? 1 : 0, C = first ? p.C0 : p.C1;
+    const __nv_bfloat16* src =
+        (first ? p.src0 + ch : p.src1 + (ch - p.C0)) + ((size_t)b << (p.lH + p.lW - 2 * up)) * C;
+    const uint32_t d0 = smem_addr(dst) + (uint32_t)lc * P * 16u;
+    if (wide) {
+#pragma unroll 4
+      for (int q = lp; q < kHaloPos; q += per) {
+        const int r = (q >= kM + 2) + (q >= 2 * (kM + 2)), col = q - r * (kM + 2);
+        const int gy = (y + r - 1) & (H - 1), gx = (x0 + col - 1) & (W - 1);
+        cp_async16(d0 + (uint32_t)q * 16u, src + (size_t)(((gy >> up) << (p.lW - up)) + (gx >> up)) * C);
       }
-      const int ch = kb * KC + 8 * c;
-      const __nv_bfloat16* src;
-      if (ch < p.C0) {
-        src = p.up0 ? p.src0 + ((((size_t)b << (p.lH + p.lW - 2)) + ((size_t)(gy >> 1) << (p.lW - 1)) + (gx >> 1)) *
-                                    p.C0 + ch)
-                    : p.src0 + ((((size_t)b << (p.lH + p.lW)) + ((size_t)gy << p.lW) + gx) * p.C0 + ch);
-      } else {
-        src = p.src1 + ((((size_t)b << (p.lH + p.lW)) + ((size_t)gy << p.lW) + gx) * p.C1 + (ch - p.C0));
+    } else {
+      const uint32_t cp = (uint32_t)chunks * P * 16u;  // bytes between the copies
+#pragma unroll 4
+      for (int q = lp; q < P; q += per) {
+        const int r = q >> p.lW, gx = q & (W - 1), gy = (y + r - 1) & (H - 1);
+        const __nv_bfloat16* g = src + (size_t)(((gy >> up) << (p.lW - up)) + (gx >> up)) * C;
+        const uint32_t d = d0 + ((uint32_t)r << p.lW) * 16u;
+#pragma unroll
+        for (int kx = 0; kx < 3; ++kx) cp_async16(d + kx * cp + (uint32_t)((gx + 1 - kx) & (W - 1)) * 16u, g);
       }
-      cp_async16(dst + ((size_t)(kx * chunks + c) * P + pos) * 16, src);
     }
   };
   // block kb uses buffer kb & 1; its k-th use is phase k of that buffer's barriers
@@ -590,7 +643,7 @@ __global__ void __launch_bounds__(kThreads) k_conv3_tc_row(ConvArgs p) {
   }
   ok = __syncthreads_and(ok ? 1 : 0) != 0;
   if (ok) {
-    tc_epilogue(p, tmem, warp, pix, true);
+    tc_epilogue(p, tmem, warp, kRowThreads / 32, pix, true);
   } else if (tid == 0) {
     atomicOr(p.err, SGN_TC_WAIT);
     // drain in order what this CTA still has in flight
