@@ -152,6 +152,19 @@ __host__ __device__ constexpr uint32_t a_bytes(int KC) { return (uint32_t)kM * K
 __host__ __device__ constexpr uint32_t b_bytes(int Co, int KC) { return (uint32_t)Co * KC * 2u; }
 __host__ __device__ constexpr uint32_t stage_bytes(int Co, int KC) { return a_bytes(KC) + b_bytes(Co, KC); }
 
+// Bias and head weights of a layer, staged in shared memory while the first
+// operands are on their way: read in the epilogue they were a chain of loads
+// from L2, 1200 to 3500 cycles of a tile's 9 to 30 thousand.
+struct __align__(16) Consts {
+  float bias[256], head[256];
+};
+__device__ __forceinline__ void load_consts(const ConvArgs& p, Consts& k, int tid, int nt) {
+  for (int i = tid; i < p.Co; i += nt) {
+    k.bias[i] = __ldg(p.bias + i);
+    if (p.head_w) k.head[i] = __ldg(p.head_w + i);
+  }
+}
+
 // The epilogue of both kernels, after the last MMA completed: this thread's
 // TMEM lane (its pixel) read back 16 columns at a time, bias, ReLU, BF16
 // store of the NHWC row; with a head, the 1x1 output convolution of the BF16
@@ -160,8 +173,8 @@ __host__ __device__ constexpr uint32_t stage_bytes(int Co, int KC) { return a_by
 // head, whose sum over the columns stays one chain of one thread. Every thread
 // of the CTA calls it (tcgen05.ld is warp-wide); valid: whether the pixel
 // exists (a ragged last tile).
-__device__ __forceinline__ void tc_epilogue(const ConvArgs& p, uint32_t tmem, int warp, int nw, int pix,
-                                            bool valid) {
+__device__ __forceinline__ void tc_epilogue(const ConvArgs& p, const Consts& k, uint32_t tmem, int warp, int nw,
+                                            int pix, bool valid) {
   tc_fence_after();
   const uint32_t lane_addr = tmem + ((uint32_t)((warp & 3) * 32) << 16);
   const int step = p.head_w ? 1 : nw >> 2;
@@ -173,9 +186,9 @@ __device__ __forceinline__ void tc_epilogue(const ConvArgs& p, uint32_t tmem, in
     __align__(16) __nv_bfloat16 o[16];
 #pragma unroll
     for (int i = 0; i < 16; ++i) {
-      const float a = fmaxf(v[i] + __ldg(p.bias + q * 16 + i), 0.f);
+      const float a = fmaxf(v[i] + k.bias[q * 16 + i], 0.f);
       o[i] = __float2bfloat16_rn(a);
-      if (p.head_w) head = fmaf(__ldg(p.head_w + q * 16 + i), __bfloat162float(o[i]), head);
+      if (p.head_w) head = fmaf(k.head[q * 16 + i], __bfloat162float(o[i]), head);
     }
     if (valid && p.out) {
       uint4* dst = reinterpret_cast<uint4*>(p.out + (size_t)pix * p.Co + q * 16);
@@ -190,6 +203,7 @@ __global__ void __launch_bounds__(kThreads) k_conv3_tc(ConvArgs p) {
   extern __shared__ __align__(1024) unsigned char sm[];
   __shared__ __align__(8) uint64_t bar_w[kStages], bar_mma[kStages];
   __shared__ uint32_t tmem_slot;
+  __shared__ Consts consts;
   const int tid = threadIdx.x, warp = tid >> 5;
   const int KC = p.KC, Co = p.Co;
   const uint32_t abytes = a_bytes(KC), sbytes = stage_bytes(Co, KC);
@@ -250,6 +264,7 @@ __global__ void __launch_bounds__(kThreads) k_conv3_tc(ConvArgs p) {
     copied = 0;
   }
   gather(0);
+  load_consts(p, consts, tid, kThreads);
   for (int s = 0; s < nsteps; ++s) {
     const int buf = stage_of(s);
     // the MMAs of step s - 2 (and so of every earlier step) are done: stage
@@ -299,7 +314,7 @@ __global__ void __launch_bounds__(kThreads) k_conv3_tc(ConvArgs p) {
   }
   ok = __syncthreads_and(ok ? 1 : 0) != 0;
   if (ok) {
-    tc_epilogue(p, tmem, warp, kThreads / 32, pix, valid);
+    tc_epilogue(p, consts, tmem, warp, kThreads / 32, pix, valid);
   } else if (tid == 0) {
     atomicOr(p.err, SGN_TC_WAIT);
     // let what this CTA still has in flight finish before its memory goes
@@ -480,8 +495,14 @@ constexpr int kHaloPos = 3 * (kM + 2);
 // positions per chunk of one halo copy, and the copies
 __host__ __device__ constexpr int halo_pos(int W) { return W >= kM ? kHaloPos : kM + 2 * W; }
 __host__ __device__ constexpr int halo_copies(int W) { return W >= kM ? 1 : 3; }
+// positions from one chunk of a copy to the next: as many as put the chunks
+// that eight lanes write together (load_block) into different banks, 2 modulo
+// 8 for four chunks of two pixels, 4 modulo 8 for two chunks of four
+__host__ __device__ constexpr int halo_stride(int KC, int W) {
+  return (halo_pos(W) & ~7) + (KC % 32 ? 4 : 2) + ((halo_pos(W) & 7) > (KC % 32 ? 4 : 2) ? 8 : 0);
+}
 __host__ __device__ constexpr uint32_t halo_bytes(int KC, int W) {
-  return (uint32_t)halo_copies(W) * halo_pos(W) * KC * 2u;
+  return (uint32_t)halo_copies(W) * halo_stride(KC, W) * KC * 2u;
 }
 // one buffer of halo + weights per channel block in flight (two when there
 // are several blocks)
@@ -496,15 +517,58 @@ __device__ __forceinline__ void cp_async_commit() { asm volatile("cp.async.commi
 __device__ __forceinline__ void cp_async_wait1() { asm volatile("cp.async.wait_group 1;\n" ::: "memory"); }
 __device__ __forceinline__ void cp_async_wait0() { asm volatile("cp.async.wait_group 0;\n" ::: "memory"); }
 
+// one lane of a converged warp
+__device__ __forceinline__ bool elect_one() {
+  uint32_t e;
+  asm volatile("{\n .reg .pred p;\n elect.sync _|p, 0xffffffff;\n selp.u32 %0, 1, 0, p;\n}\n" : "=r"(e));
+  return e != 0;
+}
+// The MMAs of one channel block: tap (ky, kx), K step j read A at
+// kx kx' + ky ky' + j aj and B at (tap KC/16 + j) bj from the block's first
+// descriptors, in units of 16 bytes (the address is a descriptor's low field
+// and stays below its 14 bits, so an offset is one addition).
+struct TapSteps {
+  uint64_t a, b;
+  uint32_t kx, ky, aj, bj;
+};
+template <int NJ>
+__device__ __forceinline__ void issue_taps(uint32_t tmem, const TapSteps& t, uint32_t idesc, int nj, bool acc) {
+  const int n = NJ ? NJ : nj;
+#pragma unroll
+  for (int tap = 0; tap < 9; ++tap) {
+    uint64_t a = t.a + (uint32_t)((tap % 3) * t.kx + (tap / 3) * t.ky), b = t.b + (uint32_t)(tap * n) * t.bj;
+#pragma unroll
+    for (int j = 0; j < n; ++j) {
+      mma_bf16(tmem, a, b, idesc, (tap > 0 || j > 0 || acc) ? 1 : 0);
+      a += t.aj;
+      b += t.bj;
+    }
+  }
+}
+// Unrolled for the usual channel counts: with loops over the taps and steps,
+// the one issuing thread needed 98 cycles an MMA and 195 a tap, more than the
+// tensor core.
+__device__ __forceinline__ void issue_block(uint32_t tmem, const TapSteps& t, uint32_t idesc, int nj, bool acc) {
+  switch (nj) {
+    case 1: return issue_taps<1>(tmem, t, idesc, nj, acc);
+    case 2: return issue_taps<2>(tmem, t, idesc, nj, acc);
+    case 3: return issue_taps<3>(tmem, t, idesc, nj, acc);
+    case 4: return issue_taps<4>(tmem, t, idesc, nj, acc);
+    case 6: return issue_taps<6>(tmem, t, idesc, nj, acc);
+    default: return issue_taps<0>(tmem, t, idesc, nj, acc);
+  }
+}
+
 __global__ void __launch_bounds__(kRowThreads) k_conv3_tc_row(ConvArgs p) {
   extern __shared__ __align__(1024) unsigned char sm[];
   __shared__ __align__(8) uint64_t bar_w[2], bar_mma[2];
   __shared__ uint32_t tmem_slot;
-  const int tid = threadIdx.x, warp = tid >> 5;
+  __shared__ Consts consts;
+  const int tid = threadIdx.x, warp = __shfl_sync(0xffffffffu, threadIdx.x >> 5, 0);
   const int KC = p.KC, Co = p.Co, nkb = p.nkb;
   const int W = 1 << p.lW, H = 1 << p.lH;
   const bool wide = W >= kM;
-  const int P = halo_pos(W);  // positions of one chunk of one halo copy
+  const int P = halo_stride(KC, W);  // positions between the chunks of a halo copy
   const uint32_t hbytes = halo_bytes(KC, W), wbytes = 9u * b_bytes(Co, KC), bufbytes = hbytes + wbytes;
   const uint32_t sm0 = smem_addr(sm);
 
@@ -538,39 +602,49 @@ __global__ void __launch_bounds__(kRowThreads) k_conv3_tc_row(ConvArgs p) {
   const uint32_t idesc = instr_desc_bf16(kM, Co);
 
   // channel block kb's halo and its nine taps' weights (one bulk copy, thread
-  // 0) into buffer bf. A thread keeps one 16-byte chunk of the channels, so
-  // its source tensor and channel are fixed for the block, and walks the input
-  // pixels: an address is a few shifts, and in narrow grids it serves all
-  // three copies.
-  const int chunks = KC >> 3, per = kRowThreads / chunks;
-  const int lc = tid % chunks, lp = tid / chunks;
+  // 0) into buffer bf. A warp copies 4 channel chunks of 8 consecutive pixels
+  // at a time (2 of 16 where KC is no multiple of 32), the chunks fastest:
+  // eight lanes, which the load unit takes together, read 2 (4) lines and
+  // write 8 banks groups. With all chunks of one pixel, or one chunk of eight
+  // pixels, such a copy of 512 bytes took 38 cycles, in bank conflicts or in
+  // lines; @.
+  // One address serves a pixel's chunks and, in narrow grids, all three copies.
+  const int chunks = KC >> 3;
+  const int lq = (chunks & 3) ? 1 : 2;  // log2 of the chunks a warp takes side by side
+  const int lpx = (tid & 31) >> lq, lc = tid & ((1 << lq) - 1);
   auto load_block = [&](int kb, int bf) {
     unsigned char* dst = sm + (size_t)bf * bufbytes;
     if (tid == 0)
       bulk_g2s(dst + hbytes, p.wimg + (size_t)kb * 9 * Co * KC, wbytes, &bar_w[bf], (p.stall && kb == 0) ? 16u : 0u);
-    if (lp >= per) return;
-    const int ch = kb * KC + 8 * lc;
-    const bool first = ch < p.C0;
-    const int up = first && p.up0 ? 1 : 0, C = first ? p.C0 : p.C1;
-    const __nv_bfloat16* src =
-        (first ? p.src0 + ch : p.src1 + (ch - p.C0)) + ((size_t)b << (p.lH + p.lW - 2 * up)) * C;
+    const int up = p.up0 ? 1 : 0, ch0 = kb * KC + 8 * lc;
+    const __nv_bfloat16* s0 = p.src0 + ((size_t)b << (p.lH + p.lW - 2 * up)) * p.C0 + ch0;
+    const __nv_bfloat16* s1 = p.src1 + ((size_t)b << (p.lH + p.lW)) * p.C1 + (ch0 - p.C0);
     const uint32_t d0 = smem_addr(dst) + (uint32_t)lc * P * 16u;
-    if (wide) {
-#pragma unroll 4
-      for (int q = lp; q < kHaloPos; q += per) {
-        const int r = (q >= kM + 2) + (q >= 2 * (kM + 2)), col = q - r * (kM + 2);
-        const int gy = (y + r - 1) & (H - 1), gx = (x0 + col - 1) & (W - 1);
-        cp_async16(d0 + (uint32_t)q * 16u, src + (size_t)(((gy >> up) << (p.lW - up)) + (gx >> up)) * C);
+    const uint32_t cp = (uint32_t)chunks * P * 16u;  // bytes between the copies
+    const int n = halo_pos(W);
+#pragma unroll 2
+    for (int q = warp * (32 >> lq) + lpx; q < n; q += (kRowThreads / 32) * (32 >> lq)) {
+      int r, gx;
+      if (wide) {
+        r = (q >= kM + 2) + (q >= 2 * (kM + 2));
+        gx = (x0 + q - r * (kM + 2) - 1) & (W - 1);
+      } else {
+        r = q >> p.lW;
+        gx = q & (W - 1);
       }
-    } else {
-      const uint32_t cp = (uint32_t)chunks * P * 16u;  // bytes between the copies
-#pragma unroll 4
-      for (int q = lp; q < P; q += per) {
-        const int r = q >> p.lW, gx = q & (W - 1), gy = (y + r - 1) & (H - 1);
-        const __nv_bfloat16* g = src + (size_t)(((gy >> up) << (p.lW - up)) + (gx >> up)) * C;
-        const uint32_t d = d0 + ((uint32_t)r << p.lW) * 16u;
+      const int gy = (y + r - 1) & (H - 1);
+      const __nv_bfloat16* g0 = s0 + (size_t)(((gy >> up) << (p.lW - up)) + (gx >> up)) * p.C0;
+      const __nv_bfloat16* g1 = s1 + (size_t)((gy << p.lW) + gx) * p.C1;
+      const uint32_t d = d0 + (wide ? (uint32_t)q : (uint32_t)r << p.lW) * 16u;
+      for (int c = 0; c < chunks; c += 1 << lq) {
+        const __nv_bfloat16* g = (ch0 + 8 * c < p.C0 ? g0 : g1) + 8 * c;
+        const uint32_t dc = d + (uint32_t)c * P * 16u;
+        if (wide) {
+          cp_async16(dc, g);
+        } else {
 #pragma unroll
-        for (int kx = 0; kx < 3; ++kx) cp_async16(d + kx * cp + (uint32_t)((gx + 1 - kx) & (W - 1)) * 16u, g);
+          for (int kx = 0; kx < 3; ++kx) cp_async16(dc + kx * cp + (uint32_t)((gx + 1 - kx) & (W - 1)) * 16u, g);
+        }
       }
     }
   };
@@ -578,17 +652,18 @@ __global__ void __launch_bounds__(kRowThreads) k_conv3_tc_row(ConvArgs p) {
   auto parity_of = [](int kb) { return (unsigned)((kb >> 1) & 1); };
 
   // A parity wait tells a phase only from the one before it, so every wait
-  // on an mbarrier here is made by thread 0, which sees every commit and every
-  // copy in order; the other threads learn the outcome through the block votes.
+  // on an mbarrier here is made by warp 0, which sees every commit and every
+  // copy in order; the other warps learn the outcome through the block votes.
   bool ok = true;
   int issued = -1, mma_seen = -1, copied = 0, copy_done = -1;
   load_block(0, 0);
   cp_async_commit();
+  load_consts(p, consts, tid, kRowThreads);
   for (int kb = 0; kb < nkb; ++kb) {
     const int bf = kb & 1;
     const bool pre = kb + 1 < nkb;
     // buffer bf ^ 1 was block kb - 1's: its MMAs must be done
-    if (tid == 0 && pre && kb >= 1) {
+    if (warp == 0 && pre && kb >= 1) {
       if (bar_wait(&bar_mma[(kb - 1) & 1], parity_of(kb - 1)))
         mma_seen = kb - 1;
       else
@@ -600,42 +675,38 @@ __global__ void __launch_bounds__(kRowThreads) k_conv3_tc_row(ConvArgs p) {
     }
     if (pre) {
       load_block(kb + 1, bf ^ 1);
-      if (tid == 0) copied = kb + 1;
+      copied = kb + 1;
     }
     cp_async_commit();
     cp_async_wait1();
     fence_async_smem();
     __syncthreads();
-    if (tid == 0) {
-      if (!bar_wait(&bar_w[bf], parity_of(kb))) {
+    if (warp == 0) {
+      if (!__all_sync(0xffffffffu, bar_wait(&bar_w[bf], parity_of(kb)))) {
         ok = false;
       } else {
         copy_done = kb;
         tc_fence_after();
-        const uint32_t hbase = sm0 + (uint32_t)bf * bufbytes, wbase = hbase + hbytes;
-        const uint32_t cstride = (uint32_t)P * 16u;  // bytes between chunks of a copy (LBO)
-#pragma unroll 1
-        for (int tap = 0; tap < 9; ++tap) {
-          const int ky = tap / 3, kx = tap % 3;
-          const uint32_t a0 =
-              hbase + (wide ? (uint32_t)((ky * (kM + 2) + kx) * 16)
-                            : (uint32_t)kx * (uint32_t)(KC >> 3) * cstride + (uint32_t)(ky * W * 16));
-          const uint32_t b0 = wbase + (uint32_t)tap * b_bytes(Co, KC);
-#pragma unroll 1
-          for (int j = 0; j < KC / 16; ++j) {
-            const uint64_t ad = smem_desc(a0 + (uint32_t)j * 2u * cstride, cstride, 128u);
-            const uint64_t bd = smem_desc(b0 + (uint32_t)j * 2u * (uint32_t)(Co / 8) * 128u,
-                                          (uint32_t)(Co / 8) * 128u, 128u);
-            mma_bf16(tmem, ad, bd, idesc, (kb > 0 || tap > 0 || j > 0) ? 1 : 0);
-          }
+        if (elect_one()) {
+          const uint32_t hbase = sm0 + (uint32_t)bf * bufbytes;
+          const uint32_t cstride = (uint32_t)P * 16u;  // bytes between chunks of a copy (LBO)
+          TapSteps t;
+          t.a = smem_desc(hbase, cstride, 128u);
+          t.b = smem_desc(hbase + hbytes, (uint32_t)(Co / 8) * 128u, 128u);
+          t.kx = wide ? 1u : (uint32_t)(chunks * P);
+          t.ky = wide ? (uint32_t)(kM + 2) : (uint32_t)W;
+          t.aj = 2u * P;
+          t.bj = 2u * Co;
+          issue_block(tmem, t, idesc, KC >> 4, kb > 0);
+          mma_commit(&bar_mma[bf]);
         }
-        mma_commit(&bar_mma[bf]);
+        __syncwarp();
         issued = kb;
       }
     }
   }
   // the last block's commit (the one before it was seen before its buffer was refilled)
-  if (ok && tid == 0) {
+  if (ok && warp == 0) {
     if (bar_wait(&bar_mma[(nkb - 1) & 1], parity_of(nkb - 1)))
       mma_seen = nkb - 1;
     else
@@ -643,7 +714,7 @@ __global__ void __launch_bounds__(kRowThreads) k_conv3_tc_row(ConvArgs p) {
   }
   ok = __syncthreads_and(ok ? 1 : 0) != 0;
   if (ok) {
-    tc_epilogue(p, tmem, warp, kRowThreads / 32, pix, true);
+    tc_epilogue(p, consts, tmem, warp, kRowThreads / 32, pix, true);
   } else if (tid == 0) {
     atomicOr(p.err, SGN_TC_WAIT);
     // drain in order what this CTA still has in flight
