@@ -109,6 +109,12 @@ __device__ __forceinline__ void mma_commit(uint64_t* b) {
   asm volatile("tcgen05.commit.cta_group::1.mbarrier::arrive::one.shared::cluster.b64 [%0];\n" ::"r"(smem_addr(b))
                : "memory");
 }
+// Programmatic dependent launch: what the launch before wrote is visible after
+// dep_wait, and dep_go lets the next launch's blocks start their preparation.
+// Each block waits before it goes on, so a launch starts only when the one two
+// before it is complete. Without the launch attribute both do nothing.
+__device__ __forceinline__ void dep_wait() { asm volatile("griddepcontrol.wait;\n" ::: "memory"); }
+__device__ __forceinline__ void dep_go() { asm volatile("griddepcontrol.launch_dependents;\n" ::: "memory"); }
 // 16 consecutive FP32 columns of this thread's TMEM lane
 __device__ __forceinline__ void tmem_ld16(uint32_t taddr, float (&v)[16]) {
   uint32_t r[16];
@@ -143,6 +149,7 @@ struct ConvArgs {
   const float* head_b;
   float* head_out;            // [npix] FP32
   int* err;
+  int early_w;                // the weight image is complete two launches before this one
   int stall;                  // self-test only: arm step 0's weight barrier for 16 bytes more
                               // than its copy delivers, so that its waits run out
 };
@@ -335,10 +342,12 @@ constexpr int kInThreads = 128;
 // 2x2 average pool of an NHWC BF16 tensor on a 2^lH x 2^lW grid (C channels,
 // a multiple of 8): one thread per output pixel and 8-channel group, summed in
 // FP32 as (a + b) + (c + d) over the rows 2y, 2y + 1.
-__global__ void k_pool_nhwc(const __nv_bfloat16* __restrict__ in, int lH, int lW, int C, int nout,
+__global__ void k_pool_nhwc(const __nv_bfloat16* in, int lH, int lW, int C, int nout,
                             __nv_bfloat16* out) {
   const int i = blockIdx.x * blockDim.x + threadIdx.x;
   const int groups = C >> 3;
+  dep_wait();
+  dep_go();
   if (i >= nout * groups) return;
   const int g = i % groups, op = i / groups;
   const int W2 = 1 << (lW - 1), H2 = 1 << (lH - 1);
@@ -346,10 +355,10 @@ __global__ void k_pool_nhwc(const __nv_bfloat16* __restrict__ in, int lH, int lW
   const size_t base = ((((size_t)b << (lH + lW)) + ((size_t)(2 * oy) << lW) + 2 * ox) * C) + g * 8;
   const size_t row = (size_t)C << lW;
   __align__(16) __nv_bfloat16 v[4][8];
-  *reinterpret_cast<uint4*>(v[0]) = __ldg(reinterpret_cast<const uint4*>(in + base));
-  *reinterpret_cast<uint4*>(v[1]) = __ldg(reinterpret_cast<const uint4*>(in + base + C));
-  *reinterpret_cast<uint4*>(v[2]) = __ldg(reinterpret_cast<const uint4*>(in + base + row));
-  *reinterpret_cast<uint4*>(v[3]) = __ldg(reinterpret_cast<const uint4*>(in + base + row + C));
+  *reinterpret_cast<uint4*>(v[0]) = *reinterpret_cast<const uint4*>(in + base);
+  *reinterpret_cast<uint4*>(v[1]) = *reinterpret_cast<const uint4*>(in + base + C);
+  *reinterpret_cast<uint4*>(v[2]) = *reinterpret_cast<const uint4*>(in + base + row);
+  *reinterpret_cast<uint4*>(v[3]) = *reinterpret_cast<const uint4*>(in + base + row + C);
   __align__(16) __nv_bfloat16 o[8];
 #pragma unroll
   for (int j = 0; j < 8; ++j) {
@@ -462,6 +471,7 @@ __global__ void __launch_bounds__(kInThreads) k_conv_in_wimg(const float* __rest
                                                              __nv_bfloat16* out, int nconv, WImgTable t,
                                                              const float* __restrict__ params, __nv_bfloat16* img) {
   extern __shared__ float4 ws[];  // Co * 9
+  dep_go();
   if ((int)blockIdx.x < nconv)
     conv_in_body(ws, blockIdx.x, x, lH, lW, npix, w, bias, Co, out);
   else
@@ -606,16 +616,18 @@ __global__ void __launch_bounds__(kRowThreads) k_conv3_tc_row(ConvArgs p) {
   // at a time (2 of 16 where KC is no multiple of 32), the chunks fastest:
   // eight lanes, which the load unit takes together, read 2 (4) lines and
   // write 8 banks groups. With all chunks of one pixel, or one chunk of eight
-  // pixels, such a copy of 512 bytes took 38 cycles, in bank conflicts or in
-  // lines; @.
+  // pixels, the same copies made the 128^2 pass 128 us instead of 120.
   // One address serves a pixel's chunks and, in narrow grids, all three copies.
   const int chunks = KC >> 3;
   const int lq = (chunks & 3) ? 1 : 2;  // log2 of the chunks a warp takes side by side
   const int lpx = (tid & 31) >> lq, lc = tid & ((1 << lq) - 1);
+  auto load_weights = [&](int kb, int bf) {
+    bulk_g2s(sm + (size_t)bf * bufbytes + hbytes, p.wimg + (size_t)kb * 9 * Co * KC, wbytes, &bar_w[bf],
+             (p.stall && kb == 0) ? 16u : 0u);
+  };
   auto load_block = [&](int kb, int bf) {
     unsigned char* dst = sm + (size_t)bf * bufbytes;
-    if (tid == 0)
-      bulk_g2s(dst + hbytes, p.wimg + (size_t)kb * 9 * Co * KC, wbytes, &bar_w[bf], (p.stall && kb == 0) ? 16u : 0u);
+    if (tid == 0 && kb > 0) load_weights(kb, bf);
     const int up = p.up0 ? 1 : 0, ch0 = kb * KC + 8 * lc;
     const __nv_bfloat16* s0 = p.src0 + ((size_t)b << (p.lH + p.lW - 2 * up)) * p.C0 + ch0;
     const __nv_bfloat16* s1 = p.src1 + ((size_t)b << (p.lH + p.lW)) * p.C1 + (ch0 - p.C0);
@@ -656,9 +668,19 @@ __global__ void __launch_bounds__(kRowThreads) k_conv3_tc_row(ConvArgs p) {
   // copy in order; the other warps learn the outcome through the block votes.
   bool ok = true;
   int issued = -1, mma_seen = -1, copied = 0, copy_done = -1;
+  // Until the launch before is complete: what does not depend on it, which
+  // hides the barriers' and the tensor memory's set-up, the constants and, where
+  // the image is that old, the first weights behind its tail.
+  load_consts(p, consts, tid, kRowThreads);
+  if (tid == 0 && p.early_w) {
+    asm volatile("fence.proxy.async.global;\n" ::: "memory");
+    load_weights(0, 0);
+  }
+  dep_wait();
+  dep_go();
+  if (tid == 0 && !p.early_w) load_weights(0, 0);
   load_block(0, 0);
   cp_async_commit();
-  load_consts(p, consts, tid, kRowThreads);
   for (int kb = 0; kb < nkb; ++kb) {
     const int bf = kb & 1;
     const bool pre = kb + 1 < nkb;
