@@ -671,7 +671,11 @@ __global__ void __launch_bounds__(kRowThreads) k_conv3_tc_row(ConvArgs p) {
   // Until the launch before is complete: what does not depend on it, which
   // hides the barriers' and the tensor memory's set-up, the constants and, where
   // the image is that old, the first weights behind its tail.
-  load_consts(p, consts, tid, kRowThreads);
+  float kb0 = 0.f, kh0 = 0.f;  // a thread's bias and head weight (Co is at most its 256 threads), stored below
+  if (tid < Co) {
+    kb0 = __ldg(p.bias + tid);
+    if (p.head_w) kh0 = __ldg(p.head_w + tid);
+  }
   if (tid == 0 && p.early_w) {
     asm volatile("fence.proxy.async.global;\n" ::: "memory");
     load_weights(0, 0);
@@ -681,6 +685,10 @@ __global__ void __launch_bounds__(kRowThreads) k_conv3_tc_row(ConvArgs p) {
   if (tid == 0 && !p.early_w) load_weights(0, 0);
   load_block(0, 0);
   cp_async_commit();
+  if (tid < Co) {
+    consts.bias[tid] = kb0;
+    consts.head[tid] = kh0;
+  }
   for (int kb = 0; kb < nkb; ++kb) {
     const int bf = kb & 1;
     const bool pre = kb + 1 < nkb;
