@@ -295,30 +295,31 @@ void build_tables(sgn_ctx* ctx) {
   std::vector<double> k2x(kx), k2y(ky);
   for (double& k : k2x) k *= two_pi / G.Lx;
   for (double& k : k2y) k *= two_pi / G.Ly;
-  auto upload = [&](const std::vector<double>& v) {
-    double* d = dalloc<double>(ctx, v.size());
-    CK(cudaMemcpy(d, v.data(), v.size() * sizeof(double), cudaMemcpyHostToDevice));
-    return d;
-  };
   std::vector<double> gkx(kx), gky(ky), kx2(kx), ky2(ky);
   for (double& k : gkx) k *= ctx->g;
   for (double& k : gky) k *= ctx->g;
   for (double& k : kx2) k *= k;
   for (double& k : ky2) k *= k;
-  ctx->tb.gkx = upload(gkx);
-  ctx->tb.gky = upload(gky);
-  ctx->tb.kx2 = upload(kx2);
-  ctx->tb.ky2 = upload(ky2);
+  // the FP64 tables of the wavenumbers side by side, in one allocation and one copy
+  std::vector<double> all;
+  const std::pair<const std::vector<double>*, double**> parts[] = {
+      {&kx, &ctx->tb.kx},   {&ky, &ctx->tb.ky},   {&k2x, &ctx->tb.k2x}, {&k2y, &ctx->tb.k2y},
+      {&gkx, &ctx->tb.gkx}, {&gky, &ctx->tb.gky}, {&kx2, &ctx->tb.kx2}, {&ky2, &ctx->tb.ky2}};
+  auto padded = [](const std::vector<double>& v) { return (v.size() + 31) & ~(size_t)31; };  // 256-byte starts
+  for (const auto& p : parts) {
+    all.insert(all.end(), p.first->begin(), p.first->end());
+    all.resize((all.size() + 31) & ~(size_t)31, 0.0);
+  }
+  double* at = dalloc<double>(ctx, all.size());
+  CK(cudaMemcpy(at, all.data(), all.size() * sizeof(double), cudaMemcpyHostToDevice));
+  for (const auto& p : parts) {
+    *p.second = at;
+    at += padded(*p.first);
+  }
   ctx->tb.twx = dalloc<cpx<fx>>(ctx, qx.size());
   ctx->tb.twy = dalloc<cpx<fx>>(ctx, qy.size());
-  ctx->tb.k2x = upload(k2x);
-  ctx->tb.k2y = upload(k2y);
-  ctx->tb.kx = dalloc<double>(ctx, G.Nxh);
-  ctx->tb.ky = dalloc<double>(ctx, G.Ny);
   CK(cudaMemcpy(ctx->tb.twx, qx.data(), qx.size() * sizeof(qx[0]), cudaMemcpyHostToDevice));
   CK(cudaMemcpy(ctx->tb.twy, qy.data(), qy.size() * sizeof(qy[0]), cudaMemcpyHostToDevice));
-  CK(cudaMemcpy(ctx->tb.kx, kx.data(), G.Nxh * sizeof(double), cudaMemcpyHostToDevice));
-  CK(cudaMemcpy(ctx->tb.ky, ky.data(), G.Ny * sizeof(double), cudaMemcpyHostToDevice));
   if (ctx->opt.precision >= 2) {
     // double-float copies: nearest FP32 pair of each FP64 entry
     std::vector<CDF> dx(tx.size()), dy(ty.size());
