@@ -1,9 +1,10 @@
 // sgn_spectral.cuh - spectral passes of the SGN hot path (Section 3).
 //
 // Templates only (plus a few host functions, each compiled in one unit): the
-// kernels are instantiated per arithmetic in sgn_spectral.cu (FP64 and the
-// shared host code), sgn_spectral_f32.cu and sgn_spectral_df.cu, which the
-// build compiles in parallel.
+// kernels are instantiated per arithmetic in sgn_spectral_f32.cu,
+// sgn_spectral_df.cu and sgn_spectral_df_rhs.cu, which the build compiles in
+// parallel with sgn_spectral.cu: the shared host code and the FP64 passes, whose
+// kernels run in fixed point (sgn_fx.cuh).
 //
 // Every 2D transform is split into an x-pass over row PAIRS and a y-pass over
 // column tiles of the half spectrum [Ny][ldS]:
@@ -311,16 +312,15 @@ __global__ void k_coef_phys(Geom G, const double* __restrict__ hp, T* h, T* cr, 
 
 // ---------------------------------------------------------- fused matvec x
 
-// Resident 256-thread blocks per SM the x-passes ask the compiler for: the
-// FP32 passes are latency bound and need the warps; the FP64 ones are
-// FP64-issue bound and keep their registers.
+// Resident 256-thread blocks per SM the x-passes ask the compiler for (FP32:
+// latency bound, they need the warps; double-float: 80 and 128 registers).
 // At 4096 points (LN = 12) a row pair takes 512 threads: one block per SM.
 template <int LN>
 constexpr int xpass_threads() { return LN == 12 ? 512 : 256; }
-template <typename T, int LN>
-constexpr int mv_min_blocks() { return LN == 12 ? 1 : ((sizeof(T) == 4 || std::is_same<T, dfl>::value) ? 3 : 2); }
-template <typename T, int LN>
-constexpr int rhs_min_blocks() { return LN == 12 ? 1 : ((sizeof(T) == 4 || std::is_same<T, dfl>::value) ? 2 : 1); }
+template <int LN>
+constexpr int mv_min_blocks() { return LN == 12 ? 1 : 3; }
+template <int LN>
+constexpr int rhs_min_blocks() { return LN == 12 ? 1 : 2; }
 // shared-memory elements per row pair of the fused RHS x-pass beyond its
 // transform buffer: the double-float pass keeps its accumulators QX, QY there
 // (8 slots per thread each)
@@ -340,7 +340,7 @@ __host__ __device__ constexpr int rhs_acc_elems(int N) { return std::is_same<T, 
 __host__ __device__ constexpr int mv_stash_elems(int N) { return 10 * (N >> 3); }
 
 template <typename T, int LN = 0, int PLAN = 0>
-__global__ void __launch_bounds__(xpass_threads<LN>(), mv_min_blocks<T, LN>()) k_mv_x(Geom G, const cpx<T>* __restrict__ tw, const T* __restrict__ kx,
+__global__ void __launch_bounds__(xpass_threads<LN>(), mv_min_blocks<LN>()) k_mv_x(Geom G, const cpx<T>* __restrict__ tw, const T* __restrict__ kx,
                                                const cpx<T>* S, const cpx<T>* Sy, const T* __restrict__ cr,
                                                const T* __restrict__ cc, cpx<T>* Cout, cpx<T>* Byout) {
   const XLayout L = x_layout<LN>(G);
@@ -426,7 +426,7 @@ template <typename T>
 constexpr bool rhs_lin_split() { return std::is_same<T, float>::value; }
 
 template <typename T, int LN = 0, int PLAN = 0>
-__global__ void __launch_bounds__(xpass_threads<LN>(), rhs_min_blocks<T, LN>()) k_rhs_x(Geom G, const cpx<T>* __restrict__ tw, const T* __restrict__ kx,
+__global__ void __launch_bounds__(xpass_threads<LN>(), rhs_min_blocks<LN>()) k_rhs_x(Geom G, const cpx<T>* __restrict__ tw, const T* __restrict__ kx,
                                                 const cpx<T>* Vx, const cpx<T>* Vy, const cpx<T>* S,
                                                 const cpx<T>* Sy, const T* __restrict__ hh,
                                                 const T* __restrict__ cr, T g, cpx<T>* Cq, cpx<T>* Qy,
@@ -712,12 +712,12 @@ __host__ __device__ constexpr size_t ystage_offset(int lN, int lC) {
 // first input's raw values in shared memory instead spilled 244 bytes at the
 // 64 registers of the FP32 pass); the y-forward passes stage every input after
 // the first; the RHS y-inverse forms i ky sigma_hat from a staged copy of
-// sigma_hat and, in FP64 below 4096 points, also stages v_y and sigma_hat (the
-// FP32 one measured 117 against 107 us with them staged: 196 KB of shared
-// memory leave little L1; FP64 at 4096 has no room for them; the double-float
-// one transforms one input at a time at three blocks per SM instead)
+// sigma_hat (with v_y and sigma_hat staged too, the FP32 one measured 117
+// against 107 us: 196 KB of shared memory leave little L1; the double-float one
+// transforms one input at a time at three blocks per SM)
 constexpr int FL_MV_INV = yf_pf(1);
 constexpr int FL_MV_FWD = yf_pf(1);
+constexpr int FL_RHS_INV = yf_dup(3);
 constexpr int FL_RHS_FWD = yf_pf(1) | yf_pf(2);
 // the double-float forward passes stage nothing: they transform one input at
 // a time and keep each finished transform in the thread's own shared-memory
@@ -735,11 +735,6 @@ constexpr int fl_rhs_fwd() { return y_stashed<T, false, 3>() ? 0 : FL_RHS_FWD; }
 template <typename T, bool INV, int NIN>
 __host__ __device__ constexpr int ystash_bytes() {
   return y_stashed<T, INV, NIN>() ? (NIN - 1) * 8 * (int)sizeof(cpx<T>) : 0;
-}
-template <typename T, int LN>
-constexpr int fl_rhs_inv() {
-  return (sizeof(T) == 4 || LN == 12 || std::is_same<T, dfl>::value) ? yf_dup(3)
-                                                                      : (yf_pf(1) | yf_pf(2) | yf_dup(3));
 }
 
 template <typename E>
@@ -1431,7 +1426,7 @@ static void set_attrs_ln_plan() {
     set_smem<T>((const void*)k_ypass_tma<T, true, 2, EpiStore<T, 2>, L, FL_MV_INV_TMA, P>);
     set_smem<T>((const void*)k_ypass_tma<T, false, 2, EpiMatvec<T, T>, L, FL_MV_FWD_TMA, P>);
   }
-  set_smem<T>((const void*)ypass_fn<T, true, 4, EpiStore<T, 4>, double, L, fl_rhs_inv<T, L>(), P>());
+  set_smem<T>((const void*)ypass_fn<T, true, 4, EpiStore<T, 4>, double, L, FL_RHS_INV, P>());
   set_smem<T>((const void*)ypass_fn<T, false, 3, EpiK<T>, T, L, fl_rhs_fwd<T>(), P>());
 }
 
@@ -1451,10 +1446,10 @@ static void set_attrs_plan() {
     set_smem<T>((const void*)k_ypass_tma<T, true, 2, EpiStore<T, 2>, 0, FL_MV_INV_TMA, P>);
     set_smem<T>((const void*)k_ypass_tma<T, false, 2, EpiMatvec<T, T>, 0, FL_MV_FWD_TMA, P>);
   }
-  set_smem<T>((const void*)ypass_fn<T, true, 4, EpiStore<T, 4>, T, 0, fl_rhs_inv<T, 0>(), P>());
+  set_smem<T>((const void*)ypass_fn<T, true, 4, EpiStore<T, 4>, T, 0, FL_RHS_INV, P>());
   set_smem<T>((const void*)ypass_fn<T, false, 2, EpiMatvec<T>, T, 0, fl_mv_fwd<T>(), P>());
   set_smem<T>((const void*)ypass_fn<T, false, 3, EpiK<T>, T, 0, fl_rhs_fwd<T>(), P>());
-  set_smem<T>((const void*)ypass_fn<T, true, 4, EpiStore<T, 4>, double, 0, fl_rhs_inv<T, 0>(), P>());
+  set_smem<T>((const void*)ypass_fn<T, true, 4, EpiStore<T, 4>, double, 0, FL_RHS_INV, P>());
 }
 
 template <typename T>
@@ -1842,11 +1837,11 @@ template <int P>
 static void set_attrs_df_rhs_plan() {
   typedef dfl T;
   set_smem<T>((const void*)k_rhs_x<T, 0, P>);
-  set_smem<T>((const void*)ypass_fn<T, true, 4, EpiStore<T, 4>, double, 0, fl_rhs_inv<T, 0>(), P>());
+  set_smem<T>((const void*)ypass_fn<T, true, 4, EpiStore<T, 4>, double, 0, FL_RHS_INV, P>());
   set_smem<T>((const void*)ypass_fn<T, false, 3, EpiK<T>, T, 0, fl_rhs_fwd<T>(), P>());
   if constexpr (P == 0) {  // 4096 points: one plan
     set_smem<T>((const void*)k_rhs_x<T, 12, P>);
-    set_smem<T>((const void*)ypass_fn<T, true, 4, EpiStore<T, 4>, double, 12, fl_rhs_inv<T, 12>(), P>());
+    set_smem<T>((const void*)ypass_fn<T, true, 4, EpiStore<T, 4>, double, 12, FL_RHS_INV, P>());
     set_smem<T>((const void*)ypass_fn<T, false, 3, EpiK<T>, T, 12, fl_rhs_fwd<T>(), P>());
   }
 }
@@ -1917,7 +1912,7 @@ cudaError_t launch_rhs(const Geom& G, const Tables<T>& tb, const Tables<S>& tbs,
   y_config<T, true, 4>(G, grid, block, smem, 0, ex.tpb(tune_type<T>(), TP_RHS_YINV), &bi);
   dispatch_ln<T>(bi ? G.lNy : 0, [&](auto ln) {
     constexpr int L = decltype(ln)::value;
-    constexpr int FL = fl_rhs_inv<T, L>();
+    constexpr int FL = FL_RHS_INV;
     y_config<T, true, 4>(G, grid, block, smem, ystage_bytes<T, S, FL>(4), ex.tpb(tune_type<T>(), TP_RHS_YINV));
     YIn<T, 4, S> yi{};
     yi.src[0] = U[1];
