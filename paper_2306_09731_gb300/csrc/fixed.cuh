@@ -341,8 +341,15 @@ __device__ __forceinline__ double scale_exp(double x, int e) {
 struct FxTw {
   long long c, s;
 };
+// on the host static, or each call would copy its 1 KB to the stack (55 ns an entry of a solver's tables, 0.2 ms at
+// 1024 x 256); device functions cannot have static variables of this kind
+#ifdef __CUDA_ARCH__
+#define FX_TABLE constexpr
+#else
+#define FX_TABLE static constexpr
+#endif
 __host__ __device__ inline FxTw fx_tw_hi(int a) {
-  constexpr FxTw t[64] = {
+  FX_TABLE FxTw t[64] = {
       {4611686018427387904ll, 0ll}, {4589479489746651964ll, -452024275624069880ll},
       {4523073764714963030ll, -899695310372275547ll}, {4413108366765438139ll, -1338701787458110889ll},
       {4260642322793532497ll, -1764815834521887442ll}, {4067143964149113252ll, -2173933740352748318ll},
@@ -379,7 +386,7 @@ __host__ __device__ inline FxTw fx_tw_hi(int a) {
   return t[a];
 }
 __host__ __device__ inline FxTw fx_tw_lo(int b) {
-  constexpr FxTw t[64] = {
+  FX_TABLE FxTw t[64] = {
       {4611686018427387904ll, 0ll}, {4611680592556051597ll, -7074234977634094ll},
       {4611664314954810277ll, -14148453308909941ll}, {4611637185661966712ll, -21222638347508465ll},
       {4611599204741358747ll, -28296773447188932ll}, {4611550372282359158ll, -35370841961828118ll},
@@ -415,6 +422,7 @@ __host__ __device__ inline FxTw fx_tw_lo(int b) {
   };
   return t[b];
 }
+#undef FX_TABLE
 __host__ __device__ inline long long fx_pack_q63(long long q62) {
   // 2 q62 as limbs; the constants' extremes are -2^62 (exactly -1) and below +2^62
   const long long w = (long long)((u64)q62 * 2ull);

@@ -277,7 +277,11 @@ std::vector<cpx<fx>> staged_twiddles_fx(int N, int lN) {
 
 void build_tables(sgn_ctx* ctx) {
   const Geom& G = ctx->G;
-  const std::vector<C64> tx = staged_twiddles(G.Nx, G.lNx), ty = staged_twiddles(G.Ny, G.lNy);
+  std::vector<C64> tx, ty;  // the FP64 passes take theirs in fixed point
+  if (ctx->opt.precision >= 1) {
+    tx = staged_twiddles(G.Nx, G.lNx);
+    ty = staged_twiddles(G.Ny, G.lNy);
+  }
   const double two_pi = 6.283185307179586476925286766559;
   std::vector<double> kx(G.Nxh), ky(G.Ny);
   for (int k = 0; k < G.Nxh; ++k) kx[k] = (k == G.Nx / 2) ? 0.0 : two_pi * k / G.Lx;
