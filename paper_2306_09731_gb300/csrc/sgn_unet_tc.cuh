@@ -5,7 +5,8 @@
 // pixels, the GEMM D[128][Co] = sum over the nine taps t of
 // A_t[128][Ci] B_t[Ci][Co], where row m of A_t holds the Ci channels of the
 // input pixel at (y + ty - 1, x + tx - 1) (wrapped) and B_t the weights of tap
-// t. One CTA of 128 threads computes one tile:
+// t. One CTA of 128 threads (256 in the row kernel, which stages its input once
+// per channel block, below) computes one tile:
 //   * the accumulator D lives in tensor memory (TMEM lane m = pixel m, one
 //     32-bit column per output channel), allocated by warp 0;
 //   * the K loop runs over (tap, channel block) steps through three
@@ -501,6 +502,14 @@ namespace unet_tc {
 // and stored with row stride exactly W. Output pixel m of the tile then reads
 // tap (ky, kx) at position m + ky W of copy kx: again 128 consecutive 16-byte
 // positions, one descriptor per tap.
+//
+// At batch 1 a layer has 2 to 128 tiles, and a tile is one serial chain: halo
+// copies, MMA issue, epilogue. At 128^2 (471,873 parameters) a channel block of
+// 32 copies its halo in 2400 to 3400 cycles (38 per warp copy of 512 bytes, the
+// rate of these copies), is issued in 1050 to 1130, and the epilogue takes 700
+// to 1900. Kept: 256 threads, division-free copies, unrolled issue, staged
+// constants, dependent launches: 201 -> 85 us a pass, 2.10 -> 1.46 ms at 256^2
+// and batch 32. Tensor pipe 9 to 15% active on the large grids.
 constexpr int kHaloPos = 3 * (kM + 2);
 // positions per chunk of one halo copy, and the copies
 __host__ __device__ constexpr int halo_pos(int W) { return W >= kM ? kHaloPos : kM + 2 * W; }
