@@ -72,8 +72,9 @@ sgn_status sgn_unet_get_params(sgn_unet_t net, float* params);
 sgn_status sgn_unet_get_grads(sgn_unet_t net, float* grads);
 
 /* out[B][1][n][n] = net(in[B][4][n][n]), 1 <= B <= max_batch; out may be
- * NULL. Keeps the activations, and the pointer in (which must stay valid), for
- * sgn_unet_backward. */
+ * NULL. in may start at any element of an array (it needs no alignment beyond
+ * float's own). Keeps the activations, and the pointer in (which must stay
+ * valid), for sgn_unet_backward. */
 sgn_status sgn_unet_forward(sgn_unet_t net, const float* in, float* out, int batch);
 
 /* out[B][1][n][n] = net(in[B][4][n][n]) on the tensor cores, 1 <= B <=

@@ -66,8 +66,13 @@ __device__ __forceinline__ __nv_bfloat16 tof<__nv_bfloat16>(float v) {
 // TY = min(H, 128 / TX, 16).
 template <int PX>
 constexpr int conv_cck() { return PX == 8 ? 4 : 8; }  // input channels per stage
-// four consecutive elements as floats
-__device__ __forceinline__ float4 load4(const float* p) { return *reinterpret_cast<const float4*>(p); }
+// four consecutive elements as floats (VEC = false: of any address)
+template <bool VEC = true>
+__device__ __forceinline__ float4 load4(const float* p) {
+  if constexpr (VEC) return *reinterpret_cast<const float4*>(p);
+  return make_float4(p[0], p[1], p[2], p[3]);
+}
+template <bool VEC = true>
 __device__ __forceinline__ float4 load4(const __nv_bfloat16* p) {
   const uint2 r = *reinterpret_cast<const uint2*>(p);
   return make_float4(__uint_as_float(r.x << 16), __uint_as_float(r.x & 0xffff0000u), __uint_as_float(r.y << 16),
@@ -87,8 +92,9 @@ __device__ __forceinline__ void store4(__nv_bfloat16* p, float a, float b, float
 
 // Stages rows [0, nrow) of a tile: row r = (channel r / RPC, line r % RPC) at
 // dst + dsto(r), tw interior pixels from element 4 on and the halo at 3 and
-// tw + 4. 16-byte (8-byte) fetches, U in flight per thread.
-template <int U, typename TI, class Src, class Dst>
+// tw + 4. 16-byte (8-byte) fetches, U in flight per thread; VEC = false: element by
+// element, for a caller's input that starts at no 16-byte boundary.
+template <int U, bool VEC, typename TI, class Src, class Dst>
 __device__ __forceinline__ void stage_rows(int nrow, int ltw, int tid, int nthr, int x0, int W, Src src, Dst dst) {
   const int lv = ltw - 2, nvec = nrow << lv;  // 4-pixel vectors per row: 2^lv
   for (int base = 0; base < nvec; base += U * nthr) {
@@ -96,7 +102,7 @@ __device__ __forceinline__ void stage_rows(int nrow, int ltw, int tid, int nthr,
 #pragma unroll
     for (int u = 0; u < U; ++u) {
       const int i = base + u * nthr + tid;
-      if (i < nvec) q[u] = load4(src(i >> lv) + x0 + 4 * (i & ((1 << lv) - 1)));
+      if (i < nvec) q[u] = load4<VEC>(src(i >> lv) + x0 + 4 * (i & ((1 << lv) - 1)));
     }
 #pragma unroll
     for (int u = 0; u < U; ++u) {
@@ -120,7 +126,7 @@ __device__ __forceinline__ void stage_rows(int nrow, int ltw, int tid, int nthr,
   }
 }
 
-template <typename TI, typename TO, bool TR, int COT, int PX>
+template <typename TI, typename TO, bool TR, int COT, int PX, bool VEC>
 __global__ void __launch_bounds__(128) k_conv3(const TI* __restrict__ in, size_t ibs, int Ci, TO* out, size_t obs,
                                                const float* __restrict__ w, const float* __restrict__ bias, int Cw,
                                                int H, int W, int lTX, int relu) {
@@ -146,7 +152,7 @@ __global__ void __launch_bounds__(128) k_conv3(const TI* __restrict__ in, size_t
   for (int c0 = 0; c0 < Ci; c0 += CCK) {
     const int nc = min(CCK, Ci - c0);
     if (c0) __syncthreads();
-    stage_rows<9, TI>(
+    stage_rows<9, VEC, TI>(
         nc * RPC, ltw, tid, blockDim.x, x0, W,
         [&](int r) {
           const int ci = (int)((unsigned)r * inv >> 16), ly = r - ci * RPC;
@@ -243,7 +249,7 @@ __host__ __device__ inline int dw_in_stride(int R, int CW) {
   const int n = (R + 2) * dw_row_stride(CW);
   return (n + 27) / 32 * 32 + 4;
 }
-template <typename TI>
+template <typename TI, bool VEC>
 __global__ void __launch_bounds__(128, 4) k_conv3_dw(const TI* __restrict__ in, size_t ibs, int Ci,
                                                   const float* __restrict__ dp, size_t dbs, int Co, int H, int W,
                                                   int B, float* part) {
@@ -272,7 +278,7 @@ __global__ void __launch_bounds__(128, 4) k_conv3_dw(const TI* __restrict__ in, 
     const int b = ch / ((H / R) * cpr), rem = ch - b * (H / R) * cpr;
     const int y0 = rem / cpr * R, x0 = (rem % cpr) * CW;
     __syncthreads();
-    stage_rows<9, TI>(
+    stage_rows<9, VEC, TI>(
         nin * (R + 2), lCW, tid, 128, x0, W,
         [&](int r) {
           const int c = (int)((unsigned)r * inv >> 16), ly = r - c * (R + 2);
@@ -668,7 +674,7 @@ void init_params(sgn_unet_ctx* net, unsigned long long seed) {
   UCK(cudaMemset(net->grads, 0, sizeof(float) * (size_t)net->P));
 }
 
-template <typename TI, typename TO, bool TR, int COT, int PX>
+template <typename TI, typename TO, bool TR, bool VEC, int COT, int PX>
 void conv3_tile(sgn_unet_ctx* net, const TI* in, size_t ibs, int Ci, TO* out, size_t obs, int Co, const float* w,
                 const float* bias, int Cw, int H, int B, bool relu) {
   int lTX = 0;
@@ -680,40 +686,40 @@ void conv3_tile(sgn_unet_ctx* net, const TI* in, size_t ibs, int Ci, TO* out, si
   const dim3 grid((unsigned)((H / (PX * TX)) * (H / TY)), Co / COT, B);
   const size_t smem =
       sizeof(float) * conv_cck<PX>() * ((size_t)(TY + 2) * (PX * TX + 8) + 9 * (size_t)COT);
-  k_conv3<TI, TO, TR, COT, PX><<<grid, TX * TY, smem, net->stream>>>(in, ibs, Ci, out, obs, w, bias, Cw, H, H, lTX,
+  k_conv3<TI, TO, TR, COT, PX, VEC><<<grid, TX * TY, smem, net->stream>>>(in, ibs, Ci, out, obs, w, bias, Cw, H, H, lTX,
                                                                     relu ? 1 : 0);
   UCK(cudaGetLastError());
 }
 // Ci input and Co output channels (Co a multiple of 16): 8 pixels x 8 channels
 // a thread where that leaves two blocks per SM (64 x 16 pixels each), else 4 x 8
-template <typename TI, typename TO, bool TR>
+template <typename TI, typename TO, bool TR, bool VEC>
 void conv3_launch(sgn_unet_ctx* net, const TI* in, size_t ibs, int Ci, TO* out, size_t obs, int Co, const float* w,
                   const float* bias, int Cw, int H, int B, bool relu) {
   if (H >= 64 && (long long)(H / 64) * (H / 16) * (Co / 8) * B >= 256)
-    conv3_tile<TI, TO, TR, 8, 8>(net, in, ibs, Ci, out, obs, Co, w, bias, Cw, H, B, relu);
+    conv3_tile<TI, TO, TR, VEC, 8, 8>(net, in, ibs, Ci, out, obs, Co, w, bias, Cw, H, B, relu);
   else
-    conv3_tile<TI, TO, TR, 8, 4>(net, in, ibs, Ci, out, obs, Co, w, bias, Cw, H, B, relu);
+    conv3_tile<TI, TO, TR, VEC, 8, 4>(net, in, ibs, Ci, out, obs, Co, w, bias, Cw, H, B, relu);
 }
-template <typename TI, typename TO>
+template <typename TI, typename TO, bool VEC = true>
 void conv3(sgn_unet_ctx* net, const TI* in, size_t ibs, int li, TO* out, size_t obs, int H, int B, bool relu) {
   const Layer& l = net->L[li];
-  conv3_launch<TI, TO, false>(net, in, ibs, l.Ci, out, obs, l.Co, net->params + l.woff, net->params + l.boff, l.Ci, H,
+  conv3_launch<TI, TO, false, VEC>(net, in, ibs, l.Ci, out, obs, l.Co, net->params + l.woff, net->params + l.boff, l.Ci, H,
                               B, relu);
 }
 // gradient with respect to the layer input (channels Ci) from dp (channels Co)
 void conv3_dx(sgn_unet_ctx* net, const float* dp, size_t dbs, int li, float* dx, size_t xbs, int H, int B) {
   const Layer& l = net->L[li];
-  conv3_launch<float, float, true>(net, dp, dbs, l.Co, dx, xbs, l.Ci, net->params + l.woff, nullptr, l.Ci, H, B,
+  conv3_launch<float, float, true, true>(net, dp, dbs, l.Co, dx, xbs, l.Ci, net->params + l.woff, nullptr, l.Ci, H, B,
                                    false);
 }
-template <typename TI>
+template <typename TI, bool VEC = true>
 void conv3_dw(sgn_unet_ctx* net, const TI* in, size_t ibs, const float* dp, size_t dbs, int li, int H, int B) {
   const Layer& l = net->L[li];
   int R, CW;
   dw_chunk(H, H, &R, &CW);
   const int splits = dw_splits(l.Ci, l.Co, H, H, B), n = l.Co * l.Ci * 9 + l.Co;
   const size_t smem = sizeof(float) * (16 * (size_t)dw_in_stride(R, CW) + (size_t)R * CW * 36);
-  k_conv3_dw<TI><<<dim3((l.Ci + 15) / 16, (l.Co + 31) / 32, splits), 128, smem, net->stream>>>(
+  k_conv3_dw<TI, VEC><<<dim3((l.Ci + 15) / 16, (l.Co + 31) / 32, splits), 128, smem, net->stream>>>(
       in, ibs, l.Ci, dp, dbs, l.Co, H, H, B, net->part);
   UCK(cudaGetLastError());
   k_part_sum<<<blocks_for(n, 32), dim3(32, 8), 0, net->stream>>>(net->part, n, splits, net->grads + l.woff);
@@ -726,6 +732,10 @@ void relu_bwd(sgn_unet_ctx* net, const T* act, size_t abs_, float* g, size_t gbs
   k_relu_bwd<T><<<blocks_for(n), 256, 0, net->stream>>>(act, abs_, g, gbs, extra, ebs, C, H * H, B);
   UCK(cudaGetLastError());
 }
+
+// Whether the vector fetches of stage_rows may read p: a caller's input, the one
+// tensor that the handle does not lay out itself, may start at any element.
+inline bool aligned16(const void* p) { return ((uintptr_t)p & 15u) == 0; }
 
 inline size_t npix(const sgn_unet_ctx* net, int l) { return (size_t)(net->n >> l) * (size_t)(net->n >> l); }
 
@@ -740,8 +750,10 @@ void forward_impl(sgn_unet_ctx* net, const float* in, float* out, int B) {
     T* A = (T*)net->A[l];
     T* S = (T*)net->CAT[l] + (size_t)w[l + 1] * N;  // s_l lives in CAT[l] after the upsampled channels
     const size_t cs = (size_t)(w[l + 1] + w[l]) * N;
-    if (l == 0)
+    if (l == 0 && aligned16(in))
       conv3<float, T>(net, in, 4 * N, iE(0), A, (size_t)w[0] * N, H, B, true);
+    else if (l == 0)
+      conv3<float, T, false>(net, in, 4 * N, iE(0), A, (size_t)w[0] * N, H, B, true);
     else
       conv3<T, T>(net, (const T*)net->Q[l - 1], (size_t)w[l - 1] * N, iE(l), A, (size_t)w[l] * N, H, B, true);
     conv3<T, T>(net, A, (size_t)w[l] * N, iS(l), S, cs, H, B, true);
@@ -839,8 +851,10 @@ void backward_impl(sgn_unet_ctx* net, const float* target, double* loss) {
     conv3_dw<T>(net, (const T*)net->A[l], bs, g0, bs, iS(l), H, B);
     conv3_dx(net, g0, bs, iS(l), g1, bs, H, B);
     relu_bwd<T>(net, (const T*)net->A[l], bs, g1, bs, nullptr, 0, w[l], H, B);
-    if (l == 0) {
+    if (l == 0 && aligned16(net->lastIn)) {
       conv3_dw<float>(net, net->lastIn, 4 * N, g1, bs, iE(0), H, B);
+    } else if (l == 0) {
+      conv3_dw<float, false>(net, net->lastIn, 4 * N, g1, bs, iE(0), H, B);
     } else {
       conv3_dw<T>(net, (const T*)net->Q[l - 1], (size_t)w[l - 1] * N, g1, bs, iE(l), H, B);
       conv3_dx(net, g1, bs, iE(l), g0, (size_t)w[l - 1] * N, H, B);
