@@ -515,16 +515,6 @@ void coef_from_spectral(sgn_ctx* ctx, const C64* hh) {
                             EX(ctx)));
 }
 
-// Whether Arnoldi steps on vectors of type T take the one-launch form: the FP64
-// ones, whose second pass nearly always runs (four kernels to one). The FP32
-// step has two to save, a wash for one solver at a time, and the cooperative
-// launches of an ensemble's members keep one another waiting (12 members: 42 ms
-// with two kernels, 58 with one).
-template <typename T>
-bool use_ortho(const sgn_ctx* ctx) {
-  return ctx->ortho && sizeof(T) == 8;
-}
-
 // One Arnoldi step of the inner or outer GMRES on the basis V (type T):
 // w = A V_j, classical Gram-Schmidt with DGKS reorthogonalisation, Givens.
 // Returns the residual estimate and H[j+1][j] through the readback.
@@ -541,15 +531,20 @@ void arnoldi_step(sgn_ctx* ctx, const Tables<T>& tb, const T* cr, const T* cc, c
   // test; the FP32 inner solve of precision 1 runs one classical Gram-Schmidt
   // pass: it only has to reduce its residual by 1e-6 and the FP64 refinement
   // checks the result (measured: same iteration and refinement counts, 4% faster)
-  const bool dgks = sizeof(T) == 8;
+  constexpr bool dgks = sizeof(T) == 8;
   // the basis is stored unnormalised (GmresDev::vscl): the update writes the
   // next basis vector itself, with no scaling pass
   const double* vscl = ctx->gst->vscl;
-  if (use_ortho<T>(ctx)) {
-    CK(launch_ortho<T>(G, V, vs, w, ctx->partials, ctx->gst, j, dgks, ctx->bar_count, ctx->rb_dev, ctx->flags,
-                       EX(ctx)));
-    sync_read(ctx);
-    return;
+  // In one launch: the FP64 step, whose second pass nearly always runs (four
+  // kernels to one). The FP32 step has two to save, a wash for one solver at a
+  // time, and the cooperative launches of an ensemble's members keep one another
+  // waiting (12 members: 42 ms with two kernels, 58 with one).
+  if constexpr (dgks) {
+    if (ctx->ortho) {
+      CK(launch_ortho(G, V, vs, w, ctx->partials, ctx->gst, j, ctx->bar_count, ctx->rb_dev, ctx->flags, EX(ctx)));
+      sync_read(ctx);
+      return;
+    }
   }
   CK(launch_dots<T>(G, V, vs, nv, w, ctx->partials, nullptr, ctx->gst->h1, cnt + 0, EX(ctx), nullptr, vscl));
   CK(launch_cgs_update<T>(G, V, vs, nv, ctx->gst->h1, w, ctx->partials, nullptr, ctx->gst, j, dgks ? 1 : 3,
@@ -1019,13 +1014,15 @@ void graph_arnoldi(sgn_ctx* ctx, const Tables<T>& tb, const T* cr, const T* cc, 
   const int* jd = &ctx->gst->j;
   const int* gate = &ctx->gst->reorth;
   unsigned* cnt = ctx->counters;
-  const bool dgks = sizeof(T) == 8;
+  constexpr bool dgks = sizeof(T) == 8;
   const double* vscl = ctx->gst->vscl;
   CK(launch_matvec<T>(G, tb, V, cr, cc, w, tmp, true, EX(ctx), jd, vs, &ctx->mvt));
-  if (use_ortho<T>(ctx)) {
-    CK(launch_ortho<T>(G, V, vs, w, ctx->partials, ctx->gst, 0, dgks, ctx->bar_count, ctx->rb_dev, ctx->flags,
-                       EX(ctx), jd, &ctl));
-    return;
+  if constexpr (dgks) {
+    if (ctx->ortho) {
+      CK(launch_ortho(G, V, vs, w, ctx->partials, ctx->gst, 0, ctx->bar_count, ctx->rb_dev, ctx->flags, EX(ctx), jd,
+                      &ctl));
+      return;
+    }
   }
   CK(launch_dots<T>(G, V, vs, m, w, ctx->partials, nullptr, ctx->gst->h1, cnt + 0, EX(ctx), jd, vscl));
   CK(launch_cgs_update<T>(G, V, vs, m, ctx->gst->h1, w, ctx->partials, nullptr, ctx->gst, 0, dgks ? 1 : 3, cnt + 1,

@@ -119,7 +119,7 @@ struct GmresDev {
   double nrm2;                // squared norm of the orthogonalised vector
   int reorth;                 // second pass needed (DGKS test)
   int pad_;
-  double hnext, inv_hnext;    // H[j+1][j] and its inverse
+  double hnext;               // H[j+1][j]
   double res;                 // |g_{j+1}|
   // device-side control of graph mode (see GraphCtl): the solve's state and
   // counters that the host reads after a graph launch
@@ -389,24 +389,22 @@ cudaError_t launch_cgs_update(const Geom& G, cpx<T>* V, size_t vstride, int nv, 
                               const cpx<T>* w, double* partials, const int* gate, GmresDev* st, int j, int pass,
                               unsigned* counter, GmresReadback* rb, const int* flags, const Exec& ex,
                               const int* jdev = nullptr, const GraphCtl* ctl = nullptr);
-// The whole orthogonalisation and Givens step of Arnoldi step j in one
+// The whole orthogonalisation and Givens step of an FP64 Arnoldi step j in one
 // cooperative launch, for vectors that ortho_fits() accepts (k_ortho): w = A X_j
 // in, X_{j+1} into slot j+1. part: 2 (MAXV + 2) NBLK doubles; count: a zeroed
 // device word of the handle's own.
 bool ortho_fits(const Geom& G);
-template <typename T>
-cudaError_t launch_ortho(const Geom& G, cpx<T>* V, size_t vstride, const cpx<T>* w, double* part, GmresDev* st, int j,
-                         bool dgks, unsigned long long* count, GmresReadback* rb, int* flags, const Exec& ex,
+cudaError_t launch_ortho(const Geom& G, cpx<double>* V, size_t vstride, const cpx<double>* w, double* part,
+                         GmresDev* st, int j, unsigned long long* count, GmresReadback* rb, int* flags, const Exec& ex,
                          const int* jdev = nullptr, const GraphCtl* ctl = nullptr);
 // r = c - w, and partial squared norm of r
 template <typename T>
 cudaError_t launch_residual(const Geom& G, const cpx<T>* c, const cpx<T>* w, cpx<T>* r, double* partials,
                             const Exec& ex);
 // y = x * f, f = *factor or 1 / *factor (device scalar); may change precision.
-// ysel (may be null): y += (*ysel) * ystride (graph mode).
 template <typename TI, typename TO>
 cudaError_t launch_scale(const Geom& G, const cpx<TI>* x, const double* factor, bool invert, cpx<TO>* y,
-                         const Exec& ex, const int* ysel = nullptr, size_t ystride = 0);
+                         const Exec& ex);
 // x += sum_i coef[i] V_i (V in TV, x in TX); ndev (may be null): nv = *ndev
 template <typename TV, typename TX>
 cudaError_t launch_axpy_multi(const Geom& G, const cpx<TV>* V, size_t vstride, int nv, const double* coef,

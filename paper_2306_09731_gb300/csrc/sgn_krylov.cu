@@ -60,7 +60,6 @@ __device__ void givens_step(GmresDev* st, int j, double nrm2, bool h2, GmresRead
   Hj[j + 1] = 0.0;
   st->nrm2 = nrm2;
   st->hnext = hn;
-  st->inv_hnext = hn > 0.0 ? 1.0 / hn : 0.0;
   st->cs[j] = cj;
   st->sn[j] = sj;
   st->g[j + 1] = -sj * gj;
@@ -407,11 +406,10 @@ constexpr int ORTHO_NE = 4, ORTHO_THR = 512, ORTHO_BLK = 152;
 
 // Block sums of 8 values over nw <= 16 warps (at least 4): the sum of value k on
 // thread 16 k (of the first 128). red: 8 * 16 doubles.
-template <typename A>
-__device__ __forceinline__ double ortho_reduce8(const A (&v)[8], double* red) {
+__device__ __forceinline__ double ortho_reduce8(const double (&v)[8], double* red) {
   const int lane = threadIdx.x & 31;
-  const A c = warp_sum8(v);
-  if ((lane & 3) == 0) red[(lane >> 2) * 16 + (threadIdx.x >> 5)] = (double)c;
+  const double c = warp_sum8(v);
+  if ((lane & 3) == 0) red[(lane >> 2) * 16 + (threadIdx.x >> 5)] = c;
   __syncthreads();
   double t = 0.0;
   if (threadIdx.x < 128) {
@@ -423,8 +421,8 @@ __device__ __forceinline__ double ortho_reduce8(const A (&v)[8], double* red) {
 }
 
 // The whole orthogonalisation of Arnoldi step j for vectors of up to ORTHO_BLK *
-// ORTHO_THR * ORTHO_NE entries: k_dots and k_cgs_update (dgks: and their gated second
-// pair) with w in registers and a grid barrier in the place of each kernel
+// ORTHO_THR * ORTHO_NE FP64 entries: k_dots and k_cgs_update and their gated second
+// pair with w in registers and a grid barrier in the place of each kernel
 // boundary. On such grids the four launches (the second pair nearly always runs,
 // as A is near the identity) are mostly latency: an Arnoldi step's
 // orthogonalisation takes about 25 us instead of 45 at 256 x 16, 50 instead of 69
@@ -432,29 +430,26 @@ __device__ __forceinline__ double ortho_reduce8(const A (&v)[8], double* red) {
 // Every block sums the partials itself, in the same order, so all take the same
 // DGKS decision. part: two regions of MAXV + 2 slots, one for each pass, as a
 // block may write its share of the next sum while others still read the last.
-template <typename T>
-__global__ void __launch_bounds__(ORTHO_THR, 1) k_ortho(Geom G, cpx<T>* V, size_t vstride, const cpx<T>* w, double* part,
-                                                  GmresDev* st, int j, int dgks, unsigned long long* count,
-                                                  GmresReadback* rb, int* flags, const int* jdev, GraphCtl ctl) {
-  typedef typename Acc<T>::type A;
+__global__ void __launch_bounds__(ORTHO_THR, 1) k_ortho(Geom G, cpx<double>* V, size_t vstride, const cpx<double>* w,
+                                                        double* part, GmresDev* st, int j, unsigned long long* count,
+                                                        GmresReadback* rb, int* flags, const int* jdev, GraphCtl ctl) {
   constexpr int CH = 7;
   if (jdev) j = *jdev;
   const int nv = j + 1, nblk = gridDim.x, lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
   __shared__ double red[8 * 32];
   __shared__ double hs[MAXV + 2];
   __shared__ double sc[MAXV + 1];
-  __shared__ A cf[MAXV + 8];
-  const size_t n = G.nspec();
-  const int nthr = nblk * blockDim.x;
-  cpx<T> z[ORTHO_NE];
+  __shared__ double cf[MAXV + 8];
+  const int n = (int)G.nspec(), nthr = nblk * blockDim.x;
+  cpx<double> z[ORTHO_NE];
   int wt[ORTHO_NE];
-  size_t e[ORTHO_NE];
+  int e[ORTHO_NE];
 #pragma unroll
   for (int k = 0; k < ORTHO_NE; ++k) {
-    e[k] = (size_t)blockIdx.x * blockDim.x + threadIdx.x + (size_t)k * nthr;
+    e[k] = blockIdx.x * blockDim.x + threadIdx.x + k * nthr;
     const bool in = e[k] < n;
-    z[k] = in ? w[e[k]] : mk((T)0, (T)0);
-    wt[k] = in ? col_weight_i(G, (int)(e[k] % G.ldS)) : 0;
+    z[k] = in ? w[e[k]] : mk(0.0, 0.0);
+    wt[k] = in ? col_weight_i(G, e[k] % G.ldS) : 0;
     if (!in) e[k] = 0;
   }
   if (threadIdx.x < MAXV + 1) sc[threadIdx.x] = (int)threadIdx.x <= j ? st->vscl[threadIdx.x] : 0.0;
@@ -467,21 +462,21 @@ __global__ void __launch_bounds__(ORTHO_THR, 1) k_ortho(Geom G, cpx<T>* V, size_
     // <X_i, w> (and |w|^2) of the thread's entries
 #pragma unroll 1
     for (int i0 = 0; i0 < nv; i0 += CH) {
-      A acc[CH + 1];
+      double acc[CH + 1];
 #pragma unroll
-      for (int i = 0; i <= CH; ++i) acc[i] = (A)0;
+      for (int i = 0; i <= CH; ++i) acc[i] = 0.0;
 #pragma unroll
       for (int k = 0; k < ORTHO_NE; ++k) {
-        if (k * nthr >= (int)n) break;
-        cpx<T> x[CH];
+        if (k * nthr >= n) break;
+        cpx<double> x[CH];
 #pragma unroll
         for (int i = 0; i < CH; ++i)
           if (i0 + i < nv) x[i] = V[(size_t)(i0 + i) * vstride + e[k]];
-        const A ax = weigh(wt[k], (A)z[k].x), ay = weigh(wt[k], (A)z[k].y);
+        const double ax = weigh(wt[k], z[k].x), ay = weigh(wt[k], z[k].y);
 #pragma unroll
         for (int i = 0; i < CH; ++i)
-          if (i0 + i < nv) acc[i] = fma(ay, (A)x[i].y, fma(ax, (A)x[i].x, acc[i]));
-        if (i0 == 0 && pass == 1 && dgks) acc[CH] = fma(ay, (A)z[k].y, fma(ax, (A)z[k].x, acc[CH]));
+          if (i0 + i < nv) acc[i] = fma(ay, x[i].y, fma(ax, x[i].x, acc[i]));
+        if (i0 == 0 && pass == 1) acc[CH] = fma(ay, z[k].y, fma(ax, z[k].x, acc[CH]));
       }
       const double tot = ortho_reduce8(acc, red);
       const int k8 = threadIdx.x >> 4;
@@ -495,35 +490,35 @@ __global__ void __launch_bounds__(ORTHO_THR, 1) k_ortho(Geom G, cpx<T>* V, size_
     __syncthreads();
     if ((int)threadIdx.x < nv) {
       const double h = hs[threadIdx.x] * sc[threadIdx.x] * sj;
-      cf[threadIdx.x] = (A)(h * sc[threadIdx.x] / sj);
+      cf[threadIdx.x] = h * sc[threadIdx.x] / sj;
       if (blockIdx.x == 0) (pass == 1 ? st->h1 : st->h2)[threadIdx.x] = h;
     } else if (threadIdx.x < MAXV + 8) {
-      cf[threadIdx.x] = (A)0;
+      cf[threadIdx.x] = 0.0;
     }
     __syncthreads();
     // X_{j+1} = w~ - sum_i (h_i s_i / s_j) X_i and its norm
-    A nrm[ORTHO_NE] = {(A)0};
+    double nrm[ORTHO_NE] = {0.0};
 #pragma unroll
     for (int k = 0; k < ORTHO_NE; ++k) {
-      if (k * nthr >= (int)n) break;
-      A zx = (A)z[k].x, zy = (A)z[k].y;
+      if (k * nthr >= n) break;
+      double zx = z[k].x, zy = z[k].y;
       for (int i = 0; i < nv; i += 4) {
-        cpx<T> x[4];
+        cpx<double> x[4];
 #pragma unroll
         for (int u = 0; u < 4; ++u)
           if (i + u < nv) x[u] = V[(size_t)(i + u) * vstride + e[k]];
 #pragma unroll
         for (int u = 0; u < 4; ++u)
           if (i + u < nv) {
-            const A c = -cf[i + u];
-            zx = fma(c, (A)x[u].x, zx);
-            zy = fma(c, (A)x[u].y, zy);
+            const double c = -cf[i + u];
+            zx = fma(c, x[u].x, zx);
+            zy = fma(c, x[u].y, zy);
           }
       }
-      z[k] = mk((T)zx, (T)zy);
-      nrm[k] = weigh(wt[k], (A)z[k].x * (A)z[k].x + (A)z[k].y * (A)z[k].y);
+      z[k] = mk(zx, zy);
+      nrm[k] = weigh(wt[k], z[k].x * z[k].x + z[k].y * z[k].y);
     }
-    A one[8] = {(nrm[0] + nrm[1]) + (nrm[2] + nrm[3])};
+    const double one[8] = {(nrm[0] + nrm[1]) + (nrm[2] + nrm[3])};
     const double tot = ortho_reduce8(one, red);
     if (threadIdx.x == 0) pr[(size_t)(MAXV + 1) * NBLK + blockIdx.x] = tot;
     const double w2 = hs[nv] * sj * sj;  // |w|^2 before the pass (first pass)
@@ -536,7 +531,7 @@ __global__ void __launch_bounds__(ORTHO_THR, 1) k_ortho(Geom G, cpx<T>* V, size_
     }
     __syncthreads();
     n2 = hs[MAXV + 1];
-    const bool need = dgks && pass == 1 && n2 < 0.5 * w2;
+    const bool need = pass == 1 && n2 < 0.5 * w2;
     if (!need) {
       if (blockIdx.x == 0 && warp == 0) {
         if (ctl.enabled && lane == 0) cudaGraphSetConditional(ctl.h_step, 0u);
@@ -549,10 +544,10 @@ __global__ void __launch_bounds__(ORTHO_THR, 1) k_ortho(Geom G, cpx<T>* V, size_
       break;
     }
   }
-  cpx<T>* out = V + (size_t)(j + 1) * vstride;
+  cpx<double>* out = V + (size_t)(j + 1) * vstride;
 #pragma unroll
   for (int k = 0; k < ORTHO_NE; ++k)
-    if ((size_t)blockIdx.x * blockDim.x + threadIdx.x + (size_t)k * nthr < n) out[e[k]] = z[k];
+    if ((int)(blockIdx.x * blockDim.x + threadIdx.x) + k * nthr < n) out[e[k]] = z[k];
 }
 
 template <typename T>
@@ -572,9 +567,7 @@ __global__ void __launch_bounds__(256) k_residual(Geom G, const cpx<T>* c, const
 }
 
 template <typename TI, typename TO>
-__global__ void k_scale(Geom G, const cpx<TI>* x, const double* factor, int invert, cpx<TO>* y, const int* ysel,
-                        size_t ystride) {
-  if (ysel) y += (size_t)(*ysel) * ystride;
+__global__ void k_scale(Geom G, const cpx<TI>* x, const double* factor, int invert, cpx<TO>* y) {
   // arithmetic in the output type: an FP32 result (the inner basis) is
   // scaled in FP32 after the conversion, which stays off the FP64 pipe
   const double f0 = *factor;
@@ -954,15 +947,14 @@ bool ortho_fits(const Geom& G) {
   if (cudaGetDevice(&dev) != cudaSuccess ||
       cudaDeviceGetAttribute(&coop, cudaDevAttrCooperativeLaunch, dev) != cudaSuccess ||
       cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev) != cudaSuccess ||
-      cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per, k_ortho<double>, ORTHO_THR, 0) != cudaSuccess) {
+      cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per, k_ortho, ORTHO_THR, 0) != cudaSuccess) {
     cudaGetLastError();
     return false;
   }
   return coop && per * sms >= ORTHO_BLK;
 }
-template <typename T>
-cudaError_t launch_ortho(const Geom& G, cpx<T>* V, size_t vstride, const cpx<T>* w, double* part, GmresDev* st, int j,
-                         bool dgks, unsigned long long* count, GmresReadback* rb, int* flags, const Exec& ex,
+cudaError_t launch_ortho(const Geom& G, cpx<double>* V, size_t vstride, const cpx<double>* w, double* part,
+                         GmresDev* st, int j, unsigned long long* count, GmresReadback* rb, int* flags, const Exec& ex,
                          const int* jdev, const GraphCtl* ctl) {
   GraphCtl c{};
   if (ctl) c = *ctl;
@@ -980,8 +972,7 @@ cudaError_t launch_ortho(const Geom& G, cpx<T>* V, size_t vstride, const cpx<T>*
   cfg.attrs = &at;
   cfg.numAttrs = 1;
   ex.begin(PK_KRYLOV);
-  const cudaError_t e = cudaLaunchKernelEx(&cfg, k_ortho<T>, G, V, vstride, w, part, st, j, dgks ? 1 : 0, count, rb,
-                                           flags, jdev, c);
+  const cudaError_t e = cudaLaunchKernelEx(&cfg, k_ortho, G, V, vstride, w, part, st, j, count, rb, flags, jdev, c);
   ex.end();
   return e != cudaSuccess ? e : cudaGetLastError();
 }
@@ -995,9 +986,9 @@ cudaError_t launch_residual(const Geom& G, const cpx<T>* c, const cpx<T>* w, cpx
 }
 template <typename TI, typename TO>
 cudaError_t launch_scale(const Geom& G, const cpx<TI>* x, const double* factor, bool invert, cpx<TO>* y,
-                         const Exec& ex, const int* ysel, size_t ystride) {
+                         const Exec& ex) {
   ex.begin(PK_KRYLOV);
-  k_scale<TI, TO><<<sweep_blocks(G, 1, NBLK), 256, 0, ex.s>>>(G, x, factor, invert ? 1 : 0, y, ysel, ystride);
+  k_scale<TI, TO><<<sweep_blocks(G, 1, NBLK), 256, 0, ex.s>>>(G, x, factor, invert ? 1 : 0, y);
   ex.end();
   return cudaGetLastError();
 }
@@ -1135,9 +1126,6 @@ cudaError_t launch_invariant_sums(const Geom& G, const double* h, const double* 
                                             double*, const int*, GmresDev*, int, int, unsigned*,            \
                                             GmresReadback*, const int*, const Exec&, const int*,            \
                                             const GraphCtl*);                                               \
-  template cudaError_t launch_ortho<T>(const Geom&, cpx<T>*, size_t, const cpx<T>*, double*, GmresDev*, int, \
-                                       bool, unsigned long long*, GmresReadback*, int*, const Exec&,         \
-                                       const int*, const GraphCtl*);                                         \
   template cudaError_t launch_residual<T>(const Geom&, const cpx<T>*, const cpx<T>*, cpx<T>*, double*,       \
                                           const Exec&);                                                     \
   template cudaError_t launch_zero<T>(const Geom&, cpx<T>*, const Exec&, const int*);                       \
@@ -1148,7 +1136,7 @@ cudaError_t launch_invariant_sums(const Geom& G, const double* h, const double* 
 SGN_KRYLOV_INST(double)
 SGN_KRYLOV_INST(float)
 template cudaError_t launch_scale<double, float>(const Geom&, const cpx<double>*, const double*, bool,
-                                                 cpx<float>*, const Exec&, const int*, size_t);
+                                                 cpx<float>*, const Exec&);
 template cudaError_t launch_axpy_multi<double, double>(const Geom&, const cpx<double>*, size_t, int,
                                                        const double*, cpx<double>*, const Exec&, const int*,
                                                        const double*);
