@@ -226,6 +226,16 @@ sgn_status sgn_elliptic_apply_noalloc(int Nx, int Ny, double Lx, double Ly,
                                       const double* h, const double* sigma, double* out,
                                       void* cuda_stream);
 
+/* Self-test of the bounded wait inside the one-launch orthogonalisation of the
+ * FP64 GMRES (grids of up to 311,296 half-spectrum entries, such as 1024 x 512),
+ * host-driven and in step graphs: on a handle of its own, a call whose grid
+ * barrier waits for one block more than there are must return SGN_ECUDA, and the
+ * same call on the same handle before and after it must give the same bits.
+ * SGN_OK if all of that held, SGN_ECUDA if not; SGN_EINVAL for other sizes than
+ * sgn_create's or a grid that orthogonalises otherwise. Allocates, and synchronises
+ * cuda_stream; a fraction of a second. */
+sgn_status sgn_grid_wait_selftest(int Nx, int Ny, void* cuda_stream);
+
 /* Message for the last failing call on ctx. With ctx NULL: the message of
  * the last failing handle-less call (sgn_create, sgn_elliptic_apply_noalloc)
  * made by the calling host thread (one slot per thread, like errno). */

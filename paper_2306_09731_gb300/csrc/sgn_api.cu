@@ -89,7 +89,7 @@ struct sgn_ctx {
   double* inv_host = nullptr;        // pinned, 4 doubles
   int* flags = nullptr;
   bool ortho = false;                      // Arnoldi steps orthogonalise in one launch (ortho_fits)
-  unsigned long long* bar_count = nullptr;  // its grid barrier
+  GridBar bar;                              // its grid barrier; the count lies 8 bytes behind flags
   unsigned* counters = nullptr;  // last-block reduction tickets (zeroed, self-resetting)
   Prof prof;
   // graph mode (opt.graph = 1): one RK4 step as an instantiated graph
@@ -487,7 +487,12 @@ void sync_read(sgn_ctx* ctx) {
   if (ctx->prof.on) ctx->prof.harvest();
 }
 
+// (a wait that ran out first: what it left unfinished may have set the others)
 void check_flags(sgn_ctx* ctx, int flags) {
+  if (flags & FLAG_WAIT) {
+    ctx->err = "a kernel stopped waiting for its tensor copies or its grid (bounded wait ran out)";
+    throw Fail{SGN_ECUDA};
+  }
   if (flags & FLAG_NONFINITE) {
     ctx->err = "non-finite depth h";
     throw Fail{SGN_ENONFINITE};
@@ -495,10 +500,6 @@ void check_flags(sgn_ctx* ctx, int flags) {
   if (flags & FLAG_CAVITATION) {
     ctx->err = "cavitation: h <= 0 somewhere";
     throw Fail{SGN_ECAVITATION};
-  }
-  if (flags & FLAG_WAIT) {
-    ctx->err = "a kernel stopped waiting for its tensor copies or its grid (bounded wait ran out)";
-    throw Fail{SGN_ECUDA};
   }
 }
 
@@ -541,7 +542,7 @@ void arnoldi_step(sgn_ctx* ctx, const Tables<T>& tb, const T* cr, const T* cc, c
   // waiting (12 members: 42 ms with two kernels, 58 with one).
   if constexpr (dgks) {
     if (ctx->ortho) {
-      CK(launch_ortho(G, V, vs, w, ctx->partials, ctx->gst, j, ctx->bar_count, ctx->rb_dev, ctx->flags, EX(ctx)));
+      CK(launch_ortho(G, V, vs, w, ctx->partials, ctx->gst, j, ctx->bar, ctx->rb_dev, ctx->flags, EX(ctx)));
       sync_read(ctx);
       return;
     }
@@ -606,6 +607,7 @@ bool gmres_fp64(sgn_ctx* ctx, int* iters_out, double* relres_out) {
     int k = 0;
     for (int j = 0; j < m; ++j) {
       arnoldi_step<double>(ctx, ctx->tb, ctx->cr, ctx->cc, V, ctx->w, ctx->tmp, j);
+      check_flags(ctx, ctx->rb_host->flags);
       ++its;
       res = ctx->rb_host->res;
       const double hnext = ctx->rb_host->hnext;
@@ -867,7 +869,9 @@ bool stage(sgn_ctx* ctx, int mode, double dt) {
   return conv;
 }
 
-void reset_flags(sgn_ctx* ctx) { CK(cudaMemsetAsync(ctx->flags, 0, sizeof(int), ctx->stream)); }
+// (with the count of the grid barrier, which a wait that ran out leaves anywhere)
+constexpr size_t kFlagBytes = 16;
+void reset_flags(sgn_ctx* ctx) { CK(cudaMemsetAsync(ctx->flags, 0, kFlagBytes, ctx->stream)); }
 
 void ensure_phys(sgn_ctx* ctx) {
   if (ctx->phys[0]) return;
@@ -1019,7 +1023,7 @@ void graph_arnoldi(sgn_ctx* ctx, const Tables<T>& tb, const T* cr, const T* cc, 
   CK(launch_matvec<T>(G, tb, V, cr, cc, w, tmp, true, EX(ctx), jd, vs, &ctx->mvt));
   if constexpr (dgks) {
     if (ctx->ortho) {
-      CK(launch_ortho(G, V, vs, w, ctx->partials, ctx->gst, 0, ctx->bar_count, ctx->rb_dev, ctx->flags, EX(ctx), jd,
+      CK(launch_ortho(G, V, vs, w, ctx->partials, ctx->gst, 0, ctx->bar, ctx->rb_dev, ctx->flags, EX(ctx), jd,
                       &ctl));
       return;
     }
@@ -1386,11 +1390,11 @@ sgn_status sgn_create(int Nx, int Ny, double Lx, double Ly, double g, const sgn_
     ctx->cc = dalloc<double>(ctx, G.nphys());
     ctx->partials = dalloc<double>(ctx, 2 * (size_t)(MAXV + 2) * NBLK);
     ctx->ortho = ortho_fits(G);
-    ctx->bar_count = dalloc<unsigned long long>(ctx, 1);
     ctx->scal = dalloc<double>(ctx, 16);
     ctx->gst = dalloc<GmresDev>(ctx, 1);
     ctx->rb_dev = dalloc<GmresReadback>(ctx, 1);
-    ctx->flags = dalloc<int>(ctx, 1);
+    ctx->flags = dalloc<int>(ctx, kFlagBytes / sizeof(int));
+    ctx->bar.count = reinterpret_cast<unsigned long long*>(ctx->flags + 2);
     ctx->counters = dalloc<unsigned>(ctx, 8);
     CK(cudaMemset(ctx->counters, 0, 8 * sizeof(unsigned)));
     if (o.precision >= 1) {
@@ -1400,7 +1404,7 @@ sgn_status sgn_create(int Nx, int Ny, double Lx, double Ly, double g, const sgn_
     }
     CK(cudaMallocHost((void**)&ctx->rb_host, sizeof(GmresReadback)));
     CK(cudaMallocHost((void**)&ctx->inv_host, 4 * sizeof(double)));
-    CK(cudaMemset(ctx->flags, 0, sizeof(int)));
+    CK(cudaMemset(ctx->flags, 0, kFlagBytes));
     CK(cudaMemset(ctx->gst, 0, sizeof(GmresDev)));
     // spectra are zero-initialised so padding never holds garbage
     for (int f = 0; f < 3; ++f) {
@@ -2020,6 +2024,52 @@ sgn_status sgn_invariants(sgn_t ctx, const double* h, const double* vx, const do
   for (int q = 0; q < 4; ++q) out[q] = ctx->inv_host[q] * dA;
   return SGN_OK;
   API_END
+}
+
+sgn_status sgn_grid_wait_selftest(int Nx, int Ny, void* cuda_stream) {
+  bool held = true;
+  for (int graph = 0; graph < 2; ++graph) {
+    sgn_options o;
+    sgn_default_options(&o);
+    o.graph = graph;
+    sgn_t ctx = nullptr;
+    const sgn_status st = sgn_create(Nx, Ny, 0.1 * Nx, 0.1 * Ny, 1.0, &o, &ctx);
+    if (st != SGN_OK) return st;
+    if (!ctx->ortho) {
+      sgn_destroy(ctx);
+      return SGN_EINVAL;
+    }
+    const size_t n = ctx->G.nphys();
+    // h, vx, vy, sigma of a call; gmres_solve takes vx as its right-hand side
+    std::vector<double> init(4 * n, 0.0), first(4 * n), again(4 * n);
+    for (size_t i = 0; i < n; ++i) {
+      const double a = 6.283185307179586 * (double)(i % Nx) / Nx, b = 6.283185307179586 * (double)(i / Nx) / Ny;
+      init[i] = 1.0 + 0.25 * cos(a) + 0.125 * sin(b);
+      init[n + i] = 0.1 * sin(a + b);
+    }
+    try {
+      ctx->stream = (cudaStream_t)cuda_stream;
+      double* f = dalloc<double>(ctx, 4 * n);
+      auto call = [&](bool stall, std::vector<double>* out) {
+        ctx->bar.stall = stall ? 1 : 0;
+        ctx->bar.polls = stall ? 1 << 12 : GridBar{}.polls;
+        free_graph(ctx);  // a captured step keeps the barrier it was captured with
+        CK(cudaMemcpyAsync(f, init.data(), 4 * n * sizeof(double), cudaMemcpyHostToDevice, ctx->stream));
+        const sgn_status r = graph ? sgn_rk4_step(ctx, f, f + n, f + 2 * n, f + 3 * n, 1e-3, 2)
+                                   : sgn_gmres_solve(ctx, f, f + n, f + 3 * n, nullptr, nullptr);
+        if (out) CK(cudaMemcpyAsync(out->data(), f, 4 * n * sizeof(double), cudaMemcpyDeviceToHost, ctx->stream));
+        CK(cudaStreamSynchronize(ctx->stream));
+        return r;
+      };
+      held = call(false, &first) == SGN_OK && call(true, nullptr) == SGN_ECUDA && call(false, &again) == SGN_OK &&
+             first == again && held;
+    } catch (Fail&) {
+      held = false;
+    }
+    cudaStreamSynchronize((cudaStream_t)cuda_stream);
+    sgn_destroy(ctx);
+  }
+  return held ? SGN_OK : SGN_ECUDA;
 }
 
 }  // extern "C"

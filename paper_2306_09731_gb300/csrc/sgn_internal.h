@@ -391,11 +391,19 @@ cudaError_t launch_cgs_update(const Geom& G, cpx<T>* V, size_t vstride, int nv, 
                               const int* jdev = nullptr, const GraphCtl* ctl = nullptr);
 // The whole orthogonalisation and Givens step of an FP64 Arnoldi step j in one
 // cooperative launch, for vectors that ortho_fits() accepts (k_ortho): w = A X_j
-// in, X_{j+1} into slot j+1. part: 2 (MAXV + 2) NBLK doubles; count: a zeroed
-// device word of the handle's own.
+// in, X_{j+1} into slot j+1. part: 2 (MAXV + 2) NBLK doubles.
 bool ortho_fits(const Geom& G);
+// Its grid barrier: count is a device word of the handle's own, zeroed with the
+// flags before each call (after a wait that ran out it need not be a multiple of
+// the grid). polls bounds a wait, 2^22 take seconds. stall: self-test only, 1 waits
+// for one arrival more than there are blocks, so that every wait runs out.
+struct GridBar {
+  unsigned long long* count = nullptr;
+  int polls = 1 << 22;
+  int stall = 0;
+};
 cudaError_t launch_ortho(const Geom& G, cpx<double>* V, size_t vstride, const cpx<double>* w, double* part,
-                         GmresDev* st, int j, unsigned long long* count, GmresReadback* rb, int* flags, const Exec& ex,
+                         GmresDev* st, int j, const GridBar& bar, GmresReadback* rb, int* flags, const Exec& ex,
                          const int* jdev = nullptr, const GraphCtl* ctl = nullptr);
 // r = c - w, and partial squared norm of r
 template <typename T>

@@ -380,24 +380,46 @@ __global__ void __launch_bounds__(256) k_cgs_update(Geom G, cpx<T>* V, size_t vs
 
 // ------------------------------------------- one Arnoldi step in one launch
 // A grid barrier of a cooperative launch: every block arrives once per barrier
-// (count: 64-bit, never reset, a multiple of the grid between launches), and
-// the wait is bounded (about a second): *flags gets FLAG_WAIT when it runs out.
-__device__ __forceinline__ void grid_barrier(unsigned long long* count, int* flags) {
+// (the count is a multiple of the grid between launches), and the wait is bounded.
+// Returns whether the grid arrived, the same to the whole block; if not, *flags
+// has FLAG_WAIT and the block has to return. A wait looks at the flags now and
+// then, so that the launches after one that gave up (a captured step has many)
+// don't each wait to their limit.
+__device__ __forceinline__ bool grid_barrier(const GridBar& bar, int* flags) {
   __syncthreads();
+  bool ok = true;
   if (threadIdx.x == 0) {
     __threadfence();
     const unsigned long long n = gridDim.x;
-    const unsigned long long target = (atomicAdd(count, 1ull) / n + 1ull) * n;
-    bool ok = false;
-    for (int it = 0; it < (1 << 22) && !ok; ++it) {
-      unsigned long long c;
-      asm volatile("ld.acquire.gpu.global.u64 %0, [%1];" : "=l"(c) : "l"(count) : "memory");
-      ok = c >= target;
+    const unsigned long long target = (atomicAdd(bar.count, 1ull) / n + 1ull) * n + (unsigned long long)bar.stall;
+    ok = false;
+    for (int left = bar.polls; left > 0 && !ok; left -= 1024) {
+      for (int it = 0; it < 1024 && !ok; ++it) {
+        unsigned long long c;
+        asm volatile("ld.acquire.gpu.global.u64 %0, [%1];" : "=l"(c) : "l"(bar.count) : "memory");
+        ok = c >= target;
+      }
+      if (!ok && (*(volatile const int*)flags & FLAG_WAIT)) break;
     }
     if (!ok) atomicOr(flags, FLAG_WAIT);
     __threadfence();
   }
-  __syncthreads();
+  return __syncthreads_and(ok ? 1 : 0) != 0;
+}
+
+// Arnoldi step j of a block whose wait ran out: block 0 ends the cycle with no
+// number for a residual, which the host loop and the graph's control take as a
+// failure, and reports the flags. While block 0 gets through its barriers, so
+// have all others arrived at them: its sums, and with them the step, are whole.
+__device__ __forceinline__ void ortho_gave_up(GmresDev* st, int j, GmresReadback* rb, const int* flags,
+                                              const GraphCtl& ctl) {
+  if (blockIdx.x != 0 || threadIdx.x != 0) return;
+  st->res = __longlong_as_double(0x7ff8000000000000ll);
+  st->hnext = 0.0;
+  rb->res = st->res;
+  rb->hnext = 0.0;
+  rb->flags = *(volatile const int*)flags;
+  if (ctl.enabled) ctl_step(st, j, ctl);
 }
 
 // Entries of w a thread of k_ortho holds at most, its threads at most and its
@@ -431,7 +453,7 @@ __device__ __forceinline__ double ortho_reduce8(const double (&v)[8], double* re
 // DGKS decision. part: two regions of MAXV + 2 slots, one for each pass, as a
 // block may write its share of the next sum while others still read the last.
 __global__ void __launch_bounds__(ORTHO_THR, 1) k_ortho(Geom G, cpx<double>* V, size_t vstride, const cpx<double>* w,
-                                                        double* part, GmresDev* st, int j, unsigned long long* count,
+                                                        double* part, GmresDev* st, int j, GridBar bar,
                                                         GmresReadback* rb, int* flags, const int* jdev, GraphCtl ctl) {
   constexpr int CH = 7;
   if (jdev) j = *jdev;
@@ -484,7 +506,7 @@ __global__ void __launch_bounds__(ORTHO_THR, 1) k_ortho(Geom G, cpx<double>* V, 
       if (threadIdx.x == 16 * CH && i0 == 0) pr[(size_t)nv * NBLK + blockIdx.x] = tot;
       __syncthreads();
     }
-    grid_barrier(count, flags);
+    if (!grid_barrier(bar, flags)) return ortho_gave_up(st, j, rb, flags, ctl);
     // V_i = s_i X_i, w = s_j w~
     reduce_slots(pr, nv + 1, hs, nblk);
     __syncthreads();
@@ -522,7 +544,7 @@ __global__ void __launch_bounds__(ORTHO_THR, 1) k_ortho(Geom G, cpx<double>* V, 
     const double tot = ortho_reduce8(one, red);
     if (threadIdx.x == 0) pr[(size_t)(MAXV + 1) * NBLK + blockIdx.x] = tot;
     const double w2 = hs[nv] * sj * sj;  // |w|^2 before the pass (first pass)
-    grid_barrier(count, flags);
+    if (!grid_barrier(bar, flags)) return ortho_gave_up(st, j, rb, flags, ctl);
     if (warp == 0) {
       double t = 0.0;
       for (int b = lane; b < nblk; b += 32) t += __ldcg(pr + (size_t)(MAXV + 1) * NBLK + b);
@@ -954,7 +976,7 @@ bool ortho_fits(const Geom& G) {
   return coop && per * sms >= ORTHO_BLK;
 }
 cudaError_t launch_ortho(const Geom& G, cpx<double>* V, size_t vstride, const cpx<double>* w, double* part,
-                         GmresDev* st, int j, unsigned long long* count, GmresReadback* rb, int* flags, const Exec& ex,
+                         GmresDev* st, int j, const GridBar& bar, GmresReadback* rb, int* flags, const Exec& ex,
                          const int* jdev, const GraphCtl* ctl) {
   GraphCtl c{};
   if (ctl) c = *ctl;
@@ -972,7 +994,7 @@ cudaError_t launch_ortho(const Geom& G, cpx<double>* V, size_t vstride, const cp
   cfg.attrs = &at;
   cfg.numAttrs = 1;
   ex.begin(PK_KRYLOV);
-  const cudaError_t e = cudaLaunchKernelEx(&cfg, k_ortho, G, V, vstride, w, part, st, j, count, rb, flags, jdev, c);
+  const cudaError_t e = cudaLaunchKernelEx(&cfg, k_ortho, G, V, vstride, w, part, st, j, bar, rb, flags, jdev, c);
   ex.end();
   return e != cudaSuccess ? e : cudaGetLastError();
 }

@@ -26,7 +26,7 @@ EXPORTS = ["sgn_default_options", "sgn_create", "sgn_destroy", "sgn_set_stream",
            "sgn_get_stats", "sgn_set_profiling", "sgn_get_profile", "sgn_elliptic_apply_noalloc",
            "sgn_diagnostics", "sgn_set_learned_guess", "sgn_record_learned", "sgn_recorded_count",
            "sgn_coarse_sample", "sgn_coarse_embed", "sgn_rk4_step_batch", "sgn_autotune", "sgn_set_tuning",
-           "sgn_last_error"]
+           "sgn_grid_wait_selftest", "sgn_last_error"]
 
 # index names of sgn_tuning's [type][pass] arrays
 TUNE_TYPES = ["fp32", "fp64", "dfl"]
@@ -113,6 +113,7 @@ def load_library(path: str | None = None, build_if_missing: bool = True) -> ctyp
         "sgn_coarse_embed": (_I, [_P, _P, _I, _D, _P]),
         "sgn_rk4_step_batch": (_I, [ctypes.POINTER(_P), _I, ctypes.POINTER(_P), ctypes.POINTER(_P),
                                     ctypes.POINTER(_P), ctypes.POINTER(_P), _D, _I, ctypes.POINTER(_I)]),
+        "sgn_grid_wait_selftest": (_I, [_I, _I, _P]),
         "sgn_last_error": (ctypes.c_char_p, [_P]),
     }
     for name, (res, args) in sig.items():
