@@ -585,13 +585,14 @@ bool gmres_fp64(sgn_ctx* ctx, int* iters_out, double* relres_out) {
     return true;
   }
   const double target = ctx->opt.tol * cnorm;
+  const int rexp = residual_exp(cnorm);
   int its = 0;
   bool conv = false;
   double res = 0.0;
   C64* const V = ctx->V;
   for (;;) {
     CK(launch_matvec<double>(G, ctx->tb, ctx->sig, ctx->cr, ctx->cc, ctx->w, ctx->tmp, true, EX(ctx)));
-    CK(launch_residual<double>(G, ctx->cvec, ctx->w, V, ctx->partials, EX(ctx)));
+    CK(launch_residual<double>(G, ctx->cvec, ctx->w, V, ctx->partials, EX(ctx), rexp));
     CK(launch_reduce(ctx->partials, 1, beta_d, true, nullptr, EX(ctx), sweep_partials(G)));
     CK(launch_readback_scalar(beta_d, ctx->flags, ctx->rb_dev, EX(ctx)));
     sync_read(ctx);
@@ -603,7 +604,7 @@ bool gmres_fp64(sgn_ctx* ctx, int* iters_out, double* relres_out) {
       break;
     }
     if (its >= ctx->opt.maxit) break;
-    CK(launch_gmres_start(ctx->gst, beta_d, false, EX(ctx)));
+    CK(launch_gmres_start(ctx->gst, beta_d, false, EX(ctx), rexp));
     int k = 0;
     for (int j = 0; j < m; ++j) {
       arnoldi_step<double>(ctx, ctx->tb, ctx->cr, ctx->cc, V, ctx->w, ctx->tmp, j);
@@ -1068,7 +1069,7 @@ void graph_gmres(sgn_ctx* ctx, GraphSeg& top) {
   long long per_sweep = count_launches(ctx, [&] {
     refine_matvec(ctx, true, EX(ctx));
     C64* r = mixed ? ctx->r64 : ctx->V;
-    CK(launch_residual<double>(G, ctx->cvec, ctx->w, r, ctx->partials, EX(ctx)));
+    CK(launch_residual<double>(G, ctx->cvec, ctx->w, r, ctx->partials, EX(ctx), 0, mixed ? nullptr : &ctx->gst->rexp));
     CK(launch_reduce(ctx->partials, 1, beta_d, true, nullptr, EX(ctx), sweep_partials(G)));
     CK(launch_ctl_sweep(ctx->gst, beta_d, ctl, EX(ctx)));
     if (mixed) CK((launch_scale<double, float>(G, r, beta_d, true, ctx->V32, EX(ctx))));

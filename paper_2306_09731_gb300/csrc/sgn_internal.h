@@ -2,6 +2,7 @@
 #pragma once
 #include <cuda.h>
 #include <cuda_runtime.h>
+#include <math.h>
 #include <stddef.h>
 #include <stdint.h>
 
@@ -116,6 +117,7 @@ struct GmresDev {
   // basis vector i is stored unnormalised, V_i = vscl[i] X_i (the
   // orthogonalised vector of step i-1, written straight into its slot)
   double vscl[MAXV + 1];
+  int rexp;                   // FP64: X_0 is the residual times 2^rexp (residual_exp)
   double nrm2;                // squared norm of the orthogonalised vector
   int reorth;                 // second pass needed (DGKS test)
   int pad_;
@@ -405,10 +407,21 @@ struct GridBar {
 cudaError_t launch_ortho(const Geom& G, cpx<double>* V, size_t vstride, const cpx<double>* w, double* part,
                          GmresDev* st, int j, const GridBar& bar, GmresReadback* rb, int* flags, const Exec& ex,
                          const int* jdev = nullptr, const GraphCtl* ctl = nullptr);
-// r = c - w, and partial squared norm of r
+// r = (c - w) 2^rexp, and partial squared norm of c - w; rexp_dev (may be null):
+// rexp = *rexp_dev
 template <typename T>
 cudaError_t launch_residual(const Geom& G, const cpx<T>* c, const cpx<T>* w, cpx<T>* r, double* partials,
-                            const Exec& ex);
+                            const Exec& ex, int rexp = 0, const int* rexp_dev = nullptr);
+// The exponent that the FP64 basis, whose first vector is the residual itself, is
+// scaled by: products of two of its vectors have the square of the right-hand
+// side's size, and a cycle's vectors shrink with the residual, so a |c| of 1e-145 or
+// of 1e153 would lose them to underflow or overflow. 0 (nothing is scaled, and no
+// bit differs) between 2^-300 and 2^300.
+__host__ __device__ inline int residual_exp(double cnorm) {
+  if (!(cnorm > 0.0) || !(cnorm < INFINITY)) return 0;
+  const int e = ilogb(cnorm);
+  return e < -300 || e > 300 ? -e : 0;
+}
 // y = x * f, f = *factor or 1 / *factor (device scalar); may change precision.
 template <typename TI, typename TO>
 cudaError_t launch_scale(const Geom& G, const cpx<TI>* x, const double* factor, bool invert, cpx<TO>* y,
@@ -435,7 +448,7 @@ cudaError_t launch_reduce(const double* partials, int n, double* out, bool sqrt_
 // launch_residual)
 int sweep_partials(const Geom& G);
 // GMRES scalar kernels (one thread)
-cudaError_t launch_gmres_start(GmresDev* st, const double* beta, bool unit, const Exec& ex);
+cudaError_t launch_gmres_start(GmresDev* st, const double* beta, bool unit, const Exec& ex, int rexp = 0);
 cudaError_t launch_backsolve(GmresDev* st, int k, const Exec& ex, const int* kdev = nullptr);
 // graph-mode control kernels (one thread); see csrc/sgn_krylov.cu
 cudaError_t launch_ctl_begin(GmresDev* st, const double* cnorm, GraphCtl ctl, const Exec& ex);

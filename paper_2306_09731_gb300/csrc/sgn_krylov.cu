@@ -574,12 +574,15 @@ __global__ void __launch_bounds__(ORTHO_THR, 1) k_ortho(Geom G, cpx<double>* V, 
 
 template <typename T>
 __global__ void __launch_bounds__(256) k_residual(Geom G, const cpx<T>* c, const cpx<T>* w, cpx<T>* r,
-                                                  double* partials) {
+                                                  double* partials, int rexp, const int* rexp_dev) {
   __shared__ double red[32];
   double acc = 0.0;
+  if (rexp_dev) rexp = *rexp_dev;
+  const T p = (T)scalbn(1.0, rexp);
   for (Walk it(G); it.ok(); it.next()) {
     const cpx<T> z = c[it.e] - w[it.e];
     r[it.e] = z;
+    if (rexp != 0) r[it.e] = mk(z.x * p, z.y * p);
     const int wt = col_weight_i(G, it.col);
     const double x = (double)z.x, y = (double)z.y;
     acc = fma(weigh(wt, x), x, fma(weigh(wt, y), y, acc));
@@ -664,12 +667,12 @@ __global__ void k_reduce(const double* partials, int n, double* out, int sqrt_ou
 // ---------------------------------------------------------- scalar kernels
 
 // g = (beta, 0, ...), the start of a GMRES cycle
-// (unit: X_0 = V_0, else X_0 = r = beta V_0)
-__global__ void k_gmres_start(GmresDev* st, const double* beta, int unit) {
+// (unit: X_0 = V_0, else X_0 = 2^rexp r = 2^rexp beta V_0)
+__global__ void k_gmres_start(GmresDev* st, const double* beta, int unit, int rexp) {
   for (int i = threadIdx.x; i <= MAXM; i += 32) st->g[i] = i == 0 ? *beta : 0.0;
   if (threadIdx.x != 0) return;
   st->res = *beta;
-  st->vscl[0] = unit ? 1.0 : 1.0 / *beta;
+  st->vscl[0] = unit ? 1.0 : scalbn(1.0 / *beta, -rexp);
 }
 
 // y = H(0:k,0:k)^{-1} g(0:k) by back substitution
@@ -703,6 +706,7 @@ __global__ void k_ctl_begin(GmresDev* st, const double* cnorm_d, GraphCtl ctl) {
   const double cn = *cnorm_d;
   st->cnorm = cn;
   st->target = ctl.tol * cn;
+  st->rexp = ctl.mixed ? 0 : residual_exp(cn);
   st->its = 0;
   st->sweeps = 0;
   st->k = 0;
@@ -721,7 +725,7 @@ __global__ void k_ctl_sweep(GmresDev* st, const double* beta_d, GraphCtl ctl) {
   st->beta = beta;
   st->k = 0;
   st->j = 0;
-  st->vscl[0] = ctl.mixed ? 1.0 : 1.0 / beta;  // X_0: r / beta in FP32, else r itself
+  st->vscl[0] = ctl.mixed ? 1.0 : scalbn(1.0 / beta, -st->rexp);  // X_0: r / beta in FP32, else 2^rexp r
   st->sweeps += 1;
   st->tot_sweeps += 1;
   const bool done = !(beta > st->target);
@@ -1000,9 +1004,9 @@ cudaError_t launch_ortho(const Geom& G, cpx<double>* V, size_t vstride, const cp
 }
 template <typename T>
 cudaError_t launch_residual(const Geom& G, const cpx<T>* c, const cpx<T>* w, cpx<T>* r, double* partials,
-                            const Exec& ex) {
+                            const Exec& ex, int rexp, const int* rexp_dev) {
   ex.begin(PK_KRYLOV);
-  k_residual<T><<<sweep_blocks(G, 1, NBLK), 256, 0, ex.s>>>(G, c, w, r, partials);
+  k_residual<T><<<sweep_blocks(G, 1, NBLK), 256, 0, ex.s>>>(G, c, w, r, partials, rexp, rexp_dev);
   ex.end();
   return cudaGetLastError();
 }
@@ -1053,9 +1057,9 @@ cudaError_t launch_reduce(const double* partials, int n, double* out, bool sqrt_
   ex.end();
   return cudaGetLastError();
 }
-cudaError_t launch_gmres_start(GmresDev* st, const double* beta, bool unit, const Exec& ex) {
+cudaError_t launch_gmres_start(GmresDev* st, const double* beta, bool unit, const Exec& ex, int rexp) {
   ex.begin(PK_KRYLOV);
-  k_gmres_start<<<1, 32, 0, ex.s>>>(st, beta, unit ? 1 : 0);
+  k_gmres_start<<<1, 32, 0, ex.s>>>(st, beta, unit ? 1 : 0, rexp);
   ex.end();
   return cudaGetLastError();
 }
@@ -1149,7 +1153,7 @@ cudaError_t launch_invariant_sums(const Geom& G, const double* h, const double* 
                                             GmresReadback*, const int*, const Exec&, const int*,            \
                                             const GraphCtl*);                                               \
   template cudaError_t launch_residual<T>(const Geom&, const cpx<T>*, const cpx<T>*, cpx<T>*, double*,       \
-                                          const Exec&);                                                     \
+                                          const Exec&, int, const int*);                                    \
   template cudaError_t launch_zero<T>(const Geom&, cpx<T>*, const Exec&, const int*);                       \
   template cudaError_t launch_axpby<T>(const Geom&, double, const cpx<T>*, double, cpx<T>*, const Exec&,     \
                                        const int*, const int*);                                               \
