@@ -55,8 +55,16 @@ __device__ __forceinline__ unsigned grp_get(const FxGrp& q, int slot) { return q
 // The scale of the complex inputs (x, y)[8] of an inverse transform (two slots),
 // and their conversion. DER: each is multiplied by i mi(s), |mi| < 2048.
 template <bool DER, class M>
-__device__ __forceinline__ FxScale fx_load8(const FxGrp& g, int slot, const double (&x)[8], const double (&y)[8],
-                                            int lN, M mi, cpx<fx> (&v)[8]) {
+__device__ __forceinline__ FxScale fx_load8(const FxGrp& g, int slot, double (&x)[8], double (&y)[8], int lN, M mi,
+                                            cpx<fx> (&v)[8]) {
+  if (DER) {
+#pragma unroll
+    for (int s = 0; s < 8; ++s)
+      if (mi(s) == 0) {
+        x[s] = fx_times0(x[s]);
+        y[s] = fx_times0(y[s]);
+      }
+  }
   unsigned mx = 0u;
 #pragma unroll
   for (int s = 0; s < 8; ++s) {
@@ -188,7 +196,10 @@ __device__ __forceinline__ FxScale fx_load_packed(const FxGrp& g, int slot, cons
   if (t == 0) {
     A[0].y = 0.0;
     B[0].y = 0.0;
-    if (!DER) {
+    if (DER) {
+      A[0].x = fx_times0(A[0].x);
+      B[0].x = fx_times0(B[0].x);
+    } else {
       an = S0[half].x;
       bn = S1[half].x;
     }
@@ -232,10 +243,6 @@ __device__ __forceinline__ FxScale fx_load_packed(const FxGrp& g, int slot, cons
     if (DER) {
       a = mul_i(a);
       b = mul_i(b);
-      if (s == 0 && t == 0) {
-        a = mk(fx{0}, fx{0});
-        b = a;
-      }
     }
     v[s] = mk(a.x - b.y, a.y + b.x);
     if (k > 0) sm[sidx<fx>(N - k, 0)] = mk(a.x + b.y, b.x - a.y);
