@@ -239,7 +239,8 @@ __device__ __forceinline__ unsigned abs_hi(double x) { return (unsigned)__double
 // 0 x: zero, but an infinity or NaN stays one. What a derivative multiplies by
 // m = 0 takes no part in its scale: the mean of a large value with small variations
 // would set it (whole numbers of 18 bits at 1024 x 256: error of the x-derivative
-// 1.6e-14 without a mean, 7.9e-13 on one of 2^30; FP64 radix-8: 5.3e-14 on both).
+// 1.6e-14 without a mean; on one of 2^30, 7.9e-13 when it counted and 2.7e-14 now;
+// FP64 radix-8: 5.3e-14 on both).
 __device__ __forceinline__ double fx_times0(double x) { return abs_hi(x) < 0x7ff00000u ? 0.0 : x; }
 
 // truncated magnitude in units of 2^(E - 1043)

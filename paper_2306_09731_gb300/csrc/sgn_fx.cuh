@@ -176,13 +176,57 @@ __device__ __forceinline__ FxScale fx_load8_fwd(const FxGrp& g, int slot, const 
   return sc;
 }
 
+// What a thread adds to the sum of moduli of the packed spectrum (fx_load_packed),
+// every entry counted twice (k and N - k): entries k = t + s T_ of both rows, and
+// on t = 0 the real ones at N/2.
+template <bool DER>
+__device__ __forceinline__ unsigned fx_packed_sum(const cpx<double> (&A)[4], const cpx<double> (&B)[4], double an,
+                                                  double bn, int E, int t, int T_) {
+  unsigned sum = 0u;
+  if (!DER && t == 0) sum = ((fx_mag(abs_hi(an), E) + fx_mag(abs_hi(bn), E)) >> 3) + 2u;
+#pragma unroll
+  for (int s = 0; s < 4; ++s) {
+    const unsigned m = fx_modulus(fx_mag(abs_hi(A[s].x), E), fx_mag(abs_hi(A[s].y), E)) +
+                       fx_modulus(fx_mag(abs_hi(B[s].x), E), fx_mag(abs_hi(B[s].y), E));
+    if (DER)
+      sum += (((m >> 3) * (unsigned)(t + s * T_)) >> 10) + 2u;
+    else
+      sum += (m >> 2) + 2u;
+  }
+  return sum;
+}
+// the conversion: Z[k] kept, Z[N - k] and Z[N/2] handed over in sm
+template <bool DER>
+__device__ __forceinline__ void fx_packed_from(const cpx<double> (&A)[4], const cpx<double> (&B)[4], double an,
+                                               double bn, int r0, int t, int lN, cpx<fx>* sm, cpx<fx> (&v)[8]) {
+  const int N = 1 << lN, T_ = N >> 3, half = N >> 1;
+#pragma unroll
+  for (int s = 0; s < 4; ++s) {
+    const int k = t + s * T_;
+    const unsigned mm = (unsigned)k << 21;
+    cpx<fx> a = mk(fx_from<DER>(A[s].x, r0, mm), fx_from<DER>(A[s].y, r0, mm));
+    cpx<fx> b = mk(fx_from<DER>(B[s].x, r0, mm), fx_from<DER>(B[s].y, r0, mm));
+    if (DER) {
+      a = mul_i(a);
+      b = mul_i(b);
+    }
+    v[s] = mk(a.x - b.y, a.y + b.x);
+    if (k > 0) sm[sidx<fx>(N - k, 0)] = mk(a.x + b.y, b.x - a.y);
+  }
+  if (t == 0)
+    sm[sidx<fx>(half, 0)] = DER ? mk(fx{0}, fx{0}) : mk(fx_from<false>(an, r0, 0u), fx_from<false>(bn, r0, 0u));
+}
+
 // The packed spectrum of two real rows from their half spectra S0, S1 (see
 // load_packed): a thread converts the entries k = t + s T_ < N/2 of both rows
 // once, keeps Z[k] = A + i B and hands Z[N - k] = conj(A) + i conj(B) over in sm
 // (free on entry and on exit). der: times i m (the factor 2 pi/Lx is left out).
-template <bool DER>
+// der may differ between the groups of a block: every barrier is outside its
+// branches. (Where the whole block takes one form, fx_load_packed_all has the two
+// as constants: 80 registers against 102 in k_fx_c2r.)
 __device__ __forceinline__ FxScale fx_load_packed(const FxGrp& g, int slot, const cpx<double>* S0,
-                                                  const cpx<double>* S1, int lN, cpx<fx>* sm, cpx<fx> (&v)[8]) {
+                                                  const cpx<double>* S1, int lN, bool der, cpx<fx>* sm,
+                                                  cpx<fx> (&v)[8]) {
   const int N = 1 << lN, T_ = N >> 3, half = N >> 1, t = g.t;
   cpx<double> A[4], B[4];
 #pragma unroll
@@ -196,7 +240,7 @@ __device__ __forceinline__ FxScale fx_load_packed(const FxGrp& g, int slot, cons
   if (t == 0) {
     A[0].y = 0.0;
     B[0].y = 0.0;
-    if (DER) {
+    if (der) {
       A[0].x = fx_times0(A[0].x);
       B[0].x = fx_times0(B[0].x);
     } else {
@@ -215,46 +259,29 @@ __device__ __forceinline__ FxScale fx_load_packed(const FxGrp& g, int slot, cons
   __syncthreads();
   const unsigned Mh = grp_get(g, slot);
   const int E = (int)(Mh >> 20);
-  // every entry counts twice (k and N - k)
-  unsigned sum = 0u;
-  if (!DER && t == 0) sum = ((fx_mag(abs_hi(an), E) + fx_mag(abs_hi(bn), E)) >> 3) + 2u;
-#pragma unroll
-  for (int s = 0; s < 4; ++s) {
-    const unsigned m = fx_modulus(fx_mag(abs_hi(A[s].x), E), fx_mag(abs_hi(A[s].y), E)) +
-                       fx_modulus(fx_mag(abs_hi(B[s].x), E), fx_mag(abs_hi(B[s].y), E));
-    if (DER)
-      sum += (((m >> 3) * (unsigned)(t + s * T_)) >> 10) + 2u;
-    else
-      sum += (m >> 2) + 2u;
-  }
-  grp_add(g, slot + 1, sum);
+  grp_add(g, slot + 1, der ? fx_packed_sum<true>(A, B, an, bn, E, t, T_) : fx_packed_sum<false>(A, B, an, bn, E, t, T_));
   __syncthreads();
   const unsigned L = grp_get(g, slot + 1);
   // |Z| <= |A| + |B|
   const unsigned m21 = 2u * fx_modulus(((Mh & 0xfffffu) | 0x100000u) + 1u, ((Mh & 0xfffffu) | 0x100000u) + 1u);
-  const FxScale sc = DER ? fx_scale(E, L, (((m21 >> 3) * (unsigned)half) >> 11) + 1u, 1029, lN)
-                         : fx_scale(E, L, (m21 >> 3) + 1u, 1040, lN);
-#pragma unroll
-  for (int s = 0; s < 4; ++s) {
-    const int k = t + s * T_;
-    const unsigned mm = (unsigned)k << 21;
-    cpx<fx> a = mk(fx_from<DER>(A[s].x, sc.r0, mm), fx_from<DER>(A[s].y, sc.r0, mm));
-    cpx<fx> b = mk(fx_from<DER>(B[s].x, sc.r0, mm), fx_from<DER>(B[s].y, sc.r0, mm));
-    if (DER) {
-      a = mul_i(a);
-      b = mul_i(b);
-    }
-    v[s] = mk(a.x - b.y, a.y + b.x);
-    if (k > 0) sm[sidx<fx>(N - k, 0)] = mk(a.x + b.y, b.x - a.y);
-  }
-  if (t == 0)
-    sm[sidx<fx>(half, 0)] =
-        DER ? mk(fx{0}, fx{0}) : mk(fx_from<false>(an, sc.r0, 0u), fx_from<false>(bn, sc.r0, 0u));
+  const FxScale sc = fx_scale(E, L, der ? (((m21 >> 3) * (unsigned)half) >> 11) + 1u : (m21 >> 3) + 1u,
+                              der ? 1029 : 1040, lN);
+  if (der)
+    fx_packed_from<true>(A, B, an, bn, sc.r0, t, lN, sm, v);
+  else
+    fx_packed_from<false>(A, B, an, bn, sc.r0, t, lN, sm, v);
   __syncthreads();
 #pragma unroll
   for (int s = 4; s < 8; ++s) v[s] = sm[sidx<fx>(t + s * T_, 0)];
   __syncthreads();
   return sc;
+}
+
+// the same with der equal across the block
+__device__ __forceinline__ FxScale fx_load_packed_all(const FxGrp& g, int slot, const cpx<double>* S0,
+                                                      const cpx<double>* S1, int lN, bool der, cpx<fx>* sm,
+                                                      cpx<fx> (&v)[8]) {
+  return der ? fx_load_packed(g, slot, S0, S1, lN, true, sm, v) : fx_load_packed(g, slot, S0, S1, lN, false, sm, v);
 }
 
 // After a forward transform of z = f0 + i f1: 2 F0[k], 2 F1[k] for the thread's
@@ -378,8 +405,7 @@ __global__ void __launch_bounds__(fx_threads<LN>()) k_fx_c2r(Geom G, const cpx<f
   const cpx<double>* in = a.in[fi];
   fx_red_zero(red, 2 * L.P);
   cpx<fx> v[8];
-  FxScale sc = der ? fx_load_packed<true>(g, 0, in + L.y0 * G.ldS, in + L.y1 * G.ldS, L.lN, sm, v)
-                   : fx_load_packed<false>(g, 0, in + L.y0 * G.ldS, in + L.y1 * G.ldS, L.lN, sm, v);
+  const FxScale sc = fx_load_packed_all(g, 0, in + L.y0 * G.ldS, in + L.y1 * G.ldS, L.lN, der, sm, v);
   fft_fx<true>(v, sm, tw, L.t, L.lN, 0, 0, sc.sh, sc.sh2);
   if (!L.valid) return;
   double* o = a.out[fi];
@@ -412,7 +438,7 @@ __global__ void __launch_bounds__(fx_threads<LN>()) k_fx_coef_x(Geom G, const cp
   fx_red_zero(red, 2 * L.P);
   cpx<fx> v[8];
   const FxScale sc =
-      fx_load_packed<false>(g, 0, Hy + L.y0 * G.ldS, Hy + L.y1 * G.ldS, L.lN, sm, v);
+      fx_load_packed(g, 0, Hy + L.y0 * G.ldS, Hy + L.y1 * G.ldS, L.lN, false, sm, v);
   fft_fx<true>(v, sm, tw, L.t, L.lN, 0, 0, sc.sh, sc.sh2);
   if (!L.valid) return;
   const double invN = 1.0 / (double)G.nphys();
@@ -469,9 +495,8 @@ __global__ void __launch_bounds__(PAR ? 384 : fx_threads<LN>(), PAR || LN == 12 
     }
     grp_max(g, slot + 4, cm);
     cpx<fx> v[8];
-    // (both forms pass the same number of barriers; a group is whole warps)
-    FxScale sc = ph == 1 ? fx_load_packed<true>(g, slot, in + o0, in + o1, lN, sm, v)
-                         : fx_load_packed<false>(g, slot, in + o0, in + o1, lN, sm, v);
+    const FxScale sc = PAR ? fx_load_packed(g, slot, in + o0, in + o1, lN, ph == 1, sm, v)
+                           : fx_load_packed_all(g, slot, in + o0, in + o1, lN, ph == 1, sm, v);
     const int Ec = (int)(grp_get(g, slot + 4) >> 20);
     const bool bad = sc.bad || Ec == 0x7ff;
     fft_fx<true>(v, sm, tw, t, lN, 0, plan, sc.sh, sc.sh2);
@@ -579,8 +604,7 @@ __global__ void __launch_bounds__(PAR ? 640 : fx_threads<LN>(), PAR || LN == 12 
     {
       const int i = L.ph;
       const cpx<double>* in = i == 1 ? Sy : (i == 3 ? Vx : (i == 4 ? Vy : S));
-      const FxScale sc = i == 0 ? fx_load_packed<true>(g, 0, in + o0, in + o1, lN, sm, v)
-                                : fx_load_packed<false>(g, 0, in + o0, in + o1, lN, sm, v);
+      const FxScale sc = fx_load_packed(g, 0, in + o0, in + o1, lN, i == 0, sm, v);
       fft_fx<true>(v, sm, tw, t, lN, 0, plan, sc.sh, sc.sh2);
       const double al = i == 0 ? alx : aly;
 #pragma unroll
@@ -659,8 +683,7 @@ __global__ void __launch_bounds__(PAR ? 640 : fx_threads<LN>(), PAR || LN == 12 
   for (int i = 0; i < 5; ++i) {
     const cpx<double>* in = i == 1 ? Sy : (i == 3 ? Vx : (i == 4 ? Vy : S));
     cpx<fx> v[8];
-    const FxScale sc = i == 0 ? fx_load_packed<true>(g, 2 * i, in + o0, in + o1, lN, sm, v)
-                              : fx_load_packed<false>(g, 2 * i, in + o0, in + o1, lN, sm, v);
+    const FxScale sc = fx_load_packed_all(g, 2 * i, in + o0, in + o1, lN, i == 0, sm, v);
     fft_fx<true>(v, sm, tw, t, lN, 0, plan, sc.sh, sc.sh2);
 #pragma unroll
     for (int s = 0; s < 8; ++s) {
