@@ -537,9 +537,16 @@ void arnoldi_step(sgn_ctx* ctx, const Tables<T>& tb, const T* cr, const T* cc, c
   // next basis vector itself, with no scaling pass
   const double* vscl = ctx->gst->vscl;
   // In one launch: the FP64 step, whose second pass nearly always runs (four
-  // kernels to one). The FP32 step has two to save, a wash for one solver at a
-  // time, and the cooperative launches of an ensemble's members keep one another
-  // waiting (12 members: 42 ms with two kernels, 58 with one).
+  // kernels to one). One solver at a time gains: five steps of the host loop at
+  // 256 x 16 take 13.6 ms against 16.6, three at 1024 x 256 12.0 against 13.4; two
+  // captured steps at 256^2 2.75 against 2.90, at 1024 x 512 6.08 against 6.49. In an
+  // ensemble a cooperative launch waits until all its blocks fit at once, and large
+  // ensembles lose (two captured steps of 16 members: 256 x 16 9.4 ms against 10.6,
+  // 256^2 20.1 against 16.2, 1024 x 512 115 against 103, mixed grids 51.5 against 40.1;
+  // two members 4.2, 12.6 and 5.0 against 4.4, 12.6 and 4.8). The rule is the grid's
+  // all the same: the two forms round differently, and a member of a batch gets
+  // the bits that it gets alone. The FP32 step has two kernels to save, a wash for
+  // one solver at a time (12 members: 42 ms with two kernels, 58 with one).
   if constexpr (dgks) {
     if (ctx->ortho) {
       CK(launch_ortho(G, V, vs, w, ctx->partials, ctx->gst, j, ctx->bar, ctx->rb_dev, ctx->flags, EX(ctx)));
