@@ -728,11 +728,10 @@ bool gmres(sgn_ctx* ctx, int* iters_out, double* relres_out) {
 }
 
 // ------------------------------------------------------- learned start
-// Kernels one network forward pass launches (13) for the launch count.
-// kernels of one sgn_unet_infer: the weight image, the first layer, two per
-// level above the bottleneck (s_l and its pool), e_l for 0 < l < D-1, b0, b1
-// and D-1 decoder layers
-int unet_launches(sgn_unet_t net) { return 4 * sgn_unet_levels(net) - 1; }
+// Kernels one sgn_unet_infer launches, for the launch count: the first layer
+// with the weight images, two per level above the bottleneck (s_l and its pool),
+// e_l for 0 < l < D-1, b0, b1 and D-1 decoder layers.
+int unet_launches(sgn_unet_t net) { return 4 * sgn_unet_levels(net) - 2; }
 
 double learned_tau(int pw, double dt) { return pw == 0 ? 1.0 : (pw == 1 ? 0.5 * dt : 0.25 * dt * dt); }
 
