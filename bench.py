@@ -228,7 +228,8 @@ def kernel_work(cls, n, tbytes):
     if cls == "rk":
         # with an FP32 right-hand side the update also reads sigma_hat and the
         # stage state (the state itself at stage 1): 3.25 more FP64 spectra
-        # per launch on average over the four stages
+        # per launch on average over the four stages (the stage's own b_hat now
+        # stands for two of the state's spectra: it reads half a spectrum less, 15.75)
         if tbytes == 4:
             return 46 * n * nxh, 3 * spec + 16.25 * spec_s
         return 30 * n * nxh, 3 * spec + 13 * spec_s

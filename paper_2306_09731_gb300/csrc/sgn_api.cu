@@ -1063,7 +1063,7 @@ void graph_gmres(sgn_ctx* ctx, GraphSeg& top) {
   ctl.h_sweep = top.handle();
   top.open();
   long long fixed = count_launches(ctx, [&] {
-      CK(launch_precond<double>(G, ctx->tb, ctx->bh, ctx->cvec, ctx->partials, EX(ctx)));
+    CK(launch_precond<double>(G, ctx->tb, ctx->bh, ctx->cvec, ctx->partials, EX(ctx)));
     CK(launch_reduce(ctx->partials, 1, cnorm_d, true, nullptr, EX(ctx), sweep_partials(G)));
     CK(launch_ctl_begin(ctx->gst, cnorm_d, ctl, EX(ctx)));
     CK(launch_zero<double>(G, ctx->sig, EX(ctx), &ctx->gst->zero_sigma));

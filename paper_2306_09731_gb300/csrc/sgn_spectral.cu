@@ -48,7 +48,7 @@ static void fx_y_config(const Geom& G, dim3& grid, dim3& block, size_t& smem, in
 // warps and fit the kernel's threads, and the GPU must have room, under two
 // blocks per SM.
 static bool fx_parallel(const dim3& grid, const dim3& block, int phases, int most = 384) {
-  return block.x % 32 == 0 && (int)block.x * phases <= most && grid.x < 304;
+  return block.x % 32 == 0 && (int)block.x * phases <= most && grid.x < kTwoPerSm;
 }
 
 template <int L>

@@ -524,97 +524,97 @@ __global__ void __launch_bounds__(xpass_threads<LN>(), rhs_min_blocks<LN>()) k_r
       __syncthreads();
     }
   } else {
-  cpx<T> QX[8], QY[8], F[8], Z[8];
-  // grad sigma
-  load_packed(QX, S + o0, S + o1, true, kx, L.t, lN);
-  fft_regs<true>(QX, sm, tw, L.t, lN, 0, PLAN);
-  load_packed(QY, Sy + o0, Sy + o1, false, kx, L.t, lN);
-  fft_regs<true>(QY, sm, tw, L.t, lN, 0, PLAN);
-#pragma unroll
-  for (int s = 0; s < 8; ++s) {
-    const int x = L.t + s * T_;
-    const T r0 = cr[p0 + x] * twoN, r1 = cr[p1 + x] * twoN;
-    const T sx0 = QX[s].x * n, sx1 = QX[s].y * n, sy0 = QY[s].x * n, sy1 = QY[s].y * n;
-    QX[s] = rhs_lin_split<T>() ? mk((T)0, (T)0) : mk(-sx0, -sx1);
-    QY[s] = rhs_lin_split<T>() ? mk((T)0, (T)0) : mk(-sy0, -sy1);
-    F[s] = mk((T)-0.5 * r0 * r0 * (sx0 * sx0 + sy0 * sy0), (T)-0.5 * r1 * r1 * (sx1 * sx1 + sy1 * sy1));
-  }
-  // sigma: -9 sigma^2 / (2 h^4)
-  load_packed(Z, S + o0, S + o1, false, kx, L.t, lN);
-  fft_regs<true>(Z, sm, tw, L.t, lN, 0, PLAN);
-#pragma unroll
-  for (int s = 0; s < 8; ++s) {
-    const int x = L.t + s * T_;
-    const T r0 = cr[p0 + x] * twoN, r1 = cr[p1 + x] * twoN;
-    const T s0 = Z[s].x * n, s1 = Z[s].y * n;
-    const T q0 = s0 * r0 * r0, q1 = s1 * r1 * r1;
-    F[s].x -= (T)4.5 * q0 * q0;
-    F[s].y -= (T)4.5 * q1 * q1;
-  }
-  // vx: h vx and |vx|^2/2
-  load_packed(Z, Vx + o0, Vx + o1, false, kx, L.t, lN);
-  fft_regs<true>(Z, sm, tw, L.t, lN, 0, PLAN);
-#pragma unroll
-  for (int s = 0; s < 8; ++s) {
-    const int x = L.t + s * T_;
-    const T a0 = hh[p0 + x], a1 = hh[p1 + x];  // h - 1
-    const T v0 = Z[s].x * n, v1 = Z[s].y * n;
-    QX[s].x += rhs_lin_split<T>() ? a0 * v0 : v0 + a0 * v0;
-    QX[s].y += rhs_lin_split<T>() ? a1 * v1 : v1 + a1 * v1;
-    F[s].x += (T)0.5 * v0 * v0;
-    F[s].y += (T)0.5 * v1 * v1;
-  }
-  // vy: h vy, |vy|^2/2 and g h
-  load_packed(Z, Vy + o0, Vy + o1, false, kx, L.t, lN);
-  fft_regs<true>(Z, sm, tw, L.t, lN, 0, PLAN);
-#pragma unroll
-  for (int s = 0; s < 8; ++s) {
-    const int x = L.t + s * T_;
-    const T a0 = hh[p0 + x], a1 = hh[p1 + x];  // h - 1
-    const T v0 = Z[s].x * n, v1 = Z[s].y * n;
-    QY[s].x += rhs_lin_split<T>() ? a0 * v0 : v0 + a0 * v0;
-    QY[s].y += rhs_lin_split<T>() ? a1 * v1 : v1 + a1 * v1;
-    // g (h - h_inf): the constant g h_inf of the Bernoulli equation (2) has no
-    // gradient; leaving it out keeps F's rounding relative to its variation
-    const T gh0 = rhs_lin_split<T>() ? (T)0 : g * a0, gh1 = rhs_lin_split<T>() ? (T)0 : g * a1;
-    F[s].x += (T)0.5 * v0 * v0 + gh0;
-    F[s].y += (T)0.5 * v1 * v1 + gh1;
-    // the split returns twice the half spectra: pre-scale by 1/2
-    QX[s] = scl(QX[s], (T)0.5);
-    QY[s] = scl(QY[s], (T)0.5);
-    F[s] = scl(F[s], (T)0.5);
-  }
-  cpx<T> f0[5], f1[5];
-  fft_regs<false>(QX, sm, tw, L.t, lN, 0, PLAN);
-  split_pair(QX, sm, L.t, lN, f0, f1);
-#pragma unroll
-  for (int s = 0; s < 5; ++s) {
-    if (!split_owns(s, L.t) || !L.valid) continue;
-    const int k = L.t + s * T_;
-    const T kv = ldr(kx + k);
-    Cq[o0 + k] = mul_ik(f0[s], -kv);
-    Cq[o1 + k] = mul_ik(f1[s], -kv);
-  }
-  __syncthreads();
-  fft_regs<false>(QY, sm, tw, L.t, lN, 0, PLAN);
-  split_pair(QY, sm, L.t, lN, f0, f1);
-#pragma unroll
-  for (int s = 0; s < 5; ++s) {
-    if (!split_owns(s, L.t) || !L.valid) continue;
-    const int k = L.t + s * T_;
-    Qy[o0 + k] = f0[s];
-    Qy[o1 + k] = f1[s];
-  }
-  __syncthreads();
-  fft_regs<false>(F, sm, tw, L.t, lN, 0, PLAN);
-  split_pair(F, sm, L.t, lN, f0, f1);
-#pragma unroll
-  for (int s = 0; s < 5; ++s) {
-    if (!split_owns(s, L.t) || !L.valid) continue;
-    const int k = L.t + s * T_;
-    Fh[o0 + k] = f0[s];
-    Fh[o1 + k] = f1[s];
-  }
+    cpx<T> QX[8], QY[8], F[8], Z[8];
+    // grad sigma
+    load_packed(QX, S + o0, S + o1, true, kx, L.t, lN);
+    fft_regs<true>(QX, sm, tw, L.t, lN, 0, PLAN);
+    load_packed(QY, Sy + o0, Sy + o1, false, kx, L.t, lN);
+    fft_regs<true>(QY, sm, tw, L.t, lN, 0, PLAN);
+  #pragma unroll
+    for (int s = 0; s < 8; ++s) {
+      const int x = L.t + s * T_;
+      const T r0 = cr[p0 + x] * twoN, r1 = cr[p1 + x] * twoN;
+      const T sx0 = QX[s].x * n, sx1 = QX[s].y * n, sy0 = QY[s].x * n, sy1 = QY[s].y * n;
+      QX[s] = rhs_lin_split<T>() ? mk((T)0, (T)0) : mk(-sx0, -sx1);
+      QY[s] = rhs_lin_split<T>() ? mk((T)0, (T)0) : mk(-sy0, -sy1);
+      F[s] = mk((T)-0.5 * r0 * r0 * (sx0 * sx0 + sy0 * sy0), (T)-0.5 * r1 * r1 * (sx1 * sx1 + sy1 * sy1));
+    }
+    // sigma: -9 sigma^2 / (2 h^4)
+    load_packed(Z, S + o0, S + o1, false, kx, L.t, lN);
+    fft_regs<true>(Z, sm, tw, L.t, lN, 0, PLAN);
+  #pragma unroll
+    for (int s = 0; s < 8; ++s) {
+      const int x = L.t + s * T_;
+      const T r0 = cr[p0 + x] * twoN, r1 = cr[p1 + x] * twoN;
+      const T s0 = Z[s].x * n, s1 = Z[s].y * n;
+      const T q0 = s0 * r0 * r0, q1 = s1 * r1 * r1;
+      F[s].x -= (T)4.5 * q0 * q0;
+      F[s].y -= (T)4.5 * q1 * q1;
+    }
+    // vx: h vx and |vx|^2/2
+    load_packed(Z, Vx + o0, Vx + o1, false, kx, L.t, lN);
+    fft_regs<true>(Z, sm, tw, L.t, lN, 0, PLAN);
+  #pragma unroll
+    for (int s = 0; s < 8; ++s) {
+      const int x = L.t + s * T_;
+      const T a0 = hh[p0 + x], a1 = hh[p1 + x];  // h - 1
+      const T v0 = Z[s].x * n, v1 = Z[s].y * n;
+      QX[s].x += rhs_lin_split<T>() ? a0 * v0 : v0 + a0 * v0;
+      QX[s].y += rhs_lin_split<T>() ? a1 * v1 : v1 + a1 * v1;
+      F[s].x += (T)0.5 * v0 * v0;
+      F[s].y += (T)0.5 * v1 * v1;
+    }
+    // vy: h vy, |vy|^2/2 and g h
+    load_packed(Z, Vy + o0, Vy + o1, false, kx, L.t, lN);
+    fft_regs<true>(Z, sm, tw, L.t, lN, 0, PLAN);
+  #pragma unroll
+    for (int s = 0; s < 8; ++s) {
+      const int x = L.t + s * T_;
+      const T a0 = hh[p0 + x], a1 = hh[p1 + x];  // h - 1
+      const T v0 = Z[s].x * n, v1 = Z[s].y * n;
+      QY[s].x += rhs_lin_split<T>() ? a0 * v0 : v0 + a0 * v0;
+      QY[s].y += rhs_lin_split<T>() ? a1 * v1 : v1 + a1 * v1;
+      // g (h - h_inf): the constant g h_inf of the Bernoulli equation (2) has no
+      // gradient; leaving it out keeps F's rounding relative to its variation
+      const T gh0 = rhs_lin_split<T>() ? (T)0 : g * a0, gh1 = rhs_lin_split<T>() ? (T)0 : g * a1;
+      F[s].x += (T)0.5 * v0 * v0 + gh0;
+      F[s].y += (T)0.5 * v1 * v1 + gh1;
+      // the split returns twice the half spectra: pre-scale by 1/2
+      QX[s] = scl(QX[s], (T)0.5);
+      QY[s] = scl(QY[s], (T)0.5);
+      F[s] = scl(F[s], (T)0.5);
+    }
+    cpx<T> f0[5], f1[5];
+    fft_regs<false>(QX, sm, tw, L.t, lN, 0, PLAN);
+    split_pair(QX, sm, L.t, lN, f0, f1);
+  #pragma unroll
+    for (int s = 0; s < 5; ++s) {
+      if (!split_owns(s, L.t) || !L.valid) continue;
+      const int k = L.t + s * T_;
+      const T kv = ldr(kx + k);
+      Cq[o0 + k] = mul_ik(f0[s], -kv);
+      Cq[o1 + k] = mul_ik(f1[s], -kv);
+    }
+    __syncthreads();
+    fft_regs<false>(QY, sm, tw, L.t, lN, 0, PLAN);
+    split_pair(QY, sm, L.t, lN, f0, f1);
+  #pragma unroll
+    for (int s = 0; s < 5; ++s) {
+      if (!split_owns(s, L.t) || !L.valid) continue;
+      const int k = L.t + s * T_;
+      Qy[o0 + k] = f0[s];
+      Qy[o1 + k] = f1[s];
+    }
+    __syncthreads();
+    fft_regs<false>(F, sm, tw, L.t, lN, 0, PLAN);
+    split_pair(F, sm, L.t, lN, f0, f1);
+  #pragma unroll
+    for (int s = 0; s < 5; ++s) {
+      if (!split_owns(s, L.t) || !L.valid) continue;
+      const int k = L.t + s * T_;
+      Fh[o0 + k] = f0[s];
+      Fh[o1 + k] = f1[s];
+    }
   }
 }
 
@@ -1348,11 +1348,12 @@ static inline void dispatch_l12(int lN, F&& f) {
 // neighbours (32-byte segments of the 16-byte types). At 256^2 (128 row pairs in
 // 128 blocks instead of 16): double-float matvec x-pass 36.2 -> 30.8 us, FP32
 // RHS x-pass 15.4 -> 12.4; at 1024 x 512 54.5 -> 49.5 and 19.2 -> 18.4.
+constexpr int kTwoPerSm = 2 * 152;
 static inline int builtin_pairs(const Geom& G) {
   const int Tn = G.Nx >> 3, half = G.Ny >> 1;
   int P = Tn >= 256 ? 1 : 256 / Tn;
   if (P > half) P = half;
-  while (P > 1 && (half + P - 1) / P < 304 && Tn * P >= 64) P >>= 1;
+  while (P > 1 && (half + P - 1) / P < kTwoPerSm && Tn * P >= 64) P >>= 1;
   return P;
 }
 // type: TuneType; nin: the pass's inputs (FP32)
@@ -1361,7 +1362,7 @@ static inline int builtin_cols(const Geom& G, int type, int nin) {
   const int Tn = G.Ny >> 3;
   int C = 256 / Tn;
   C = C < 1 ? 1 : (C > 64 ? 64 : C);
-  while (C > 2 && (G.Nxh + C - 1) / C < 304 && Tn * C >= 64) C >>= 1;
+  while (C > 2 && (G.Nxh + C - 1) / C < kTwoPerSm && Tn * C >= 64) C >>= 1;
   return C;
 }
 template <typename T>

@@ -235,8 +235,10 @@ __global__ void __launch_bounds__(128) k_conv3(const TI* __restrict__ in, size_t
 // of up to 128 pixels (R rows x CW columns); a thread one input channel and 4
 // output channels: 36 sums in registers, fed by 10 vector loads per 4 pixels and
 // 72 packed FMAs: 71 us a layer on average in the step above. (One block per
-// channel pair read every activation 9 Co times.) A chunk is summed on its own before it is added, so that no sum
-// runs over more than 128 terms. Fixed order: deterministic.
+// channel pair read every activation 9 Co times.) A chunk is summed on its own (128
+// terms at most), a block adds its chunks one after another (chunks / splits of
+// them: up to 219, the most at 512^2, batch 64 and 16 to 16 channels), and the blocks'
+// sums go through k_part_sum. Fixed order: deterministic.
 constexpr int DWPX = 128;
 __host__ __device__ inline void dw_chunk(int H, int W, int* R, int* CW) {
   *CW = W < 64 ? W : 64;
@@ -1052,7 +1054,10 @@ sgn_status create_impl(int n, int max_batch, int act_bf16, unsigned long long se
       ioff += 9ll * l.Ci * l.Co;
       int sm = l.row ? (int)unet_tc::row_smem_bytes(l.Co, l.KC, l.nkb, side)
                      : unet_tc::kStages * (int)unet_tc::stage_bytes(l.Co, l.KC);
-      // at most 512 / cols CTAs per SM, so that TMEM is never oversubscribed
+      // at most 512 / cols CTAs of this launch per SM: they all get their TMEM.
+      // With dependent launches, blocks of the next layer may share the SM, and
+      // their tcgen05.alloc waits until those here are through; it cannot lock
+      // up, as a block lets the next launch go only after its own allocation.
       int cols = 32;
       while (cols < l.Co) cols <<= 1;
       const int ctas = 512 / cols;
