@@ -20,6 +20,11 @@
  *    not aliasing each other unless stated. The caller owns them.
  *  - Wavenumbers k = 2*pi*m/L; the Nyquist wavenumber is set to 0 in every i*k
  *    multiplier and in M, so M equals L exactly at h = 1.
+ *  - The FP64 transforms (precision 0, precision 1's refinement residual, and the
+ *    calls on single fields in every precision) run in block fixed point: one
+ *    scale per row pair or column, its error below that of FP64 butterflies.
+ *    Magnitudes below 2^-1022 count as zero, in inputs and results, and a
+ *    transform with an infinity or NaN among its inputs returns NaN everywhere.
  *  - Calls are enqueued on the handle's stream (sgn_set_stream; default: the
  *    legacy default stream). Calls that run GMRES synchronise that stream once
  *    per GMRES iteration to read the convergence test.
@@ -41,7 +46,8 @@ typedef enum {
   SGN_ENOTCONV = 2,     /* GMRES hit maxit; the best iterate is still returned */
   SGN_ECAVITATION = 3,  /* h <= 0 somewhere (the paper assumes h > 0, Section 1) */
   SGN_ENONFINITE = 4,   /* NaN or Inf in h */
-  SGN_ECUDA = 5,        /* a CUDA runtime error; see sgn_last_error */
+  SGN_ECUDA = 5,        /* a CUDA runtime error, or a kernel's bounded wait that ran
+                           out; see sgn_last_error */
   SGN_ENOMEM = 6        /* device allocation failed in sgn_create */
 } sgn_status;
 
