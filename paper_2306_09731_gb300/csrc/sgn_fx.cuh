@@ -563,11 +563,11 @@ __global__ void __launch_bounds__(PAR ? 384 : fx_threads<LN>(), PAR || LN == 12 
           const cpx<fx> a0 = stash[(2 * s) * T_ + t], a1 = stash[(2 * s + 1) * T_ + t];
           const int sa = qc - qa, sb = qc - qb;
           cpx<fx> z;
-          z.x = fx_sar(a0.x, sa) + fx_sar(mul_q(b0[s].y, km), sb);
-          z.y = fx_sar(a0.y, sa) - fx_sar(mul_q(b0[s].x, km), sb);
+          z.x = fx_sar1(a0.x, sa) + fx_sar1(mul_q(b0[s].y, km), sb);
+          z.y = fx_sar1(a0.y, sa) - fx_sar1(mul_q(b0[s].x, km), sb);
           Cout[o0 + kc] = fx_out(z, qc, nan);
-          z.x = fx_sar(a1.x, sa) + fx_sar(mul_q(b1[s].y, km), sb);
-          z.y = fx_sar(a1.y, sa) - fx_sar(mul_q(b1[s].x, km), sb);
+          z.x = fx_sar1(a1.x, sa) + fx_sar1(mul_q(b1[s].y, km), sb);
+          z.y = fx_sar1(a1.y, sa) - fx_sar1(mul_q(b1[s].x, km), sb);
           Cout[o1 + kc] = fx_out(z, qc, nan);
         } else {
           Byout[o0 + kc] = fx_out(b0[s], q, nan);
@@ -927,8 +927,8 @@ __global__ void __launch_bounds__(PAR ? 384 : fx_threads<LN>(), PAR || LN == 12 
     // z0 - i k z1, aligned to the larger of the two scales plus one bit
     const int q1 = q[1] + ek - 1021, qc = (q[0] > q1 ? q[0] : q1) + 1;
     cpx<fx> z;
-    z.x = fx_sar(z0.x, qc - q[0]) + fx_sar(mul_q(z1.y, km), qc - q1);
-    z.y = fx_sar(z0.y, qc - q[0]) - fx_sar(mul_q(z1.x, km), qc - q1);
+    z.x = fx_sar1(z0.x, qc - q[0]) + fx_sar1(mul_q(z1.y, km), qc - q1);
+    z.y = fx_sar1(z0.y, qc - q[0]) - fx_sar1(mul_q(z1.x, km), qc - q1);
     int qz = qc;
     if (NIN == 2) {
       if (a.minv) {
